@@ -193,9 +193,11 @@ void mhc_destroy(mhc_ctx *ctx);
  *                 1: 256 threads per 64 x 64 tile, 4 x 4 micro-tiles, all warps on one step at a time;
  *                 2: 64 threads per tile, 8 x 8 micro-tiles;
  *                 3: 4 warps per tile, each warp testing whole steps (8 x 16 micro-tiles per lane);
- *                 4: one warp per tile walking its steps in order (8 x 16 micro-tiles per lane, pairs that
- *                    already hit dropped from later steps, first hits stored at once);
- *                 5: as 4 with one warp per 32 x 32 quarter tile (4 x 8 micro-tiles, culling per quarter);
+ *                 4: the 32 x 32 blocks with an active step listed first, then one warp per listed block walking its
+ *                    steps in order (pairs that already hit dropped from later steps, first hits stored at once); the
+ *                    hypotheses are tiled in a compact order of each object's grid, so that few blocks come close;
+ *                 5: one warp per 32 x 32 quarter tile of ascending hypotheses walking its steps in order (4 x 8
+ *                    micro-tiles, culling per quarter);
  *                 6: every active (quarter tile, step) an item, all tested in parallel by persistent warps (a
  *                    pair's first step by atomicMin in scratch, the table and the risk terms written after);
  *                    for small scenes (at most 2^22 items and 2^26 table entries; larger ones use 5);

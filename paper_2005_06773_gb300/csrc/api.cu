@@ -106,6 +106,44 @@ void append_rectangle(float hl, float hw, std::vector<PolyVertex> &out) {
     out.push_back(make_float4(-hl, -hw, 0.f, -1.f));
 }
 
+// How an object's hypotheses lie in space t seconds ahead: the distance of neighbours along grid_a and along grid_b.
+// Vehicles: da t^2 / 2 and, for steering angles, v^2 db t^2 / (2 L); path hypotheses: the paths' mean distance at
+// their last section.  Pedestrians: da t for speeds (da t^2 / 2 for accelerations) and speed x heading step x t.
+void neighbour_distance(const mhc_object &o, double t, double &along_a, double &along_b) {
+    float a_lo = o.grid_a[0], a_hi = a_lo, b_lo = o.grid_b[0], b_hi = b_lo;
+    for (int q = 1; q < o.n_a; ++q) { a_lo = std::min(a_lo, o.grid_a[q]); a_hi = std::max(a_hi, o.grid_a[q]); }
+    for (int q = 1; q < o.n_b; ++q) { b_lo = std::min(b_lo, o.grid_b[q]); b_hi = std::max(b_hi, o.grid_b[q]); }
+    const double da = o.n_a > 1 ? ((double)a_hi - a_lo) / (o.n_a - 1) : 0.0;
+    const double db = o.n_b > 1 ? ((double)b_hi - b_lo) / (o.n_b - 1) : 0.0;
+    const double far = std::max(std::fabs((double)a_lo), std::fabs((double)a_hi));
+    if (o.kind == MHC_VEHICLE && o.paths) {
+        const float *p = o.paths + 6, *q = o.paths + 9LL * (o.n_b - 1) + 6;
+        along_b = o.n_b > 1 ? std::hypot((double)q[0] - p[0], (double)q[1] - p[1]) / (o.n_b - 1) : 0.0;
+    } else if (o.kind == MHC_VEHICLE) {
+        along_b = (double)o.v0 * o.v0 * db * t * t / (2.0 * 2.7);
+    } else {
+        along_b = (o.flags & MHC_PED_ACCEL_GRID ? 0.5 * far * t : far) * db * t;
+    }
+    along_a = o.kind == MHC_PEDESTRIAN && !(o.flags & MHC_PED_ACCEL_GRID) ? da * t : 0.5 * da * t * t;
+}
+
+// The order of an object's hypotheses in its collision tiles (hypothesis_at): strips of w grid_b values, such that
+// a tile of w x 32 / w hypotheses is about as long as it is wide: w^2 = 32 along_a / along_b, doubled because braking
+// hypotheses fan out less than along_b says (11 objects: w = 5, where 4 to 6 leave the fewest active steps; 12 cars
+// of 64 x 32: 3, best at 3 and 4).  Where even 32 grid_b values are narrow (the paper's EGO, 343 of them), strips of
+// few grid_a values run along grid_b instead.  Path hypotheses keep their order (a few paths per acceleration:
+// already compact).
+int tile_order(const mhc_object &o) {
+    if (o.paths || o.n_a < 2 || o.n_b < 2) return 0;
+    double along_a, along_b;
+    neighbour_distance(o, 1.0, along_a, along_b);
+    if (!(along_a > 0.0) || !(along_b > 0.0)) return 0;
+    const double w = std::sqrt(64.0 * along_a / along_b);
+    if (w >= 22.0 && o.n_b > 16) return 2 * 1 + 1;         // one grid_a value per strip
+    if (w >= 12.0 && o.n_b > 16) return 2 * 2 + 1;
+    return 2 * std::max(1, std::min(o.n_b, (int)(w + 0.5)));
+}
+
 // Validates scenario `si` and appends it to the layout.
 int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
     char sw[48] = "";
@@ -194,7 +232,7 @@ int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
             if (!(src.radius > 0.f) || !finite(src.radius)) return fail(MHC_E_INVALID, where() + "pedestrian needs a positive radius");
             d.rad = src.radius; d.circ = src.radius;
         }
-        d.scen = si; d.n_steps = N; d.substeps = sc->substeps; d.model = sc->model; d.tau = sc->tau;
+        d.scen = si; d.n_steps = N; d.substeps = sc->substeps; d.order = tile_order(src); d.tau = sc->tau;
         d.tau_i_d = (double)sc->tau / (double)sc->substeps;
         if (src.kind == MHC_VEHICLE) {
             d.regime_off = (int)L.regimes.size();
@@ -248,7 +286,6 @@ int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
         const int a = obj0 + la, b = obj0 + lb;
         const ObjDesc &A = L.objs[a], &B = L.objs[b];
         p.a = a; p.b = b;
-        p.tiles_a = (A.h + kTile - 1) / kTile;
         p.tiles_b = (B.h + kTile - 1) / kTile;
         p.off = L.n_entries;
         p.tile_start = L.n_tiles;
@@ -262,7 +299,6 @@ int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
         copy_object_fields(p, A, B);
         p.ego_side = la == sc->ego ? 0 : (lb == sc->ego ? 1 : -1);
         p.n_steps = N;
-        p.scen = si;
         p.kofs = L.n_kofs;
         p.lsum_base = S.lsum_base;
         p.mass_base = S.mass_base;
@@ -271,7 +307,7 @@ int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
         p.co_local = p.ego_side == 0 ? lb : (p.ego_side == 1 ? la : 0);
         p.index = (int)L.pairs.size();
         L.n_entries += (long long)A.h * B.h;
-        L.n_tiles += (long long)p.tiles_a * p.tiles_b;
+        L.n_tiles += pair_tiles(p);
         L.n_kofs += N;
         L.pairs.push_back(p);
     };
@@ -337,7 +373,7 @@ int build_layout(const mhc_scenario *sc, int n_scen, Layout &L) {
     for (size_t q = 0; q < key.size(); ++q) {
         PairDesc d = L.pairs[key[q].second];
         d.tile_start = tiles;
-        tiles += (long long)d.tiles_a * d.tiles_b;
+        tiles += pair_tiles(d);
         L.pairs_c[q] = d;
     }
     return MHC_OK;
@@ -429,7 +465,11 @@ Scratch scratch_of(const Layout &L, bool with_weights) {
                                 : 0;
     if (blocklist_eligible(L))   // variant 6 or 8 takes the space, never both in one call
         s.items = std::max(s.items, kAlign + align_up(4 * sizeof(ActiveBlock) * (size_t)L.n_tiles));
-    s.total = s.desc + s.weights + s.bounds + s.prob + s.acc + s.items;
+    s.least = s.desc + s.weights + s.bounds + s.prob + s.acc + s.items;
+    // variant 4: the poses in tile order (and the list of active blocks), where the records of variant 6 or 8 would be
+    size_t tiles = align_up(sizeof(float4) * 32 * (size_t)L.n_bounds) + align_up(sizeof(int) * 32 * (size_t)L.n_tiles32);
+    tiles += kAlign + align_up(4 * sizeof(BlockRef) * (size_t)L.n_tiles);
+    s.total = s.least - s.items + std::max(s.items, tiles);
     return s;
 }
 
@@ -622,15 +662,14 @@ int log2_floor(long long v) {
     return r;
 }
 
-// Collision configuration for a scenario: the forced variant, else the tuned one of its size class, else
-// the default (a warp per tile for at least 32 tiles per SM, else a warp per quarter tile).
-// The collision layout without tuning.  Large scenes: a warp per tile in step order; small ones, whose
-// time is the closest pairs' long step chains: every active step in parallel where the item list fits,
-// else a warp per quarter tile.
+// The collision layout without tuning.  Large scenes (32 tiles per SM and more): a warp per active block, in step
+// order; small ones, whose time is the closest pairs' step chains: a CTA per block, its steps spread over the warps.
 int default_variant(const mhc_ctx *ctx, const Layout &L) {
     return L.n_tiles >= 32LL * ctx->n_sm ? 4 : 7;
 }
 
+// Collision configuration for a scenario: the forced variant, else the tuned one of its size class, else the
+// default.
 void pick_collide_config(const mhc_ctx *ctx, const Layout &L, bool fused, int &variant, int &cull) {
     cull = ctx->cull;
     if (ctx->variant != 0) { variant = ctx->variant; return; }
@@ -740,11 +779,30 @@ int launch_all(mhc_ctx *ctx, const Layout &L, const DevDesc &D, Bump &bump, cons
     if (coll_in) {
         float4 *bounds = static_cast<float4 *>(bump.take(sizeof(float4) * (size_t)L.n_bounds));
         if (!bounds) return fail(MHC_E_NOMEM, "arena too small for tile bounds");
+        CollideArgs c{};
+        // poses in tile order for layout 4 (and the list of active blocks); without room for them (an
+        // arena sized to the least) or without culling, it takes the blocks of ascending tiles and reads the planes
+        float4 *tile_poses = nullptr;
+        int *tile_order = nullptr;
+        if (variant == 4 && cull && L.n_tiles > 0) {
+            tile_poses = static_cast<float4 *>(bump.take(sizeof(float4) * 32 * (size_t)L.n_bounds));
+            if (tile_poses) tile_order = static_cast<int *>(bump.take(sizeof(int) * 32 * (size_t)L.n_tiles32));
+            if (tile_order) {
+                c.list_counts = static_cast<unsigned long long *>(bump.take(kAlign));
+                c.list = static_cast<BlockRef *>(bump.take(sizeof(BlockRef) * (size_t)(4 * L.n_tiles)));
+            }
+            if (!c.list || !c.list_counts) tile_poses = nullptr;
+        }
+        if (variant == 8) {   // the block records and their count (zeroed by the bounds kernel, else a memset)
+            c.item_count = static_cast<unsigned long long *>(bump.take(kAlign));
+            c.active_count = c.item_count + 1;
+            c.recs = static_cast<ActiveBlock *>(bump.take(sizeof(ActiveBlock) * (size_t)(4 * L.n_tiles)));
+            if (!c.item_count || !c.recs) return fail(MHC_E_NOMEM, "arena too small for the block records");
+        }
         // small tables: the quarter-tile layout writes the -1s of its own blocks (one launch less); large ones
         // are filled by the HBM-rate fill kernel (in-kernel 2-byte row stores cost issue slots there)
         const bool fill_in_bounds = !fill_in_gen && (variant == 7 || variant == 8) && cull &&
                                     (long long)L.warp_obj.size() * L.max_steps > 0;
-        CollideArgs c{};
         if (variant == 6) {   // the item list and its two counters (zeroed by the bounds kernel, else a memset)
             c.max_items = 4 * L.n_tiles * (long long)L.max_steps;
             c.item_count = static_cast<unsigned long long *>(bump.take(kAlign));
@@ -755,12 +813,6 @@ int launch_all(mhc_ctx *ctx, const Layout &L, const DevDesc &D, Bump &bump, cons
             c.blocks = static_cast<ItemBlock *>(bump.take(sizeof(ItemBlock) * (size_t)(4 * L.n_tiles)));
             if (!c.items || !c.item_count || !c.first32 || !c.active || !c.blocks)
                 return fail(MHC_E_NOMEM, "arena too small for the step items");
-        }
-        if (variant == 8) {   // the block records and their count (zeroed by the bounds kernel, else a memset)
-            c.item_count = static_cast<unsigned long long *>(bump.take(kAlign));
-            c.active_count = c.item_count + 1;
-            c.recs = static_cast<ActiveBlock *>(bump.take(sizeof(ActiveBlock) * (size_t)(4 * L.n_tiles)));
-            if (!c.item_count || !c.recs) return fail(MHC_E_NOMEM, "arena too small for the block records");
         }
         bool counts_zeroed = false;
         {
@@ -774,8 +826,9 @@ int launch_all(mhc_ctx *ctx, const Layout &L, const DevDesc &D, Bump &bump, cons
                 b.objs = D.objs; b.warp_obj = D.warp_obj; b.warp_first = D.warp_first;
                 b.n_warps = (int)L.warp_obj.size(); b.max_steps = L.max_steps; b.x = coll_in->x; b.y = coll_in->y;
                 b.bounds = bounds;
+                b.c = coll_in->c; b.s = coll_in->s; b.tile_poses = tile_poses; b.tile_order = tile_order;
                 const bool launches = (long long)b.n_warps * b.max_steps > 0;
-                if ((variant == 6 || variant == 8) && launches) b.zero_counts = c.item_count;
+                if (launches) b.zero_counts = tile_poses ? c.list_counts : c.item_count;   // (null: no list)
                 if (fill_in_bounds) { b.fill = table; b.n_fill = L.n_entries; }
                 e = launch_bounds(b, st, pdl());
                 if (e != cudaSuccess) return cuda_fail(e, "bounds kernel launch");
@@ -787,6 +840,7 @@ int launch_all(mhc_ctx *ctx, const Layout &L, const DevDesc &D, Bump &bump, cons
         c.max_steps = L.max_steps; c.cull = cull; c.variant = variant; c.fill_blocks = fill_in_collide;
         c.max_ctas = ctx->collide_max_ctas;
         c.x = coll_in->x; c.y = coll_in->y; c.c = coll_in->c; c.s = coll_in->s;
+        c.tile_poses = tile_poses; c.tile_order = tile_order;
         c.bounds = bounds; c.polys = D.polys; c.table = table; c.counters = ctx->counters;
         if (fused) {
             c.probf = r.probf;
@@ -794,11 +848,11 @@ int launch_all(mhc_ctx *ctx, const Layout &L, const DevDesc &D, Bump &bump, cons
             c.lfix = r.lfix;
             c.acc = r.acc;
         }
-        if ((variant == 6 || variant == 8) && !counts_zeroed) {
+        if (c.item_count && !counts_zeroed) {
             MHC_CUDA(cudaMemsetAsync(c.item_count, 0, 2 * sizeof(unsigned long long), st));
             after_kernel = false;
         }
-        TimedScope ts(ctx, st, MHC_K_COLLIDE, variant == 6 ? 3 : (variant == 8 ? 2 : 1));
+        TimedScope ts(ctx, st, MHC_K_COLLIDE, variant == 6 ? 3 : (variant == 8 || tile_poses ? 2 : 1));
         cudaError_t e = launch_collide(c, st, pdl());
         if (e != cudaSuccess) return cuda_fail(e, "collision kernel launch");
         if (L.n_tiles > 0) after_kernel = true;

@@ -79,7 +79,7 @@ std::vector<std::pair<int, int>> plan_group_ranges(const Layout &L) {
     std::vector<long long> tiles(L.n_scen, 0);
     long long total = 0;
     for (int q = 0; q < L.n_scen; ++q) {
-        for (int p = L.pair0[q]; p < L.pair0[q + 1]; ++p) tiles[q] += (long long)L.pairs[p].tiles_a * L.pairs[p].tiles_b;
+        for (int p = L.pair0[q]; p < L.pair0[q + 1]; ++p) tiles[q] += pair_tiles(L.pairs[p]);
         total += tiles[q];
     }
     int s0 = 0;
@@ -299,13 +299,17 @@ int mhc_plan_create(mhc_ctx *ctx, const mhc_scenario *scens, int32_t n_scen, con
         const size_t desc = plan_groups_pack(p, scens, traj_weights, nullptr);
         if (!desc) { delete p; return fail(MHC_E_INVALID, "plan group layout failed"); }
         size_t off = desc;
-        for (PlanGroup &G : p->groups) {
-            const Scratch SG = scratch_of(G.L, !G.w.empty());
-            G.work = p->dev + off;
-            G.work_bytes = SG.total - SG.desc - SG.weights + 2 * kAlign;
-            off = align_up(off + G.work_bytes);
-            group_slices(p, G);
+        for (const bool least : {false, true}) {   // with room for the poses in tile order, else without
+            off = desc;
+            for (PlanGroup &G : p->groups) {
+                const Scratch SG = scratch_of(G.L, !G.w.empty());
+                G.work = p->dev + off;
+                G.work_bytes = (least ? SG.least : SG.total) - SG.desc - SG.weights + 2 * kAlign;
+                off = align_up(off + G.work_bytes);
+            }
+            if (off <= scratch_bytes) break;
         }
+        for (PlanGroup &G : p->groups) group_slices(p, G);
         if (scratch_bytes < off) {
             delete p;
             return fail(MHC_E_NOMEM, "plan scratch smaller than mhc_batch_info.plan_bytes");
@@ -314,7 +318,7 @@ int mhc_plan_create(mhc_ctx *ctx, const mhc_scenario *scens, int32_t n_scen, con
     } else {
         p->groups.clear();
         const Scratch S = scratch_of(p->L, p->has_w);
-        if (scratch_bytes < S.total) {
+        if (scratch_bytes < S.least) {
             delete p;
             return fail(MHC_E_NOMEM, "plan scratch smaller than mhc_batch_info.plan_bytes");
         }

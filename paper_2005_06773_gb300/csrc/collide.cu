@@ -6,10 +6,12 @@
 //         tile's active steps are staged into shared memory a chunk at a time and tested in any order, the
 //         earliest hit kept with a shared atomicMin;
 //   3     a CTA of 4 warps per tile, each warp testing whole steps;
-//   4, 5  one warp per 64 x 64 tile (4 warps per CTA) or per 32 x 32 quarter (1-warp CTAs) walking the
-//         active steps in ascending order: a register mask remembers the pairs that already hit, so only
-//         first hits are stored and later candidates of those pairs cost nothing; the warp stages its own
-//         poses with the next step's loads in flight, and loops over blocks when the grid is capped;
+//   4     one warp per 32 x 32 block with an active step, the objects' hypotheses in a compact order
+//         (collide_tiles.cu; the large-scene default);
+//   5     one warp per 32 x 32 quarter tile (1-warp CTAs) walking the active steps in ascending order: a
+//         register mask remembers the pairs that already hit, so only first hits are stored and later
+//         candidates of those pairs cost nothing; the warp stages its own poses with the next step's loads in
+//         flight, and loops over blocks when the grid is capped;
 //   6     step items: (32 x 32 block, active step) pairs listed by one kernel and taken in any order by a
 //         persistent kernel that keeps each pair's earliest step with a global atomicMin; a third kernel
 //         writes the int16 table (and the fused risk terms) for the blocks with active steps;
@@ -33,219 +35,10 @@
 #include <algorithm>
 #include <cstdint>
 
-#include "mhc_internal.cuh"
+#include "collide_common.cuh"
 
 namespace mhc {
 namespace {
-
-constexpr float kEps = 1e-5f;
-constexpr float kEps0 = 1e-4f;
-constexpr float kFar = 1.0e6f;   // padding poses far outside any scene
-
-__device__ __forceinline__ bool rect_rect(float dx, float dy, float ca, float sa, float la, float wa,
-                                          float cb, float sb, float lb, float wb) {
-    const float c = fabsf(fmaf(ca, cb, sa * sb));
-    const float s = fabsf(fmaf(sa, cb, -ca * sb));
-    const float pau = fabsf(fmaf(dx, ca, dy * sa));
-    const float pav = fabsf(fmaf(dy, ca, -dx * sa));
-    const float pbu = fabsf(fmaf(dx, cb, dy * sb));
-    const float pbv = fabsf(fmaf(dy, cb, -dx * sb));
-    return pau <= la + fmaf(lb, c, wb * s) && pav <= wa + fmaf(lb, s, wb * c) &&
-           pbu <= lb + fmaf(la, c, wa * s) && pbv <= wb + fmaf(la, s, wa * c);
-}
-
-// rectangle at the origin of d (axis (c, s), half extents l, w) against a disc of radius r at offset d
-__device__ __forceinline__ bool rect_disc(float dx, float dy, float c, float s, float l, float w, float r) {
-    const float ex = fmaxf(fabsf(fmaf(dx, c, dy * s)) - l, 0.0f);
-    const float ey = fmaxf(fabsf(fmaf(dy, c, -dx * s)) - w, 0.0f);
-    return fmaf(ex, ex, ey * ey) <= r * r;
-}
-
-// Convex outlines (Section IV-C.1 lets an outline be as detailed as needed); in a pair with an outline a
-// plain rectangle comes as a 4-gon.  Two convex polygons are disjoint iff the supporting line of some edge
-// of one has the whole other polygon strictly on its outer side (the edges of their Minkowski difference
-// are the edges of the two), so each edge is one test: edge e of A (body-frame vertex v_e, outward unit
-// normal n_e, support h_e = n_e . v_e) separates iff min over B's vertices w of
-// (R_a n_e) . (d + R_b w) > h_e, d = p_b - p_a.  The normal is turned into B's frame once per edge and B's
-// vertices are read as stored.  Only the kernels instantiated for batches with outlines contain it.
-__device__ __forceinline__ bool outline_outline(float dx, float dy, float ca, float sa, float cb, float sb,
-                                               const PolyVertex *A, int na, const PolyVertex *B, int nb) {
-    const float cr = fmaf(ca, cb, sa * sb), sr = fmaf(sa, cb, -ca * sb);   // R_b^T R_a = R(psi_a - psi_b)
-    for (int e = 0; e < na; ++e) {
-        const float4 v = A[e];
-        const float h = fmaf(v.z, v.x, v.w * v.y);
-        const float nwx = fmaf(ca, v.z, -sa * v.w), nwy = fmaf(sa, v.z, ca * v.w);
-        const float o = fmaf(nwx, dx, nwy * dy);
-        const float mx = fmaf(cr, v.z, -sr * v.w), my = fmaf(sr, v.z, cr * v.w);
-        float lo = INFINITY;
-        for (int q = 0; q < nb; ++q) {
-            const float4 w = B[q];
-            lo = fminf(lo, fmaf(mx, w.x, my * w.y));
-        }
-        if (o + lo > h) return false;
-    }
-    for (int e = 0; e < nb; ++e) {   // B's edges: A's vertices relative to p_b are -d + R_a w
-        const float4 v = B[e];
-        const float h = fmaf(v.z, v.x, v.w * v.y);
-        const float nwx = fmaf(cb, v.z, -sb * v.w), nwy = fmaf(sb, v.z, cb * v.w);
-        const float o = -fmaf(nwx, dx, nwy * dy);
-        const float mx = fmaf(cr, v.z, sr * v.w), my = fmaf(-sr, v.z, cr * v.w);   // R_a^T R_b = R(psi_b - psi_a)
-        float lo = INFINITY;
-        for (int q = 0; q < na; ++q) {
-            const float4 w = A[q];
-            lo = fminf(lo, fmaf(mx, w.x, my * w.y));
-        }
-        if (o + lo > h) return false;
-    }
-    return true;
-}
-
-// Outline A at the origin of d (axis (c, s)) against a disc of radius r at offset d: the disc's centre in
-// A's frame lies inside A, or within r of one of its edges (segment distance).
-__device__ __forceinline__ bool outline_disc(float dx, float dy, float c, float s, const PolyVertex *A, int n,
-                                            float r) {
-    const float qx = fmaf(dx, c, dy * s), qy = fmaf(dy, c, -dx * s);
-    float smax = -INFINITY;
-    for (int e = 0; e < n; ++e) {
-        const float4 v = A[e];
-        smax = fmaxf(smax, fmaf(v.z, qx - v.x, v.w * (qy - v.y)));
-    }
-    if (smax > r) return false;   // beyond some edge's line by more than r
-    if (smax <= 0.0f) return true; // centre inside
-    float d2 = INFINITY;
-    for (int e = 0; e < n; ++e) {
-        const float4 v = A[e], w = A[e + 1 == n ? 0 : e + 1];
-        const float ex = w.x - v.x, ey = w.y - v.y, px = qx - v.x, py = qy - v.y;
-        const float t = fminf(fmaxf(fmaf(px, ex, py * ey) / fmaf(ex, ex, ey * ey), 0.0f), 1.0f);
-        const float rx = fmaf(-t, ex, px), ry = fmaf(-t, ey, py);
-        d2 = fminf(d2, fmaf(rx, rx, ry * ry));
-    }
-    return d2 <= r * r;
-}
-
-// The exact test of one broad-phase candidate: d = p_b - p_a, (ca, sa) / (cb, sb) the body axes, la / wa
-// and lb / wb the half extents of rectangles, ra / rb the radii of discs.  OUTL: the batch has outlines
-// (combos 4..6); the kernels without them keep the short rectangle and disc tests alone.
-// The shape combination of a pair and its outlines, copied out of the descriptor once per block: a field read
-// through the descriptor in a loop with atomics would be read again after every atomic.
-struct PairShape {
-    int combo, poly_a, nv_a, poly_b, nv_b;
-};
-
-__device__ __forceinline__ PairShape shape_of(const PairDesc &P) { return {P.combo, P.poly_a, P.nv_a, P.poly_b, P.nv_b}; }
-
-template <bool OUTL>
-__device__ __forceinline__ bool narrow_hit(const PairShape P, const PolyVertex *polys, float dx, float dy,
-                                           float2 qa, float2 qb, float la, float wa, float lb, float wb,
-                                           float ra, float rb) {
-    if (!OUTL) {
-        switch (P.combo) {
-            case 0: return rect_rect(dx, dy, qa.x, qa.y, la, wa, qb.x, qb.y, lb, wb);
-            case 1: return rect_disc(dx, dy, qa.x, qa.y, la, wa, rb);
-            case 2: return rect_disc(-dx, -dy, qb.x, qb.y, lb, wb, ra);
-            default: return fmaf(dx, dx, dy * dy) <= (ra + rb) * (ra + rb);
-        }
-    }
-    switch (P.combo) {
-        case 0: return rect_rect(dx, dy, qa.x, qa.y, la, wa, qb.x, qb.y, lb, wb);
-        case 1: return rect_disc(dx, dy, qa.x, qa.y, la, wa, rb);
-        case 2: return rect_disc(-dx, -dy, qb.x, qb.y, lb, wb, ra);
-        case 3: return fmaf(dx, dx, dy * dy) <= (ra + rb) * (ra + rb);
-        case 4: return outline_outline(dx, dy, qa.x, qa.y, qb.x, qb.y, polys + P.poly_a, P.nv_a, polys + P.poly_b, P.nv_b);
-        case 5: return outline_disc(dx, dy, qa.x, qa.y, polys + P.poly_a, P.nv_a, rb);
-        default: return outline_disc(-dx, -dy, qb.x, qb.y, polys + P.poly_b, P.nv_b, ra);
-    }
-}
-
-// Narrow-phase work counters by shape class (CollideArgs::counters [2 + class]): 0 rectangle-rectangle,
-// 1 rectangle-disc, 2 disc-disc, 3 outline-outline, 4 outline-disc (the PairDesc combos 0, 1|2, 3, 4, 5|6).
-__device__ __forceinline__ int narrow_class(int combo) {
-    return combo == 0 ? 0 : (combo <= 2 ? 1 : (combo <= 4 ? combo - 1 : 4));
-}
-
-__device__ __forceinline__ void count_narrow(const CollideArgs &a, int combo, unsigned long long n) {
-    atomicAdd(a.counters + 1, n);
-    atomicAdd(a.counters + 2 + narrow_class(combo), n);
-}
-
-// Queue slots of one compaction round: each lane brings cnt (0..8) candidates; off = the candidates of the
-// lanes below it, total = all of them (one ballot per bit of cnt instead of a shuffle scan: four
-// independent instructions, not a chain of five).  Returns false when no lane has any (uniform).
-__device__ __forceinline__ bool queue_offsets(int cnt, int lane, int &off, int &total) {
-    const unsigned b0 = __ballot_sync(0xffffffffu, cnt & 1), b1 = __ballot_sync(0xffffffffu, cnt & 2);
-    const unsigned b2 = __ballot_sync(0xffffffffu, cnt & 4), b3 = __ballot_sync(0xffffffffu, cnt & 8);
-    if (!(b0 | b1 | b2 | b3)) return false;
-    const unsigned lt = (1u << lane) - 1u;
-    off = __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt) + 8 * __popc(b3 & lt);
-    total = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2) + 8 * __popc(b3);
-    return true;
-}
-
-// Position of the r-th set bit (r counted from 0, below popc(m)) of m, by halving popcounts.
-__device__ __forceinline__ int nth_set_bit(unsigned m, int r) {
-    int pos = 0, c = __popc(m & 0xffffu);
-    if (r >= c) { r -= c; m >>= 16; pos += 16; }
-    c = __popc(m & 0xffu);
-    if (r >= c) { r -= c; m >>= 8; pos += 8; }
-    c = __popc(m & 0xfu);
-    if (r >= c) { r -= c; m >>= 4; pos += 4; }
-    c = __popc(m & 0x3u);
-    if (r >= c) { r -= c; m >>= 2; pos += 2; }
-    return pos + (r >= (int)(m & 1u) ? 1 : 0);
-}
-
-// Candidate selection without a queue: lane L holds a mask `cand` of its candidates; slot s of the warp's
-// candidates in (lane, bit) order belongs to the last lane whose exclusive count is <= s (a 5-step
-// shuffle search), and is that lane's (s - its count)-th bit.  Every lane takes one slot per round, so the
-// exact tests run with all lanes busy.  Calls fn(owner lane, bit) for each slot (warp-uniform call).
-template <typename Fn>
-__device__ __forceinline__ void for_each_candidate(unsigned cand, int lane, Fn &&fn) {
-    const unsigned cnt = __popc(cand);
-    unsigned incl = cnt;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned v = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += v;
-    }
-    const unsigned excl = incl - cnt;
-    const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
-    for (unsigned s0 = 0; s0 < total; s0 += 32) {
-        const unsigned s = s0 + lane;
-        int owner = 0;
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-            const unsigned e = __shfl_sync(0xffffffffu, excl, owner + step);
-            if (e <= s) owner += step;
-        }
-        const unsigned m = __shfl_sync(0xffffffffu, cand, owner);
-        const unsigned e = __shfl_sync(0xffffffffu, excl, owner);
-        if (s < total) fn(owner, nth_set_bit(m, (int)(s - e)));
-    }
-}
-
-// The pair of collision tile g: the last pair (in collision-grid order) whose first tile is <= g.  A 64-way
-// search by the whole warp (every lane must call it with the same g): each round the lanes probe 64
-// evenly spaced pairs at once (two each) and keep the span between the last probe <= g and the next, so up
-// to 64 pairs take one round of loads and 4,096 two (a binary search is a chain of log2 n dependent loads).
-__device__ __forceinline__ int pair_of_tile(const CollideArgs &a, long long g) {
-    const int lane = threadIdx.x & 31;
-    int lo = 0, hi = a.n_pairs - 1;
-    while (lo < hi) {   // 64 probes per round (two per lane): a scene of up to 64 pairs in one round of loads
-        const long long span = hi - lo + 1;
-        const bool le0 = a.pairs[lo + (int)(span * (2 * lane) / 64)].tile_start <= g;
-        const bool le1 = a.pairs[lo + (int)(span * (2 * lane + 1) / 64)].tile_start <= g;
-        const unsigned long long m = (unsigned long long)__ballot_sync(0xffffffffu, le0) |
-                                     (unsigned long long)__ballot_sync(0xffffffffu, le1) << 32;
-        // probe q = 2 lane + (0 | 1) sits at bit lane + 32 (q & 1); probe 0 always holds: pairs[lo] <= g
-        const unsigned even = (unsigned)m, odd = (unsigned)(m >> 32);
-        const int le = 31 - __clz(even), lo2 = odd ? 31 - __clz(odd) : -1;   // last true even / odd probe
-        const int L = 2 * lo2 + 1 > 2 * le ? 2 * lo2 + 1 : 2 * le;           // the true probes form a prefix
-        const int nlo = lo + (int)(span * L / 64);
-        hi = L == 63 ? hi : lo + (int)(span * (L + 1) / 64) - 1;
-        lo = nlo;
-    }
-    return lo;
-}
 
 constexpr int kMaxChunks = (32767 + 31) / 32;   // 32-step activity words for the longest horizon
 constexpr int kFusedHistSteps = 1024;            // per-CTA step histograms in shared memory up to this N
@@ -851,26 +644,22 @@ __global__ void __launch_bounds__(WARPS * 32) collide_warp_kernel(const CollideA
     }
 }
 
-// Warp-per-tile layouts: each warp owns one TE x TE block of hypothesis pairs (a whole 64 x 64 tile, or
-// one 32 x 32 quarter of it) and walks its active steps in ascending order on its own (no CTA barrier
-// anywhere).  A lane holds an MI x MJ micro-block (rows lr + 8 m, columns lc + 4 n, lr = lane / 4,
-// lc = lane % 4; 8 x 16 for TE = 64, 4 x 8 for TE = 32) and a register mask of its pairs that have
-// already hit: because the steps come in order, the first narrow-phase hit of a pair is its first
-// collision step, it is stored at once, and later candidates of that pair are dropped before any further
-// work.  The warp stages each step's poses in its own shared-memory slot; the next active step's poses
-// are loaded into registers while the current step is tested.  Activity (culling against the blocks'
-// bounding boxes) is decided 32 steps at a time with one ballot.  Fused risk terms are added per hit with
-// global atomics; the per-step histogram terms of one step's hits are summed over the warp first.
-// One TE x TE block (warp task gw) walked by the calling warp; pa_s .. s_new are the warp's own slots.
-template <int TE, bool FUSED, bool OUTL>
+// Warp-per-block layout: each warp owns one 32 x 32 block of hypothesis pairs (a quarter of a 64 x 64 tile) and walks
+// its active steps in ascending order on its own (no CTA barrier anywhere).  A lane holds a 4 x 8 micro-block (rows
+// lr + 8 m, columns lc + 4 n, lr = lane / 4, lc = lane % 4) and a register mask of its pairs that have already hit:
+// because the steps come in order, the first narrow-phase hit of a pair is its first collision step, it is stored at
+// once, and later candidates of that pair are dropped before any further work.  The warp stages each step's poses in
+// its own shared-memory slot; the next active step's poses are loaded into registers while the current step is
+// tested.  Activity (culling against the blocks' bounding boxes) is decided 32 steps at a time with one ballot.
+// Fused risk terms are added per hit with global atomics; the per-step histogram terms of one step's hits are summed
+// over the warp first.  One block (warp task gw) walked by the calling warp; pa_s .. s_new are the warp's own slots.
+template <bool FUSED, bool OUTL>
 __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, int lane, float4 *pa_s, float4 *pb_s,
                                            float2 *ra_s, float2 *rb_s, float *prob_s) {
-    static_assert(TE == 64 || TE == 32, "block edge");
-    constexpr int MI = TE / 8, MJ = TE / 4;       // micro-block of a lane
-    constexpr int SUB = kTile / TE;               // blocks per tile edge
-    const long long g = gw / (SUB * SUB);                 // the 64 x 64 tile
+    constexpr int MI = 4, MJ = 8;                 // micro-block of a lane
+    const long long g = gw >> 2;                  // the 64 x 64 tile
     if (g >= a.n_tiles) return;
-    const int quarter = (int)(gw - g * (SUB * SUB));
+    const int quarter = (int)(gw & 3);
     const int lo = pair_of_tile(a, g);
     const PairDesc &P = a.pairs[lo];   // fields read where used (fewer live registers)
     const PairShape shape = shape_of(P);
@@ -878,32 +667,26 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
     const ObjDesc &B = a.objs[P.b];
     const int t = (int)(g - P.tile_start);          // < tiles_a x tiles_b <= n_tiles < 2^31
     const int ta = t / P.tiles_b, tb = t - ta * P.tiles_b;
-    const int ba_idx = ta * SUB + quarter / SUB, bb_idx = tb * SUB + quarter % SUB;   // blocks along a, b
-    const int i0 = ba_idx * TE, j0 = bb_idx * TE;
-    const int rows = min(TE, A.h - i0), cols = min(TE, B.h - j0);
+    const int i0 = (ta * 2 + (quarter >> 1)) * 32, j0 = (tb * 2 + (quarter & 1)) * 32;
+    const int rows = min(32, A.h - i0), cols = min(32, B.h - j0);
     if (rows <= 0 || cols <= 0) return;                    // a quarter past a ragged edge
     const int lr = lane >> 2, lc = lane & 3;
     const int N = P.n_steps;
-    const int na = (rows + kBoundTile - 1) / kBoundTile, nb = (cols + kBoundTile - 1) / kBoundTile;
     const float4 *bA0 = a.bounds + A.bounds_base + (long long)(i0 / kBoundTile) * N;
     const float4 *bB0 = a.bounds + B.bounds_base + (long long)(j0 / kBoundTile) * N;
     const float la = A.hl, wa = A.hw, ra = A.rad, lb = B.hl, wb = B.hw, rb = B.rad;
     const float rc2 = P.rc2 + kEps0;
     const float ka = 0.5f * (1.0f - kEps);
     const float r_cull = P.r_cull;
-    if (TE == 32 && a.fill_blocks) {   // this block's table entries start as -1 (coalesced 64-byte row stores)
+    if (a.fill_blocks) {   // this block's table entries start as -1 (coalesced 64-byte row stores)
         int16_t *row = a.table + P.off + (long long)i0 * B.h + j0;
         for (int r = 0; r < rows; ++r, row += B.h)
             for (int c = lane; c < cols; c += 32) row[c] = (int16_t)-1;
         __syncwarp();      // the fill is ordered before this warp's first-hit stores
     }
     if (FUSED) {   // the block's probabilities, read at every first hit (kept off the hit path's latency)
-#pragma unroll
-        for (int u = 0; u < TE / 32; ++u) {
-            const int r = lane + 32 * u;
-            prob_s[r] = r < rows ? a.probf[A.traj_off + i0 + r] : 0.0f;
-            prob_s[TE + r] = r < cols ? a.probf[B.traj_off + j0 + r] : 0.0f;
-        }
+        prob_s[lane] = lane < rows ? a.probf[A.traj_off + i0 + lane] : 0.0f;
+        prob_s[32 + lane] = lane < cols ? a.probf[B.traj_off + j0 + lane] : 0.0f;
     }
 
     // activity of the 32 steps from k0 (one ballot)
@@ -911,16 +694,7 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
         const int k = k0 + lane;
         bool act = k < N;
         if (act && a.cull) {
-            float4 ba = bA0[k];
-            if (na > 1) {
-                const float4 q = bA0[N + k];
-                ba = make_float4(fminf(ba.x, q.x), fminf(ba.y, q.y), fmaxf(ba.z, q.z), fmaxf(ba.w, q.w));
-            }
-            float4 bb = bB0[k];
-            if (nb > 1) {
-                const float4 q = bB0[N + k];
-                bb = make_float4(fminf(bb.x, q.x), fminf(bb.y, q.y), fmaxf(bb.z, q.z), fmaxf(bb.w, q.w));
-            }
+            const float4 ba = bA0[k], bb = bB0[k];
             act = (ba.x - r_cull <= bb.z) && (bb.x - r_cull <= ba.z) && (ba.y - r_cull <= bb.w) &&
                   (bb.y - r_cull <= ba.w);
         }
@@ -939,17 +713,14 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
         }
         return k0 + __ffs(m) - 1;
     };
-    // this lane's share of a step's poses: rows lane (+ 32) of A, then columns lane (+ 32) of B
-    constexpr int NU = 2 * (TE / 32);
-    float px[NU], py[NU], pc[NU], ps[NU];
+    // this lane's share of a step's poses: row `lane` of A, then column `lane` of B
+    float px[2], py[2], pc[2], ps[2];
     auto load_step = [&](int k) {
 #pragma unroll
-        for (int u = 0; u < NU; ++u) {
-            const bool isA = u < NU / 2;
-            const int r = lane + 32 * (isA ? u : u - NU / 2);
-            const bool ok = isA ? r < rows : r < cols;
-            const long long idx = isA ? A.pose_base + (long long)k * A.h + i0 + r
-                                      : B.pose_base + (long long)k * B.h + j0 + r;
+        for (int u = 0; u < 2; ++u) {
+            const bool isA = u == 0, ok = isA ? lane < rows : lane < cols;
+            const long long idx = isA ? A.pose_base + (long long)k * A.h + i0 + lane
+                                      : B.pose_base + (long long)k * B.h + j0 + lane;
             px[u] = ok ? __ldg(a.x + idx) : (isA ? kFar : -kFar);
             py[u] = ok ? __ldg(a.y + idx) : 0.0f;
             pc[u] = ok ? __ldg(a.c + idx) : 1.0f;
@@ -957,7 +728,7 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
         }
     };
 
-    unsigned long long found_lo = 0ull, found_hi = 0ull;   // bit MJ m + n of the lane's pairs
+    unsigned found = 0u;                // bit MJ m + n of the lane's pairs
     unsigned long long narrow = 0, hit_cnt = 0, hit_mass = 0;
     int active_steps = 0;
     int k = next_step(-1);
@@ -965,78 +736,67 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
     while (k >= 0) {
         __syncwarp();                       // the previous step's slot is no longer read
 #pragma unroll
-        for (int u = 0; u < NU; ++u) {
-            const bool isA = u < NU / 2;
-            const int r = lane + 32 * (isA ? u : u - NU / 2);
+        for (int u = 0; u < 2; ++u) {
             const float q2 = fmaf(px[u], px[u], py[u] * py[u]);
-            if (isA) {
-                pa_s[r] = make_float4(px[u], py[u], ka * q2, 0.0f);
-                ra_s[r] = make_float2(pc[u], ps[u]);
+            if (u == 0) {
+                pa_s[lane] = make_float4(px[u], py[u], ka * q2, 0.0f);
+                ra_s[lane] = make_float2(pc[u], ps[u]);
             } else {
-                pb_s[r] = make_float4(px[u], py[u], 0.5f * fmaf(1.0f - kEps, q2, -rc2), 0.0f);
-                rb_s[r] = make_float2(pc[u], ps[u]);
+                pb_s[lane] = make_float4(px[u], py[u], 0.5f * fmaf(1.0f - kEps, q2, -rc2), 0.0f);
+                rb_s[lane] = make_float2(pc[u], ps[u]);
             }
         }
         __syncwarp();
         const int kn = next_step(k);
         if (kn >= 0) load_step(kn);         // in flight while this step is tested
         ++active_steps;
-        // broad phase: candidate bit MJ m + n (bits 0-63 in c_lo, 64-127 in c_hi)
+        // broad phase: candidate bit MJ m + n
         float ax[MI], ay[MI], ah[MI];
 #pragma unroll
         for (int m = 0; m < MI; ++m) {
             const float4 q = pa_s[lr + 8 * m];
             ax[m] = q.x; ay[m] = q.y; ah[m] = q.z;
         }
-        unsigned long long c_lo = 0ull, c_hi = 0ull;
+        unsigned cand = 0u;
 #pragma unroll
         for (int n = 0; n < MJ; ++n) {
             const float4 qb = pb_s[lc + 4 * n];
 #pragma unroll
-            for (int m = 0; m < MI; ++m) {
-                if (fmaf(ax[m], qb.x, fmaf(ay[m], qb.y, -qb.z)) >= ah[m]) {
-                    const int bit = MJ * m + n;
-                    if (bit < 64) c_lo |= 1ull << bit;
-                    else c_hi |= 1ull << (bit - 64);
-                }
-            }
+            for (int m = 0; m < MI; ++m)
+                if (fmaf(ax[m], qb.x, fmaf(ay[m], qb.y, -qb.z)) >= ah[m]) cand |= 1u << (MJ * m + n);
         }
-        c_lo &= ~found_lo;
-        c_hi &= ~found_hi;
-        if (__ballot_sync(0xffffffffu, (c_lo | c_hi) != 0ull)) {
+        cand &= ~found;
+        if (__ballot_sync(0xffffffffu, cand != 0u)) {
             bool any_hit = false;
             unsigned long long step_cnt = 0, step_mass = 0;
             // each lane tests the candidates of its own micro-block (a loop as long as the lane with the most;
             // measured faster than compacting them into a warp queue first), so a hit sets its own mask bit
-            for (int h = 0; h < 2; ++h) {
-                unsigned long long cm = h ? c_hi : c_lo;
-                while (cm) {
-                    const int bit = 64 * h + __ffsll((long long)cm) - 1;
-                    cm &= cm - 1ull;
-                    ++narrow;
-                    const int m = bit / MJ, n = bit % MJ;
-                    const int i = lr + 8 * m, j = lc + 4 * n;
-                    const float4 qa4 = pa_s[i], qb4 = pb_s[j];
-                    const float dx = qb4.x - qa4.x, dy = qb4.y - qa4.y;
-                    const float2 qa = ra_s[i], qb = rb_s[j];
-                    if (!narrow_hit<OUTL>(shape, a.polys, dx, dy, qa, qb, la, wa, lb, wb, ra, rb)) continue;
-                    any_hit = true;
-                    if (h) found_hi |= 1ull << (bit - 64); else found_lo |= 1ull << bit;
-                    a.table[P.off + (long long)(i0 + i) * B.h + j0 + j] = (int16_t)k;
-                    if (FUSED) {
-                        const float pa_ = prob_s[i], pb_ = prob_s[TE + j];
-                        const unsigned long long w = to_fixed(pa_ * pb_, kFixProb);
-                        ++step_cnt;
-                        step_mass += w;
-                        if (P.ego_side >= 0) {
-                            const int e = P.ego_side == 0 ? i0 + i : j0 + j;     // the EGO hypothesis
-                            const float pco = P.ego_side == 0 ? pb_ : pa_;       // the CO hypothesis
-                            atomicAdd(a.acc.mass + P.mass_base + (long long)e * P.n_obj_s + P.co_local,
-                                      to_fixed(pco, kFixProb));
-                            atomicAdd(a.acc.hits + P.hits_base + e, 1ull);
-                            atomicAdd(a.acc.lsum + P.lsum_base + ((long long)e * N + k) * P.n_obj_s + P.co_local,
-                                      to_fixed(neg_log_survival(pco), kFixLog));
-                        }
+            while (cand) {
+                const int bit = __ffs(cand) - 1;
+                cand &= cand - 1u;
+                ++narrow;
+                const int m = bit / MJ, n = bit % MJ;
+                const int i = lr + 8 * m, j = lc + 4 * n;
+                const float4 qa4 = pa_s[i], qb4 = pb_s[j];
+                const float dx = qb4.x - qa4.x, dy = qb4.y - qa4.y;
+                const float2 qa = ra_s[i], qb = rb_s[j];
+                if (!narrow_hit<OUTL>(shape, a.polys, dx, dy, qa, qb, la, wa, lb, wb, ra, rb)) continue;
+                any_hit = true;
+                found |= 1u << bit;
+                a.table[P.off + (long long)(i0 + i) * B.h + j0 + j] = (int16_t)k;
+                if (FUSED) {
+                    const float pa_ = prob_s[i], pb_ = prob_s[32 + j];
+                    const unsigned long long w = to_fixed(pa_ * pb_, kFixProb);
+                    ++step_cnt;
+                    step_mass += w;
+                    if (P.ego_side >= 0) {
+                        const int e = P.ego_side == 0 ? i0 + i : j0 + j;     // the EGO hypothesis
+                        const float pco = P.ego_side == 0 ? pb_ : pa_;       // the CO hypothesis
+                        atomicAdd(a.acc.mass + P.mass_base + (long long)e * P.n_obj_s + P.co_local,
+                                  to_fixed(pco, kFixProb));
+                        atomicAdd(a.acc.hits + P.hits_base + e, 1ull);
+                        atomicAdd(a.acc.lsum + P.lsum_base + ((long long)e * N + k) * P.n_obj_s + P.co_local,
+                                  to_fixed(neg_log_survival(pco), kFixLog));
                     }
                 }
             }
@@ -1064,7 +824,7 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
     }
     if (a.counters && lane == 0) {
         if (narrow) count_narrow(a, P.combo, narrow);
-        if (active_steps) atomicAdd(a.counters, (unsigned long long)active_steps * TE * TE);
+        if (active_steps) atomicAdd(a.counters, (unsigned long long)active_steps * 32 * 32);
     }
     if (FUSED && lane == 0 && hit_cnt) {
         atomicAdd(a.acc.count + P.index, hit_cnt);
@@ -1072,21 +832,16 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
     }
 }
 
-// The warp-per-block layouts: each warp takes blocks gw = blockIdx.x * WARPS + warp, then every
-// gridDim.x * WARPS further (a grid smaller than the work, max_ctas, leaves SM room to other streams).
-template <int WARPS, int TE, bool FUSED, bool OUTL>
-__global__ void __launch_bounds__(WARPS * 32, (TE == 64 ? 16 : 24) / WARPS) collide_tile_kernel(const CollideArgs a) {
+// Each warp (a CTA of its own: a finished warp frees its slot at once) takes blocks gw = blockIdx.x, then every
+// gridDim.x further (a grid smaller than the work, max_ctas, leaves SM room to other streams).
+template <bool FUSED, bool OUTL>
+__global__ void __launch_bounds__(32, 24) collide_tile_kernel(const CollideArgs a) {
     pdl_start();
-    constexpr int SUB = kTile / TE;
-    __shared__ float4 s_pa[WARPS][TE];            // x, y, h_a
-    __shared__ float4 s_pb[WARPS][TE];            // x, y, h_b
-    __shared__ float2 s_ra[WARPS][TE];            // c, s
-    __shared__ float2 s_rb[WARPS][TE];
-    __shared__ float s_prob[WARPS][FUSED ? 2 * TE : 1];    // fused: the block's row and column probabilities
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long total = a.n_tiles * (SUB * SUB);
-    for (long long gw = (long long)blockIdx.x * WARPS + warp; gw < total; gw += (long long)gridDim.x * WARPS)
-        tile_block<TE, FUSED, OUTL>(a, gw, lane, s_pa[warp], s_pb[warp], s_ra[warp], s_rb[warp], s_prob[warp]);
+    __shared__ float4 s_pa[32], s_pb[32];         // x, y, h
+    __shared__ float2 s_ra[32], s_rb[32];         // c, s
+    __shared__ float s_prob[FUSED ? 64 : 1];      // fused: the block's row and column probabilities
+    for (long long gw = blockIdx.x; gw < a.n_tiles * 4; gw += gridDim.x)
+        tile_block<FUSED, OUTL>(a, gw, threadIdx.x, s_pa, s_pb, s_ra, s_rb, s_prob);
 }
 
 // ---- step-item layout (variant 6): the active (block, step) pairs of a small scene in parallel ----------
@@ -1468,18 +1223,6 @@ struct BlockJob {
     float rcull, rc2, la, wa, ra, lb, wb, rb;
 };
 
-// Asynchronous 4- and 8-byte copies global -> shared (both addresses aligned to the size); cp_async_wait()
-// returns once the calling thread's copies have landed (a barrier then shows them to the CTA).
-__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // Active steps k0 .. k0 + 31 of a block (one ballot over the two bound tiles' boxes; every lane calls it).
 __device__ __forceinline__ unsigned block_chunk_mask(const CollideArgs &a, const BlockJob &J, int k0) {
     const int k = k0 + (threadIdx.x & 31);
@@ -1834,15 +1577,12 @@ cudaError_t launch_warp_variant(const CollideArgs &a, cudaStream_t st, bool pdl)
                          smem, st, pdl, a);
 }
 
-template <int WARPS, int TE, bool FUSED, bool OUTL>
+template <bool FUSED, bool OUTL>
 cudaError_t launch_tile_variant(const CollideArgs &a, cudaStream_t st, bool pdl) {
-    constexpr int SUB = kTile / TE;
-    const long long warps = a.n_tiles * SUB * SUB;
-    long long blocks = (warps + WARPS - 1) / WARPS;
+    long long blocks = a.n_tiles * 4;
     if (a.max_ctas > 0 && blocks > a.max_ctas) blocks = a.max_ctas;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    return launch_kernel(collide_tile_kernel<WARPS, TE, FUSED, OUTL>, dim3((unsigned)blocks), dim3(WARPS * 32), 0,
-                         st, pdl, a);
+    return launch_kernel(collide_tile_kernel<FUSED, OUTL>, dim3((unsigned)blocks), dim3(32), 0, st, pdl, a);
 }
 
 template <bool OUTL>
@@ -1883,10 +1623,9 @@ cudaError_t launch_collide_t(const CollideArgs &a, cudaStream_t st, bool pdl) {
         return a.probf ? launch_kernel(block_kernel<kBlockWarps, true, OUTL>, grid, block, 0, st, pdl, a)
                        : launch_kernel(block_kernel<kBlockWarps, false, OUTL>, grid, block, 0, st, pdl, a);
     }
-    if (a.variant == 4)
-        return a.probf ? launch_tile_variant<4, 64, true, OUTL>(a, st, pdl) : launch_tile_variant<4, 64, false, OUTL>(a, st, pdl);
+    if (a.variant == 4) return launch_tiles(a, st, pdl);
     if (a.variant == 5)   // one warp per CTA: a finished warp frees its slot at once (small, uneven grids)
-        return a.probf ? launch_tile_variant<1, 32, true, OUTL>(a, st, pdl) : launch_tile_variant<1, 32, false, OUTL>(a, st, pdl);
+        return a.probf ? launch_tile_variant<true, OUTL>(a, st, pdl) : launch_tile_variant<false, OUTL>(a, st, pdl);
     // variant 1: 4 x 4 micro-tiles with 256 threads (8 warps share each tile's tests); variant 2: 8 x 8 with
     // 64 threads; variant 3: one warp per step (8 x 16 lanes).  The caller picks one (autotuned per size).
     const bool many = a.variant == 2;

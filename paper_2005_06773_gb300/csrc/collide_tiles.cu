@@ -1,0 +1,392 @@
+// collide_tiles.cu -- collision layout 4: a warp per active 32 x 32 block of hypothesis pairs, in the objects' tile
+// order.
+//
+// The bounds kernel has written each object's poses tile by tile (CollideArgs::tile_poses: 32 poses of one step side
+// by side, in the compact order of hypothesis_at) together with the boxes around them, so that a block's active
+// steps are few and a step's poses are one 16-byte load per lane and side.  Without that array (culling off, or an
+// arena sized to the least) the same kernels take ascending tiles and read the pose planes.
+//
+// A step of a block, by one warp: the 32 + 32 poses go to a shared slot, the broad phase runs on a 4 x 8 micro-block
+// per lane (rows lr + 8 m, columns lc + 4 n), and the candidates are queued and tested one per lane.  Compact tiles
+// put 30 to 70 candidates into an active step, on few lanes (the lane with the most has four to eight): a loop over
+// each lane's own candidates would run the exact test with a quarter of the lanes busy, and one over the rows that
+// have any (a lane per column) with a fifth (3.7 ms against 2.7 ms on 32 cars).
+#include <algorithm>
+#include <cstdint>
+
+#include "collide_common.cuh"
+
+namespace mhc {
+namespace {
+
+constexpr int MI = 4, MJ = 8;          // micro-block of a lane
+
+// One step's poses in shared memory.
+struct StepSlot {
+    float4 pa[32], pb[32];             // x, y, h of the broad phase
+    float4 qa[32], qb[32];             // x, y, c, s
+};
+
+// This lane's row of a and column of b at one step.
+struct StepPoses {
+    float4 a, b;
+};
+
+// One side's pose `idx` of the tile-ordered array, or of the planes; past the object's end: far from everything.
+template <bool TILED>
+__device__ __forceinline__ float4 load_pose(const CollideArgs &a, long long idx, bool ok, float far) {
+    if (TILED) return __ldg(a.tile_poses + idx);     // x = NaN past the end: no test passes
+    return ok ? make_float4(__ldg(a.x + idx), __ldg(a.y + idx), __ldg(a.c + idx), __ldg(a.s + idx))
+              : make_float4(far, 0.0f, 1.0f, 0.0f);
+}
+
+// The shapes of a pair: the half extents of rectangles, the radii of discs.
+struct Extents {
+    float la, wa, ra, lb, wb, rb;
+};
+
+// Stages a step's poses in a slot and returns the lane's broad-phase candidates (bit MJ m + n).
+__device__ __forceinline__ unsigned stage_and_sweep(StepSlot &S, const StepPoses &p, float rc2, int lane) {
+    const int lr = lane >> 2, lc = lane & 3;
+    const float ka = 0.5f * (1.0f - kEps);
+    S.pa[lane] = make_float4(p.a.x, p.a.y, ka * fmaf(p.a.x, p.a.x, p.a.y * p.a.y), 0.0f);
+    S.pb[lane] = make_float4(p.b.x, p.b.y, 0.5f * fmaf(1.0f - kEps, fmaf(p.b.x, p.b.x, p.b.y * p.b.y), -rc2), 0.0f);
+    S.qa[lane] = p.a;
+    S.qb[lane] = p.b;
+    __syncwarp();
+    float ax[MI], ay[MI], ah[MI];
+#pragma unroll
+    for (int m = 0; m < MI; ++m) {
+        const float4 q = S.pa[lr + 8 * m];
+        ax[m] = q.x; ay[m] = q.y; ah[m] = q.z;
+    }
+    unsigned cand = 0u;
+#pragma unroll
+    for (int n = 0; n < MJ; ++n) {
+        const float4 q = S.pb[lc + 4 * n];
+#pragma unroll
+        for (int m = 0; m < MI; ++m)
+            if (fmaf(ax[m], q.x, fmaf(ay[m], q.y, -q.z)) >= ah[m]) cand |= 1u << (MJ * m + n);
+    }
+    return cand;
+}
+
+// A queued candidate: lane << 5 | bit of its micro-block, and the row and column that means.
+__device__ __forceinline__ int queued_row(int e) { return (e >> 7 & 7) + (e & 24); }
+__device__ __forceinline__ int queued_col(int e) { return (e >> 5 & 3) + 4 * (e & 7); }
+
+template <bool OUTL>
+__device__ __forceinline__ bool overlap(const StepSlot &S, const PairShape &shape, const PolyVertex *polys,
+                                        const Extents &x, int e) {
+    const float4 qa = S.qa[queued_row(e)], qb = S.qb[queued_col(e)];
+    return narrow_hit<OUTL>(shape, polys, qb.x - qa.x, qb.y - qa.y, make_float2(qa.z, qa.w), make_float2(qb.z, qb.w),
+                            x.la, x.wa, x.lb, x.wb, x.ra, x.rb);
+}
+
+__device__ __forceinline__ bool boxes_meet(const float4 &a, const float4 &b, float r) {
+    return (a.x - r <= b.z) && (b.x - r <= a.z) && (a.y - r <= b.w) && (b.y - r <= a.w);
+}
+
+// Active steps among k0 .. k0 + 31 of the four 32 x 32 blocks of a 64 x 64 tile (bit b of m[2 qa + qb]: step k0 + b;
+// qa / qb: the second 32 rows / columns), one ballot each.  box_a, box_b: the tile's first boxes.
+struct TileBoxes {
+    long long box_a, box_b;
+    int N;
+    bool two_a, two_b;                 // the tile has a second 32 rows / columns
+    float r_cull;
+};
+
+__device__ __forceinline__ void active_steps(const CollideArgs &a, const TileBoxes &T, int k0, int lane, unsigned m[4]) {
+    const int k = k0 + lane;
+    bool m00 = k < T.N, m01 = m00 && T.two_b, m10 = m00 && T.two_a, m11 = m01 && T.two_a;
+    if (a.cull && m00) {
+        const float4 a0 = a.bounds[T.box_a + k], b0 = a.bounds[T.box_b + k];
+        const float4 a1 = T.two_a ? a.bounds[T.box_a + T.N + k] : a0, b1 = T.two_b ? a.bounds[T.box_b + T.N + k] : b0;
+        m00 = boxes_meet(a0, b0, T.r_cull);
+        m01 = m01 && boxes_meet(a0, b1, T.r_cull);
+        m10 = m10 && boxes_meet(a1, b0, T.r_cull);
+        m11 = m11 && boxes_meet(a1, b1, T.r_cull);
+    }
+    m[0] = __ballot_sync(0xffffffffu, m00);
+    m[1] = __ballot_sync(0xffffffffu, m01);
+    m[2] = __ballot_sync(0xffffffffu, m10);
+    m[3] = __ballot_sync(0xffffffffu, m11);
+}
+
+// Sum of v over the warp (v <= 2^62, and the sum too): three 32-bit reductions.
+__device__ __forceinline__ unsigned long long reduce_terms(unsigned long long v) {
+    const unsigned m0 = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xffffffu);
+    const unsigned m1 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 24) & 0xffffffu);
+    const unsigned m2 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 48));
+    return m0 + ((unsigned long long)m1 << 24) + ((unsigned long long)m2 << 48);
+}
+
+// ---- the list of active blocks ------------------------------------------------------------------------------
+//
+// The walk runs over the blocks that come close only (a fifth to a quarter of them), those with many active steps
+// first: a warp that starts last then has little to do.  A warp lists `per_warp` consecutive 64 x 64
+// tiles: lane 4 u + q keeps block q (rows 32 (q >> 1), columns 32 (q & 1)) of tile u.  Large scenes take 8 tiles per
+// warp, one search for eight tiles and one pair of atomics per CTA; small ones 1, to use every SM.
+constexpr int kListWarps = 8;
+constexpr int kHeavySteps = 12;         // active steps from which a block is listed from the front
+
+__global__ void __launch_bounds__(32 * kListWarps) block_list_kernel(const CollideArgs a, int per_warp) {
+    pdl_trigger();
+    __shared__ int s_heavy[kListWarps], s_light[kListWarps];
+    __shared__ unsigned long long s_at[2];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long g0 = ((long long)blockIdx.x * kListWarps + w) * per_warp;
+    BlockRef ref{};
+    int n = 0;                                      // active steps of this lane's block
+    int pair = 0;
+    if (g0 < a.n_tiles) pair = pair_of_tile(a, g0);   // uploaded data: before the wait
+    pdl_wait();
+    const int mine = lane >> 2, q = lane & 3;
+    for (int u = 0; u < per_warp && g0 + u < a.n_tiles; ++u) {
+        const long long g = g0 + u;
+        while (pair + 1 < a.n_pairs && a.pairs[pair + 1].tile_start <= g) ++pair;
+        const PairDesc &P = a.pairs[pair];
+        const int t = (int)(g - P.tile_start);      // < tiles_a x tiles_b <= n_tiles < 2^31
+        const int ta = t / P.tiles_b, tb = t - ta * P.tiles_b, N = P.n_steps;
+        const TileBoxes T{P.bounds_a + (long long)(2 * ta) * N, P.bounds_b + (long long)(2 * tb) * N, N,
+                          ta * kTile + 32 < P.h_a, tb * kTile + 32 < P.h_b, P.r_cull};
+        if (mine == u) {
+            ref.pair = pair;
+            ref.tile_a = 2 * ta + (q >> 1);
+            ref.tile_b = 2 * tb + (q & 1);
+        }
+        for (int k0 = 0; k0 < N; k0 += 32) {
+            unsigned m[4];
+            active_steps(a, T, k0, lane, m);
+            if (mine == u) n += __popc(q < 2 ? (q ? m[1] : m[0]) : (q == 2 ? m[2] : m[3]));
+        }
+    }
+    const unsigned active = __ballot_sync(0xffffffffu, n > 0), heavy = __ballot_sync(0xffffffffu, n >= kHeavySteps);
+    const unsigned light = active & ~heavy, lt = (1u << lane) - 1u;
+    if (lane == 0) { s_heavy[w] = __popc(heavy); s_light[w] = __popc(light); }
+    __syncthreads();
+    int h0 = 0, l0 = 0, hn = 0, ln = 0;
+#pragma unroll
+    for (int v = 0; v < kListWarps; ++v) {
+        if (v == w) { h0 = hn; l0 = ln; }
+        hn += s_heavy[v];
+        ln += s_light[v];
+    }
+    if (threadIdx.x == 0 && hn) s_at[0] = atomicAdd(a.list_counts, (unsigned long long)hn);
+    if (threadIdx.x == 32 && ln) s_at[1] = atomicAdd(a.list_counts + 1, (unsigned long long)ln);
+    __syncthreads();
+    if (n == 0) return;
+    // at most 4 blocks per tile: the front and the back never meet
+    if (heavy >> lane & 1u) a.list[s_at[0] + h0 + __popc(heavy & lt)] = ref;
+    else a.list[4 * a.n_tiles - 1 - (long long)(s_at[1] + l0 + __popc(light & lt))] = ref;
+}
+
+// Entry `it` of the list (heavy blocks first); `front`, `listed`: its heavy blocks and all.
+__device__ __forceinline__ BlockRef listed_block(const CollideArgs &a, long long it, long long front) {
+    return a.list[it < front ? it : 4 * a.n_tiles - 1 - (it - front)];
+}
+
+// ---- layout 4: a warp per block, its steps in ascending order -------------------------------------------------
+//
+// A block's steps come in order, so the first overlap of a pair is its first collision step: it is stored at once,
+// and the pair's bit in `found` drops its later candidates.  The warps take the listed blocks one after another from
+// a counter, up to kWalkBlocks each.  Without the list (UNLISTED: culling off, or no room for the tile-ordered poses) they take every block
+// of ascending tiles, strided, and read the pose planes.
+//
+// Bound by instruction issue: about 400 warp instructions per (block, step) item, half of them the sweep.  Measured
+// (collision stage, listing included): 32 cars of 2048 hypotheses 1.79 ms, 256 uneven scenarios 6.3 ms; a warp per 64 x
+// 64 tile of consecutive hypotheses took 4.77 and 11.8 ms (five and two times the executed tests), compact tiles
+// without the list 2.67 and 8.9 ms (a third of the launch was its last warps), with it but with warps that stay until
+// the list is empty 1.73 ms (requests of higher priority then wait for the whole launch).
+constexpr int kWalkWarps = 4;
+constexpr int kWalkCtas = 6;            // per SM: bounds the registers to 80
+constexpr int kWalkBlocks = 16;         // blocks a warp takes before its CTA makes room (for a stream of higher priority)
+
+struct WalkSlot {
+    StepSlot step;
+    unsigned short queue[8 * 32];      // the candidates of one round: at most 8 of each lane
+    unsigned found[32];                // [lane] micro-block pairs that have hit
+    int order[2][32];                  // hypotheses of the rows and columns
+    float prob[2][32];                 // their probabilities (fused)
+};
+
+template <bool FUSED, bool OUTL, bool UNLISTED>
+__device__ __forceinline__ void walk_block(const CollideArgs &a, const BlockRef &B, int lane, WalkSlot &S) {
+    const PairDesc &P = a.pairs[B.pair];               // fields read where used (fewer live registers)
+    const int ha = P.h_a, hb = P.h_b, N = P.n_steps;
+    const int ia = 32 * B.tile_a + lane, jb = 32 * B.tile_b + lane;   // this lane's positions
+    const long long box_a = P.bounds_a + (long long)B.tile_a * N, box_b = P.bounds_b + (long long)B.tile_b * N;
+    const float r_cull = P.r_cull;
+    auto chunk = [&](int k0) -> unsigned {             // active steps among k0 .. k0 + 31
+        const int k = k0 + lane;
+        bool act = k < N;
+        if (act && (!UNLISTED || a.cull)) act = boxes_meet(a.bounds[box_a + k], a.bounds[box_b + k], r_cull);
+        return __ballot_sync(0xffffffffu, act);
+    };
+    int k0 = 0;
+    unsigned mask = chunk(0);
+    auto next = [&]() -> int {
+        while (!mask) {
+            k0 += 32;
+            if (k0 >= N) return -1;
+            mask = chunk(k0);
+        }
+        const int b = __ffs(mask) - 1;
+        mask &= mask - 1u;
+        return k0 + b;
+    };
+    int k = next();
+    if (k < 0) return;
+    StepPoses cur;
+    auto load = [&](int kk) {
+        if (UNLISTED) {
+            cur.a = load_pose<false>(a, P.pose_a + (long long)kk * ha + ia, ia < ha, kFar);
+            cur.b = load_pose<false>(a, P.pose_b + (long long)kk * hb + jb, jb < hb, -kFar);
+        } else {
+            cur.a = load_pose<true>(a, 32 * (box_a + kk) + lane, true, 0.0f);
+            cur.b = load_pose<true>(a, 32 * (box_b + kk) + lane, true, 0.0f);
+        }
+    };
+    load(k);
+    {
+        const int hi = UNLISTED ? ia : a.tile_order[32LL * (P.tile_a + B.tile_a) + lane];
+        const int hj = UNLISTED ? jb : a.tile_order[32LL * (P.tile_b + B.tile_b) + lane];
+        S.order[0][lane] = hi;
+        S.order[1][lane] = hj;
+        S.found[lane] = 0u;
+        if (FUSED) {
+            S.prob[0][lane] = ia < ha ? a.probf[P.traj_a + hi] : 0.0f;
+            S.prob[1][lane] = jb < hb ? a.probf[P.traj_b + hj] : 0.0f;
+        }
+    }
+    const PairShape shape = shape_of(P);
+    const Extents ext{P.hl_a, P.hw_a, P.rad_a, P.hl_b, P.hw_b, P.rad_b};
+    const float rc2 = P.rc2 + kEps0;
+    const int ego_side = P.ego_side;
+    unsigned narrow = 0;
+    unsigned long long hit_cnt = 0, hit_mass = 0;
+    int steps = 0;
+    while (k >= 0) {
+        __syncwarp();                   // the previous step's slot is no longer read
+        unsigned cand = stage_and_sweep(S.step, cur, rc2, lane) & ~S.found[lane];
+        const int kn = next();
+        if (kn >= 0) load(kn);          // in flight while this step's candidates are tested
+        ++steps;
+        unsigned cnt = 0;
+        unsigned long long mass = 0;
+        for (;;) {                      // rounds of at most 8 candidates of each lane
+            const int n = min(__popc(cand), 8);
+            int off, total;
+            if (!queue_offsets(n, lane, off, total)) break;
+            for (int u = 0; u < n; ++u, cand &= cand - 1u) S.queue[off + u] = (unsigned short)(lane << 5 | (__ffs(cand) - 1));
+            __syncwarp();
+            narrow += total;
+            for (int u = lane; u < total; u += 32) {
+                const int e = S.queue[u];
+                if (!overlap<OUTL>(S.step, shape, a.polys, ext, e)) continue;
+                atomicOr(&S.found[e >> 5], 1u << (e & 31));
+                const int i = queued_row(e), j = queued_col(e), hi = S.order[0][i], hj = S.order[1][j];
+                a.table[P.off + (long long)hi * hb + hj] = (int16_t)k;
+                ++cnt;
+                if (!FUSED) continue;
+                mass += to_fixed(S.prob[0][i] * S.prob[1][j], kFixProb);
+                if (ego_side >= 0) {
+                    const int eg = ego_side == 0 ? hi : hj;                              // the EGO hypothesis
+                    const long long co = ego_side == 0 ? P.traj_b + hj : P.traj_a + hi;  // the CO hypothesis
+                    atomicAdd(a.acc.mass + P.mass_base + (long long)eg * P.n_obj_s + P.co_local, a.pfix[co]);
+                    atomicAdd(a.acc.hits + P.hits_base + eg, 1ull);
+                    atomicAdd(a.acc.lsum + P.lsum_base + ((long long)eg * N + k) * P.n_obj_s + P.co_local, a.lfix[co]);
+                }
+            }
+            __syncwarp();
+        }
+        if (FUSED && __any_sync(0xffffffffu, cnt != 0u)) {   // the step's terms summed over the warp
+            const unsigned c = __reduce_add_sync(0xffffffffu, cnt);
+            mass = reduce_terms(mass);
+            if (lane == 0) {
+                atomicAdd(a.acc.count_k + P.kofs + k, (unsigned long long)c);
+                atomicAdd(a.acc.H + P.kofs + k, mass);
+            }
+            hit_cnt += c;
+            hit_mass += mass;
+        }
+        k = kn;
+    }
+    if (lane != 0) return;
+    if (a.counters) {
+        if (narrow) count_narrow(a, P.combo, narrow);
+        atomicAdd(a.counters, (unsigned long long)steps * 32 * 32);
+    }
+    if (FUSED && hit_cnt) {
+        atomicAdd(a.acc.count + P.index, hit_cnt);
+        atomicAdd(a.acc.P + P.index, hit_mass);
+    }
+}
+
+template <bool FUSED, bool OUTL, bool UNLISTED>
+__global__ void __launch_bounds__(32 * kWalkWarps, kWalkCtas) walk_kernel(const CollideArgs a) {
+    pdl_start();
+    __shared__ WalkSlot slots[kWalkWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    WalkSlot &S = slots[warp];
+    if (UNLISTED) {                                 // every 32 x 32 block of every tile (four per tile)
+        const long long stride = (long long)gridDim.x * kWalkWarps;
+        for (long long gw = (long long)blockIdx.x * kWalkWarps + warp; gw < 4 * a.n_tiles; gw += stride) {
+            BlockRef B;
+            B.pair = pair_of_tile(a, gw >> 2);
+            const PairDesc &P = a.pairs[B.pair];
+            const int t = (int)((gw >> 2) - P.tile_start), ta = t / P.tiles_b, q = (int)(gw & 3);
+            B.tile_a = 2 * ta + (q >> 1);
+            B.tile_b = 2 * (t - ta * P.tiles_b) + (q & 1);
+            if (32 * B.tile_a < P.h_a && 32 * B.tile_b < P.h_b) walk_block<FUSED, OUTL, true>(a, B, lane, S);
+            __syncwarp();
+        }
+        return;
+    }
+    const long long front = (long long)a.list_counts[0], listed = front + (long long)a.list_counts[1];
+    unsigned long long taken = 0;
+    if (lane == 0) taken = atomicAdd(a.list_counts + 2, 1ull);
+    for (int u = 0; u < kWalkBlocks; ++u) {
+        const long long it = (long long)__shfl_sync(0xffffffffu, taken, 0);
+        if (it >= listed) return;
+        if (lane == 0 && u + 1 < kWalkBlocks) taken = atomicAdd(a.list_counts + 2, 1ull);   // in flight meanwhile
+        walk_block<FUSED, OUTL, false>(a, listed_block(a, it, front), lane, S);
+        __syncwarp();
+    }
+}
+
+template <bool OUTL>
+cudaError_t launch_listed(const CollideArgs &a, cudaStream_t st, bool pdl) {
+    // 8 tiles per warp once that still gives every SM a few warps
+    const int per_warp = a.n_tiles >= 152LL * 8 * 32 ? 8 : 1;
+    const long long tiles = (long long)kListWarps * per_warp;
+    cudaError_t e = launch_kernel(block_list_kernel, dim3((unsigned)((a.n_tiles + tiles - 1) / tiles)), dim3(32 * kListWarps),
+                                  0, st, pdl, a, per_warp);
+    if (e != cudaSuccess) return e;
+    // CTAs for every block of every tile (the warps of those past the last listed block leave at once)
+    const long long ctas = (4 * a.n_tiles + kWalkWarps * kWalkBlocks - 1) / (kWalkWarps * kWalkBlocks);
+    const dim3 grid((unsigned)ctas), block(32 * kWalkWarps);
+    return a.probf ? launch_kernel(walk_kernel<true, OUTL, false>, grid, block, 0, st, true, a)
+                   : launch_kernel(walk_kernel<false, OUTL, false>, grid, block, 0, st, true, a);
+}
+
+template <bool OUTL>
+cudaError_t launch_unlisted(const CollideArgs &a, cudaStream_t st, bool pdl) {
+    long long ctas = a.n_tiles;                     // a warp per block
+    if (a.max_ctas > 0 && ctas > a.max_ctas) ctas = a.max_ctas;
+    const dim3 grid((unsigned)ctas), block(32 * kWalkWarps);
+    return a.probf ? launch_kernel(walk_kernel<true, OUTL, true>, grid, block, 0, st, pdl, a)
+                   : launch_kernel(walk_kernel<false, OUTL, true>, grid, block, 0, st, pdl, a);
+}
+
+}  // namespace
+
+cudaError_t launch_tiles(const CollideArgs &a, cudaStream_t st, bool pdl) {
+    if (a.tile_poses) {     // the table's -1s and the list's counts are written beforehand
+        if (!a.tile_order || !a.list || !a.list_counts) return cudaErrorInvalidValue;
+        return a.polys ? launch_listed<true>(a, st, pdl) : launch_listed<false>(a, st, pdl);
+    }
+    return a.polys ? launch_unlisted<true>(a, st, pdl) : launch_unlisted<false>(a, st, pdl);
+}
+
+}  // namespace mhc

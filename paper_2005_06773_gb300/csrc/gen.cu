@@ -630,7 +630,10 @@ __global__ void __launch_bounds__(128, 6) gen_kernel(const GenArgs a) {
 // generation kernel, the poses after it.  With `fill` set, the CTAs past the bounds write the table's -1s
 // (16-byte stores on the aligned body) before the wait: nothing earlier in the launch sequence reads the
 // table, so the HBM-rate fill overlaps the generation kernel's tail, and the collision kernel stores first
-// hits only.
+// hits only.  TILED: the tiles are taken in the objects' tile order (hypothesis_at) and the poses go out once more,
+// 512 bytes per tile and step, so that the walk reads a step of a tile with one 16-byte load per lane: 35 us
+// instead of 15 on the 32-vehicle scene, 0.35 ms instead of 0.11 on the 256-scenario batch (HBM: 52 and 340 MB of
+// poses read and written), for collision kernels 2.9 and 5.4 ms shorter.
 constexpr int kFillCtas = 152 * 4;
 // Fill CTAs of the generation launch (the rest of each SM integrates).  Two per SM spread the fill's stores
 // over every SM, which a table much larger than the generation work needs to reach the HBM rate (32-vehicle
@@ -643,6 +646,7 @@ constexpr int kBoundSteps = 8;          // steps per warp task
 
 __device__ __forceinline__ float box_op(bool is_max, float u, float v) { return is_max ? fmaxf(u, v) : fminf(u, v); }
 
+template <bool TILED>
 __global__ void __launch_bounds__(256) bounds_kernel(const BoundsArgs a) {
     pdl_trigger();
     const int chunks = (a.max_steps + kBoundSteps - 1) / kBoundSteps;
@@ -656,7 +660,7 @@ __global__ void __launch_bounds__(256) bounds_kernel(const BoundsArgs a) {
     const long long g = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     bool live = g < total;
-    int k0 = 0, first = 0, h = 0, n_steps = 0;
+    int k0 = 0, first = 0, h = 0, n_steps = 0, i = 0, tile = 0;
     long long pose_base = 0, bounds_base = 0;
     if (live) {
         const int w = (int)(g / chunks);
@@ -666,25 +670,38 @@ __global__ void __launch_bounds__(256) bounds_kernel(const BoundsArgs a) {
         h = o.h;
         n_steps = o.n_steps;
         pose_base = o.pose_base;
-        bounds_base = o.bounds_base;
+        bounds_base = o.bounds_base + (long long)(first / kBoundTile) * n_steps;
+        i = first + lane;                           // past the object's end: not loaded
+        tile = w;
+        if (TILED && i < h) i = hypothesis_at(o, i);
     }
     pdl_wait();
     if (a.zero_counts && g == 0 && lane == 0) {
         a.zero_counts[0] = 0ull;
         a.zero_counts[1] = 0ull;
+        a.zero_counts[2] = 0ull;
     }
     if (!live || k0 >= n_steps) return;             // uniform over the warp
-    const int i = first + lane;
+    if (TILED && k0 == 0) a.tile_order[32LL * tile + lane] = i;
     float v[4 * kBoundSteps];                       // value 4 s + q of step k0 + s
+    float cv[kBoundSteps], sv[kBoundSteps];         // the headings, for the poses in tile order
 #pragma unroll
     for (int s = 0; s < kBoundSteps; ++s) {
         const bool ok = i < h && k0 + s < n_steps;
         const long long idx = pose_base + (long long)(k0 + s) * h + i;
         const float x = ok ? a.x[idx] : INFINITY, y = ok ? a.y[idx] : INFINITY;
+        cv[s] = TILED && ok ? a.c[idx] : 1.0f;
+        sv[s] = TILED && ok ? a.s[idx] : 0.0f;
         v[4 * s] = x;
         v[4 * s + 1] = y;
         v[4 * s + 2] = ok ? x : -INFINITY;
         v[4 * s + 3] = ok ? y : -INFINITY;
+    }
+    if (TILED) {
+        float4 *tp = a.tile_poses + 32 * (bounds_base + k0) + lane;
+#pragma unroll
+        for (int s = 0; s < kBoundSteps; ++s)
+            if (k0 + s < n_steps) tp[32 * s] = make_float4(i < h ? v[4 * s] : NAN, v[4 * s + 1], cv[s], sv[s]);
     }
     // levels 16, 8, 4: the kept values keep their quantity (q = index mod 4)
 #pragma unroll
@@ -711,7 +728,7 @@ __global__ void __launch_bounds__(256) bounds_kernel(const BoundsArgs a) {
     }
     const int s = lane >> 2;                        // lane L holds value L: step k0 + L / 4, quantity L % 4
     if (k0 + s < n_steps) {
-        float *out = reinterpret_cast<float *>(a.bounds + bounds_base + (long long)(first / kBoundTile) * n_steps + k0);
+        float *out = reinterpret_cast<float *>(a.bounds + bounds_base + k0);
         out[lane] = v[0];
     }
 }
@@ -740,7 +757,8 @@ cudaError_t launch_bounds(const BoundsArgs &a, cudaStream_t st, bool pdl) {
     long long blocks = (total + 7) / 8;
     if (a.fill && a.n_fill > 0) blocks += std::min((long long)kFillCtas, (a.n_fill / 8 + 255) / 256 + 1);
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    return launch_kernel(bounds_kernel, dim3((unsigned)blocks), dim3(256), 0, st, pdl, a);
+    return a.tile_poses ? launch_kernel(bounds_kernel<true>, dim3((unsigned)blocks), dim3(256), 0, st, pdl, a)
+                        : launch_kernel(bounds_kernel<false>, dim3((unsigned)blocks), dim3(256), 0, st, pdl, a);
 }
 
 }  // namespace mhc

@@ -43,7 +43,10 @@ inline void copy_object_fields(PairDesc &p, const ObjDesc &A, const ObjDesc &B) 
     p.h_a = A.h; p.h_b = B.h;
     p.hl_a = A.hl; p.hw_a = A.hw; p.rad_a = A.rad;
     p.hl_b = B.hl; p.hw_b = B.hw; p.rad_b = B.rad;
+    p.tile_a = A.tile_base; p.tile_b = B.tile_base;
 }
+// 64 x 64 collision tiles of a pair.
+inline long long pair_tiles(const PairDesc &p) { return (long long)((p.h_a + kTile - 1) / kTile) * p.tiles_b; }
 constexpr long long kGenScanMaxTraj = 4096;           // a scenario's hypotheses up to which generation is parallel in time
 
 inline size_t align_up(size_t v) { return (v + kAlign - 1) & ~(kAlign - 1); }
@@ -86,6 +89,7 @@ bool items_eligible(const Layout &L);
 // Device scratch each call needs (besides caller buffers).
 struct Scratch {
     size_t desc = 0, bounds = 0, prob = 0, acc = 0, weights = 0, items = 0, total = 0;
+    size_t least = 0;   // `total` without the poses in tile order: the collision kernels then read the planes
     long long acc_words = 0;
 };
 
@@ -138,7 +142,7 @@ struct mhc_ctx {
     bool has_last = false;
     int cull = 1;
     int variant = 0;
-    int collide_max_ctas = 0;        // > 0: CTA cap of the warp-per-block collision layouts (serving's large lane)
+    int collide_max_ctas = 0;        // > 0: CTA cap of collision layout 5 and of 4 without its list (serving's large lane)
     int gen_scan = 2;
     bool score = false;                            // MHC_OPT_SCORE                // generation: 1 a warp per hypothesis (parallel in time), 0 a thread each, 2 auto
     int n_sm = 152;

@@ -63,6 +63,7 @@ struct Batch {
     std::vector<float> w;
     size_t res_off = 0, res_bytes = 0;            // poses, table, risk outputs (resident)
     size_t scr_off = 0, scr_bytes = 0;            // descriptors, weights, bounds, risk scratch
+    size_t scr_least = 0;                         // the same without the poses in tile order
     bool scr_held = false;
     mhc_poses poses{};
     int16_t *table = nullptr;
@@ -215,7 +216,9 @@ Batch *build_batch(Server *S, std::vector<Request *> &take) {
     if (ok) ok = gather_weights(b->L, any_w ? wp.data() : nullptr, b->w) == MHC_OK;
     if (ok) {
         b->res_bytes = resident_bytes(b->L);
-        b->scr_bytes = scratch_of(b->L, !b->w.empty()).total + kAlign;
+        const Scratch sc = scratch_of(b->L, !b->w.empty());
+        b->scr_bytes = sc.total + kAlign;
+        b->scr_least = sc.least + kAlign;
     }
     if (!ok) { delete b; return nullptr; }
     return b;
@@ -225,7 +228,12 @@ Batch *build_batch(Server *S, std::vector<Request *> &take) {
 // puts the requests back).
 bool admit_batch(Server *S, Batch *b, std::vector<Request *> &take) {
     if (!pool_alloc(S->pool, b->res_bytes, &b->res_off)) { b->res_bytes = 0; return false; }
-    if (!(b->scr_held = pool_alloc(S->pool, b->scr_bytes, &b->scr_off))) {
+    b->scr_held = pool_alloc(S->pool, b->scr_bytes, &b->scr_off);
+    if (!b->scr_held && b->scr_least < b->scr_bytes) {
+        b->scr_bytes = b->scr_least;
+        b->scr_held = pool_alloc(S->pool, b->scr_bytes, &b->scr_off);
+    }
+    if (!b->scr_held) {
         pool_free(S->pool, b->res_off);
         b->res_bytes = 0;
         return false;
@@ -501,7 +509,7 @@ int mhc_submit(mhc_ctx *ctx, const mhc_scenario *scen, const float *const *traj_
     r->sc = *scen;
     r->sc.objects = r->objs.data();
     for (const PairDesc &p : L.pairs) r->tests += (long long)L.objs[p.a].h * L.objs[p.b].h * p.n_steps;
-    r->bytes = resident_bytes(L) + scratch_of(L, r->has_w).total + 2 * kAlign;
+    r->bytes = resident_bytes(L) + scratch_of(L, r->has_w).least + 2 * kAlign;
     r->small = r->tests <= S->cfg.small_tests;
     plan_generation(L, S->shadow.n_sm, S->shadow.gen_scan);
     r->L = std::move(L);

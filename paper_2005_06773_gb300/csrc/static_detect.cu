@@ -144,7 +144,6 @@ extern "C" int mhc_detect_collisions_static(const mhc_scenario *sc, const mhc_po
             const ObjDesc &A = objs[a], &B = objs[b];
             p.a = a;
             p.b = b;
-            p.tiles_a = (A.h + kTile - 1) / kTile;
             p.tiles_b = (B.h + kTile - 1) / kTile;
             p.off = entries;
             p.tile_start = tiles;
@@ -157,7 +156,7 @@ extern "C" int mhc_detect_collisions_static(const mhc_scenario *sc, const mhc_po
             p.index = n_pairs - 1;
             mhc::host::copy_object_fields(p, A, B);
             entries += (long long)A.h * B.h;
-            tiles += (long long)p.tiles_a * p.tiles_b;
+            tiles += mhc::host::pair_tiles(p);
         }
     }
     if (tiles > 0x7fffffffLL) return fail(MHC_E_INVALID, "too many collision tiles for one launch");
