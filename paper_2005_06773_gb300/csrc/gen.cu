@@ -24,10 +24,18 @@ __device__ __forceinline__ void kahan_add(float &hi, float &c, float d) {
     hi = t;
 }
 
+// sincosf as one function body: inlined at every use it was most of the generation kernel's code, and a warp that runs
+// its chain once fetches every instruction of it.
+__device__ __noinline__ float2 sincos_any(float x) {
+    float s, c;
+    sincosf(x, &s, &c);
+    return make_float2(s, c);
+}
+
 // sin / cos of the angle (a_hi + a_lo) to first order in the small part a_lo.
 __device__ __forceinline__ void sincos2(float a_hi, float a_lo, float &sn, float &cs) {
-    float s0, c0;
-    sincosf(a_hi, &s0, &c0);
+    const float2 sc = sincos_any(a_hi);
+    const float s0 = sc.x, c0 = sc.y;
     cs = fmaf(-s0, a_lo, c0);
     sn = fmaf(c0, a_lo, s0);
 }
@@ -35,7 +43,9 @@ __device__ __forceinline__ void sincos2(float a_hi, float a_lo, float &sn, float
 // sin / cos by the Taylor series to x^9 / x^10 (|x| <= 0.5: error < 2e-11), sincosf beyond.
 __device__ __forceinline__ void sincos_half(float x, float &sn, float &cs) {
     if (fabsf(x) > 0.5f) {
-        sincosf(x, &sn, &cs);
+        const float2 sc = sincos_any(x);
+        sn = sc.x;
+        cs = sc.y;
         return;
     }
     const float x2 = x * x;
@@ -53,7 +63,9 @@ __device__ __forceinline__ void sincos_half(float x, float &sn, float &cs) {
 // sin / cos by the Taylor series to x^5 / x^6 (|x| <= 0.1: error < 3e-11), sincosf beyond.
 __device__ __forceinline__ void sincos_tenth(float x, float &sn, float &cs) {
     if (fabsf(x) > 0.1f) {
-        sincosf(x, &sn, &cs);
+        const float2 sc = sincos_any(x);
+        sn = sc.x;
+        cs = sc.y;
         return;
     }
     const float x2 = x * x;
@@ -301,7 +313,7 @@ __device__ __forceinline__ void df_add(float &hi, float &lo, float bh, float bl)
 
 // inclusive warp scan of double-float values (lane order = time order)
 __device__ __forceinline__ void df_scan(float &hi, float &lo, int lane) {
-#pragma unroll
+#pragma unroll 1
     for (int d = 1; d < 32; d <<= 1) {
         const float h2 = __shfl_up_sync(0xffffffffu, hi, d), l2 = __shfl_up_sync(0xffffffffu, lo, d);
         if (lane >= d) {
@@ -309,6 +321,21 @@ __device__ __forceinline__ void df_scan(float &hi, float &lo, int lane) {
             df_add(th, tl, hi, lo);
             hi = th;
             lo = tl;
+        }
+    }
+}
+
+// df_scan of two values at once
+__device__ __forceinline__ void df_scan2(float &ah, float &al, float &bh, float &bl, int lane) {
+#pragma unroll 1
+    for (int d = 1; d < 32; d <<= 1) {
+        float a2 = __shfl_up_sync(0xffffffffu, ah, d), a3 = __shfl_up_sync(0xffffffffu, al, d);
+        float b2 = __shfl_up_sync(0xffffffffu, bh, d), b3 = __shfl_up_sync(0xffffffffu, bl, d);
+        if (lane >= d) {
+            df_add(a2, a3, ah, al);
+            df_add(b2, b3, bh, bl);
+            ah = a2; al = a3;
+            bh = b2; bl = b3;
         }
     }
 }
@@ -330,21 +357,34 @@ __device__ __forceinline__ Aff aff_then(const Aff &first, const Aff &second) {
     return r;
 }
 
+// What a lane keeps of its sub-steps between the phases of a round: one slot per sub-step in shared memory (the loops
+// over them stay rolled, a fifth of the unrolled code: the warp runs this chain once, and fetching straight-line code
+// was most of its time).  Latency-bound where a scene has few hypotheses: 32 of them end 6.0 us after the descriptor
+// copy, 11.4 us with the loops unrolled and sincosf inlined at its 17 uses; the 11-object scene's 3,571, six warps per
+// scheduler and by then bound by issue, 11.0 us against 12.8.
+constexpr int kScanSteps = 5;          // sub-steps per lane and round: a 150-sub-step horizon takes one round
+struct ScanSlot {                      // [slip sine, cosine, heading increment, next accelerations, dx, dy][sub-step][lane]
+    float v[7][kScanSteps][32];
+    __device__ __forceinline__ float &at(int q, int c, int lane) { return v[q][c][lane]; }
+};
+
 // One vehicle hypothesis by the whole warp (every lane calls it).  Rounds of 32 x 5 sub-steps; lane L
-// takes sub-steps L*5 .. L*5+4 of the round (five per lane keeps the unrolled loops short and out of
-// local memory; a 150-sub-step horizon still takes one round).  Per round: compose and scan the lanes'
+// takes sub-steps L*5 .. L*5+4 of the round.  Per round: compose and scan the lanes'
 // state maps, run the lanes' sub-steps from their start states (the same per-sub-step arithmetic as the
 // sequential integration), scan the heading increments, form the position increments (heading trig
 // exact at the lane's first sub-step, then rotated by each increment as the sequential integration
 // rotates it), scan them, and store the poses of the output steps that end in each lane's sub-steps
 // (exact heading trig).
 __device__ void vehicle_scan(const ObjDesc &o, float acc, float delta, const Regime &g, int N, int K, int lane,
-                             long long base, int h, int i, float *X, float *Y, float *C, float *S) {
-    constexpr int CS = 5;
+                             long long base, int h, int i, float *X, float *Y, float *C, float *S, ScanSlot &slot) {
+    constexpr int CS = kScanSteps;
+    enum { kSb, kCb, kDps, kAx, kAy, kDx, kDy };
     const int NK = N * K;
+    const int low_lo = g.low_lo, low_hi = g.low_hi, n_stop = g.n_stop;
     const float ti = (float)o.tau_i_d;
     const float hti2 = 0.5f * ti * ti;
     const float dv = (float)__dmul_rn((double)acc, o.tau_i_d);
+    const float v0 = o.v0;
     const float L = o.lf + o.lr;
     const float inv_m = 1.0f / o.m, inv_iz = 1.0f / o.Iz;
     const float k11 = -(o.caf + o.car) * inv_m;
@@ -353,9 +393,12 @@ __device__ void vehicle_scan(const ObjDesc &o, float acc, float delta, const Reg
     const float k22 = -(o.caf * o.lf * o.lf + o.car * o.lr * o.lr) * inv_iz;
     const float kb1 = o.caf * inv_m * delta;
     const float kb2 = o.caf * o.lf * inv_iz * delta;
-    const float tdel = tanf(delta);
-    const float beta_kin = atanf(o.lr * tdel / L);
-    const float kappa = cosf(beta_kin) * tdel / L;
+    float beta_kin = 0.0f, kappa = 0.0f;
+    if (low_lo < min(low_hi, NK)) {                   // (uniform over the warp) the hypothesis enters the low regime
+        const float tdel = tanf(delta);
+        beta_kin = atanf(o.lr * tdel / L);
+        kappa = cosf(beta_kin) * tdel / L;
+    }
     const float stop_den = 0.5f / fabsf(acc == 0.0f ? 1.0f : acc);
 
     float beta = 0.0f, r = 0.0f;                      // lateral state at the round's first sub-step
@@ -367,13 +410,13 @@ __device__ void vehicle_scan(const ObjDesc &o, float acc, float delta, const Reg
         const int n0 = nr + lane * csa;
         // 1. the lane's state map, composed over its sub-steps, and the warp scan of the maps
         Aff F{1.0f, 0.0f, 0.0f, 1.0f, 0.0f, 0.0f};
-#pragma unroll
-        for (int c = 0; c < CS; ++c) {
+#pragma unroll 1
+        for (int c = 0; c < csa; ++c) {
             const int n = n0 + c;
-            if (c >= csa || n >= NK || n >= g.n_stop) continue;   // outside the lane / frozen state: identity
-            const float v = fmaf((float)n, dv, o.v0);
+            if (n >= NK || n >= n_stop) continue;     // past the end / frozen state: identity
+            const float v = fmaf((float)n, dv, v0);
             Aff m;
-            if (n >= g.low_lo && n < g.low_hi) {
+            if (n >= low_lo && n < low_hi) {
                 m = Aff{0.0f, 0.0f, 0.0f, 0.0f, beta_kin, v * kappa};
             } else {
                 const float iv = __fdividef(1.0f, fmaxf(v, 1e-3f));
@@ -383,7 +426,7 @@ __device__ void vehicle_scan(const ObjDesc &o, float acc, float delta, const Reg
             F = aff_then(F, m);
         }
         Aff P = F;
-#pragma unroll
+#pragma unroll 1
         for (int d = 1; d < 32; d <<= 1) {
             Aff q;
             q.m00 = __shfl_up_sync(0xffffffffu, P.m00, d); q.m01 = __shfl_up_sync(0xffffffffu, P.m01, d);
@@ -399,17 +442,15 @@ __device__ void vehicle_scan(const ObjDesc &o, float acc, float delta, const Reg
         float bs = fmaf(E.m00, beta, fmaf(E.m01, r, E.c0));
         float rs = fmaf(E.m10, beta, fmaf(E.m11, r, E.c1));
 
-        // 2. the lane's sub-steps in order: slip trig, heading increments, next accelerations
-        float sbv[CS], cbv[CS], dps[CS], axn[CS], ayn[CS];
+        // 2. the lane's sub-steps in order: slip trig, heading increments and their sum, next accelerations
         float ax_last = 0.0f, ay_last = 0.0f;             // the acceleration after the lane's last sub-step
-#pragma unroll
-        for (int c = 0; c < CS; ++c) {
-            sbv[c] = 0.0f; cbv[c] = 1.0f; dps[c] = 0.0f; axn[c] = 0.0f; ayn[c] = 0.0f;
-            if (c >= csa) continue;
+        float dh = 0.0f, dl = 0.0f;
+#pragma unroll 1
+        for (int c = 0; c < csa; ++c) {
             const int n = n0 + c;
-            const bool move = n < NK && n < g.n_stop;
-            const bool low = n >= g.low_lo && n < g.low_hi;
-            const float v = fmaf((float)n, dv, o.v0);
+            const bool move = n < NK && n < n_stop;
+            const bool low = n >= low_lo && n < low_hi;
+            const float v = fmaf((float)n, dv, v0);
             const float iv = __fdividef(1.0f, fmaxf(v, 1e-3f));
             const float bd_ot = fmaf(k11 * iv, bs, fmaf(fmaf(k12 * iv, iv, -1.0f), rs, kb1 * iv));
             const float rd_ot = fmaf(k21, bs, fmaf(k22 * iv, rs, kb2));
@@ -419,18 +460,20 @@ __device__ void vehicle_scan(const ObjDesc &o, float acc, float delta, const Reg
             const float rd = low ? 0.0f : rd_ot;
             float sb, cb;
             sincos_half(b_use, sb, cb);
-            sbv[c] = sb;
-            cbv[c] = cb;
             const float w = v * (bd + r_use);
-            axn[c] = fmaf(cb, acc, -sb * w);
-            ayn[c] = fmaf(sb, acc, cb * w);
-            dps[c] = move ? fmaf(r_use, ti, rd * hti2) : 0.0f;
+            const float dp = move ? fmaf(r_use, ti, rd * hti2) : 0.0f;
+            ax_last = fmaf(cb, acc, -sb * w);
+            ay_last = fmaf(sb, acc, cb * w);
+            slot.at(kSb, c, lane) = sb;
+            slot.at(kCb, c, lane) = cb;
+            slot.at(kDps, c, lane) = dp;
+            slot.at(kAx, c, lane) = ax_last;
+            slot.at(kAy, c, lane) = ay_last;
+            df_add(dh, dl, dp, 0.0f);
             if (move) {
                 bs = fmaf(bd, ti, b_use);
                 rs = fmaf(rd, ti, r_use);
             }
-            ax_last = axn[c];
-            ay_last = ayn[c];
         }
         // the next round starts from the state after every lane's maps
         {
@@ -443,9 +486,6 @@ __device__ void vehicle_scan(const ObjDesc &o, float acc, float delta, const Reg
         }
 
         // 3. heading at every sub-step start: lane sums, scanned
-        float dh = 0.0f, dl = 0.0f;
-#pragma unroll
-        for (int c = 0; c < CS; ++c) df_add(dh, dl, dps[c], 0.0f);
         float ih = dh, il = dl;
         df_scan(ih, il, lane);
         float hh = ph, hl = pl;                                       // heading at the lane's first sub-step
@@ -454,44 +494,41 @@ __device__ void vehicle_scan(const ObjDesc &o, float acc, float delta, const Reg
             if (lane > 0) df_add(hh, hl, eh, el);
         }
         const float th = __shfl_sync(0xffffffffu, ih, 31), tl = __shfl_sync(0xffffffffu, il, 31);
-        const float h_start = hh, l_start = hl;
 
         // 4. position increments
-        float ax_in = __shfl_up_sync(0xffffffffu, ax_last, 1), ay_in = __shfl_up_sync(0xffffffffu, ay_last, 1);
-        if (lane == 0) { ax_in = ax; ay_in = ay; }
-        float dxv[CS], dyv[CS];
+        float axu = __shfl_up_sync(0xffffffffu, ax_last, 1), ayu = __shfl_up_sync(0xffffffffu, ay_last, 1);
+        if (lane == 0) { axu = ax; ayu = ay; }
         float sxh = 0.0f, sxl = 0.0f, syh = 0.0f, syl = 0.0f;
         float sp, cp;                                  // heading trig: exact at the lane start, then rotated
         sincos2(hh, hl, sp, cp);
-#pragma unroll
-        for (int c = 0; c < CS; ++c) {
-            dxv[c] = dyv[c] = 0.0f;
-            if (c >= csa) continue;
+#pragma unroll 1
+        for (int c = 0; c < csa; ++c) {
             const int n = n0 + c;
-            const float cpb = fmaf(cp, cbv[c], -sp * sbv[c]);
-            const float spb = fmaf(sp, cbv[c], cp * sbv[c]);
-            const float axu = c ? axn[c - 1] : ax_in, ayu = c ? ayn[c - 1] : ay_in;
-            const float v = fmaf((float)n, dv, o.v0);
-            const bool stop_now = n == g.n_stop;
+            const float sb = slot.at(kSb, c, lane), cb = slot.at(kCb, c, lane), dp = slot.at(kDps, c, lane);
+            const float cpb = fmaf(cp, cb, -sp * sb);
+            const float spb = fmaf(sp, cb, cp * sb);
+            const float v = fmaf((float)n, dv, v0);
+            const bool stop_now = n == n_stop;
             const float d_stop = v * v * stop_den;
             float dx = stop_now ? cpb * d_stop : fmaf(cpb * v, ti, fmaf(cp, axu, -sp * ayu) * hti2);
             float dy = stop_now ? spb * d_stop : fmaf(spb * v, ti, fmaf(sp, axu, cp * ayu) * hti2);
-            if (n >= NK || n > g.n_stop) dx = dy = 0.0f;
-            dxv[c] = dx;
-            dyv[c] = dy;
+            if (n >= NK || n > n_stop) dx = dy = 0.0f;
+            slot.at(kDx, c, lane) = dx;
+            slot.at(kDy, c, lane) = dy;
             df_add(sxh, sxl, dx, 0.0f);
             df_add(syh, syl, dy, 0.0f);
-            if (dps[c] != 0.0f) {                      // rotate (cos, sin) of the heading by the increment
+            axu = slot.at(kAx, c, lane);
+            ayu = slot.at(kAy, c, lane);
+            if (dp != 0.0f) {                          // rotate (cos, sin) of the heading by the increment
                 float sd, cd;
-                sincos_tenth(dps[c], sd, cd);
+                sincos_tenth(dp, sd, cd);
                 const float c2 = fmaf(cp, cd, -sp * sd);
                 sp = fmaf(sp, cd, cp * sd);
                 cp = c2;
             }
         }
         float ixh = sxh, ixl = sxl, iyh = syh, iyl = syl;
-        df_scan(ixh, ixl, lane);
-        df_scan(iyh, iyl, lane);
+        df_scan2(ixh, ixl, iyh, iyl, lane);
 
         // 5. poses of the output steps ending in this lane's sub-steps
         float px = xh, pxl = xl, py = yh, pyl = yl;
@@ -503,24 +540,24 @@ __device__ void vehicle_scan(const ObjDesc &o, float acc, float delta, const Reg
                 df_add(py, pyl, fh, fl);
             }
         }
-        hh = h_start;
-        hl = l_start;
-#pragma unroll
-        for (int c = 0; c < CS; ++c) {
-            if (c >= csa) continue;
-            const int n = n0 + c;
-            df_add(px, pxl, dxv[c], 0.0f);
-            df_add(py, pyl, dyv[c], 0.0f);
-            df_add(hh, hl, dps[c], 0.0f);
-            if (n < NK && (n + 1) % K == 0) {                // the pose stores the exact heading trig
-                const int k = (n + 1) / K - 1;
-                float sp, cp;
-                sincos2(hh, hl, sp, cp);
-                const long long idx = base + (long long)k * h + i;
-                X[idx] = __fadd_rn(px, pxl);
-                Y[idx] = __fadd_rn(py, pyl);
-                C[idx] = cp;
-                S[idx] = sp;
+        int k = n0 / K, left = K - (n0 - k * K);       // the output step in progress, its sub-steps still to do
+#pragma unroll 1
+        for (int c = 0; c < csa; ++c) {
+            df_add(px, pxl, slot.at(kDx, c, lane), 0.0f);
+            df_add(py, pyl, slot.at(kDy, c, lane), 0.0f);
+            df_add(hh, hl, slot.at(kDps, c, lane), 0.0f);
+            if (--left == 0) {                               // the pose stores the exact heading trig
+                if (n0 + c < NK) {
+                    float so, co;
+                    sincos2(hh, hl, so, co);
+                    const long long idx = base + (long long)k * h + i;
+                    X[idx] = __fadd_rn(px, pxl);
+                    Y[idx] = __fadd_rn(py, pyl);
+                    C[idx] = co;
+                    S[idx] = so;
+                }
+                left = K;
+                ++k;
             }
         }
 
@@ -528,16 +565,14 @@ __device__ void vehicle_scan(const ObjDesc &o, float acc, float delta, const Reg
         df_add(ph, pl, th, tl);
         df_add(xh, xl, __shfl_sync(0xffffffffu, ixh, 31), __shfl_sync(0xffffffffu, ixl, 31));
         df_add(yh, yl, __shfl_sync(0xffffffffu, iyh, 31), __shfl_sync(0xffffffffu, iyl, 31));
-        ax = __shfl_sync(0xffffffffu, ax_last, 31);       // used only after a full round (csa = 8)
+        ax = __shfl_sync(0xffffffffu, ax_last, 31);       // used only after a full round (csa = 5)
         ay = __shfl_sync(0xffffffffu, ay_last, 31);
     }
 }
 
 // LAYOUTS: 1 every task is a warp per hypothesis, 2 every task is a thread per hypothesis, 3 both (a kernel
-// holding one layout only has a smaller instruction footprint: the integration is latency-bound and
-// instruction fetch was its largest stall).  Bounded to 80 registers (six CTAs per SM), where the
-// integration has no spills: faster than 64 (eight per SM, all of the 11-object scene's CTAs resident)
-// on the 11-object and 32-vehicle scenes.
+// holding one layout only has a smaller instruction footprint).  Bounded to 80 registers (six CTAs per SM), where the
+// integration has no spills.
 // table[0, n) = -1 by CTA b of nb (16-byte stores on the aligned body).
 __device__ __forceinline__ void fill_part(int16_t *table, long long n, long long b, long long nb) {
     const long long tid = b * blockDim.x + threadIdx.x, stride = nb * blockDim.x;
@@ -589,16 +624,29 @@ __global__ void __launch_bounds__(128, 6) gen_kernel(const GenArgs a) {
     const int w = bid * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (w >= a.n_warps) return;                          // whole warps leave
     if ((LAYOUTS & 1) && (LAYOUTS == 1 || w < a.n_scan)) {   // one hypothesis by the whole warp
+        __shared__ ScanSlot slots[4];
         const int lane = threadIdx.x & 31;
-        const int k = last_le(a.warp_first, a.n_scan_objs, w, lane);
-        const ObjDesc &o = a.objs[a.warp_obj[k]];
-        const int i = w - a.warp_first[k];
+        int first, obj;
+        if (a.n_scan_objs <= 32) {                       // one round of loads: entry `lane` and its object
+            const bool in = lane < a.n_scan_objs;
+            first = in ? a.warp_first[lane] : 0x7fffffff;
+            obj = in ? a.warp_obj[lane] : 0;
+            const int k = 31 - __clz(__ballot_sync(0xffffffffu, first <= w));
+            first = __shfl_sync(0xffffffffu, first, k);
+            obj = __shfl_sync(0xffffffffu, obj, k);
+        } else {
+            const int k = last_le(a.warp_first, a.n_scan_objs, w, lane);
+            first = a.warp_first[k];
+            obj = a.warp_obj[k];
+        }
+        const ObjDesc &o = a.objs[obj];
+        const int i = w - first;
         const int ia = i / o.n_b, ib = i - ia * o.n_b;
         const float ga = a.grids[o.grid_off + ia];
         const float gb = a.grids[o.grid_off + o.n_a + ib];
         if (o.kind == kVehicle)
             vehicle_scan(o, ga, gb, a.regimes[o.regime_off + ia], o.n_steps, o.substeps, lane, o.pose_base, o.h, i,
-                         a.x, a.y, a.c, a.s);
+                         a.x, a.y, a.c, a.s, slots[threadIdx.x >> 5]);
         else
             pedestrian(o, ga, gb, o.n_steps, o.tau, o.pose_base, o.h, i, a.x, a.y, a.c, a.s, lane, 32);
         return;
