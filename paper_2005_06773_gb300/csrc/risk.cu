@@ -15,6 +15,7 @@
 // instructions: each term (p_a p_b, p, -log(1 - p)) is formed in FP32 and added exactly as unsigned
 // 64-bit fixed point by integer atomics (exact, order-independent, bitwise reproducible).  FP64 -- a
 // narrow pipe on this GPU -- runs only in dense per-warp steps.
+#include "collide_common.cuh"
 #include "mhc_internal.cuh"
 #include "prepare.cuh"
 
@@ -190,29 +191,40 @@ __device__ void convert_pair_totals(const RiskArgs &a, long long t, long long nt
     }
 }
 
+// One element per thread and pass, the four kinds in one index space: their loads overlap.
 __device__ void convert_walk_totals(const RiskArgs &a, long long t, long long nt) {
-    for (long long q = t; q < a.n_obj; q += nt)
-        if (a.attr_obj) a.attr_obj[q] = from_fixed(a.acc.attr_obj[q], kFixProb);
-    for (long long q = t; q < a.n_steps_total; q += nt)
-        if (a.attr_step) a.attr_step[q] = from_fixed(a.acc.attr_step[q], kFixProb);
-    for (long long q = t; q < 4LL * a.n_scen; q += nt)
-        if (a.scalars) a.scalars[q] = (q & 3) < 3 ? a.acc.scalars[q] : 0.0;
-    for (long long q = t; q < a.n_scen; q += nt)
-        if (a.n_escape) a.n_escape[q] = (int)a.acc.n_escape[q];
+    const long long b1 = a.n_obj, b2 = b1 + a.n_steps_total, b3 = b2 + 4LL * a.n_scen, n = b3 + a.n_scen;
+    for (long long q = t; q < n; q += nt) {
+        if (q < b2) {
+            const unsigned long long v = q < b1 ? a.acc.attr_obj[q] : a.acc.attr_step[q - b1];
+            double *out = q < b1 ? a.attr_obj : a.attr_step;
+            if (out) out[q < b1 ? q : q - b1] = from_fixed(v, kFixProb);
+        } else if (q < b3) {
+            if (a.scalars) a.scalars[q - b2] = ((q - b2) & 3) < 3 ? a.acc.scalars[q - b2] : 0.0;
+        } else {
+            if (a.n_escape) a.n_escape[q - b3] = (int)a.acc.n_escape[q - b3];
+        }
+    }
 }
 
 // One warp per EGO hypothesis of the batch (its scenario found by binary search).
 //  * collision-free hypothesis: its escape-route rank (Section VI-A) = the number of collision-free
 //    hypotheses of its scenario more probable than it, ties by index, counted 32 at a time with ballots on
 //    integer keys (probabilities are non-negative, so their bit patterns order like the values);
-//  * otherwise the chronological walk: the (step, object) cells are read in ascending order 32 at a time,
-//    384 per group with the twelve loads in flight together; a warp prefix sum of the cells' fixed-point
-//    log-survival sums L (exact 64-bit integers) gives each cell the survival S = exp(-sum of the earlier
-//    cells' L), and the cell contributes S q with q = 1 - exp(-L) (Eq. p21 over the cell's collisions:
+//  * otherwise the chronological walk: the (step, object) cells are copied to shared memory 384 at a time and the
+//    non-empty ones (a tenth of them on the 11-object scene) moved together in ascending order; a warp prefix sum of
+//    their fixed-point log-survival sums L (exact 64-bit integers) gives each cell the survival S = exp(-sum of the
+//    earlier cells' L), and the cell contributes S q with q = 1 - exp(-L) (Eq. p21 over the cell's collisions:
 //    the product of their survival factors is exp(-L)).  Every term is formed in FP32 (relative error
 //    below 5e-7) and the terms are summed in FP64.
+// The attribution per object and step goes out with atomics, or (IN_PLACE, scenes of many cells) each term replaces
+// its cell's sum, for attribution_kernel to add up: 2,048 hypotheses with 1,600 cells each spent 180 us of 215 in
+// atomics on 82 addresses.
 // Every CTA first converts a slice of the pair totals; the last CTA to finish converts the walk's own
 // totals (or a separate grid-wide kernel does, for large batches).
+// Bound by latency: a chain of loads (hits, masses and cells), the walk, a fence and the last CTA's conversion.  The
+// loops stay rolled: each warp runs them about once, and fetching the unrolled code was most of a short walk (40 cells:
+// 3.5 us).
 constexpr float kLogScale = 1.0f / 1099511627776.0f;   // 2^-40: the fixed point of the log-survival sums
 
 // exp(-x 2^-40) for a fixed-point log-survival sum x: x = hi + lo with hi the nearest FP32 value (exact
@@ -223,14 +235,18 @@ __device__ __forceinline__ float survival(unsigned long long x) {
     return expf(-hi * kLogScale) * (1.0f - (float)lo * kLogScale);
 }
 
+constexpr int kEgoWarps = 2;
 constexpr int kEscapeBatch = 8;    // escape ranking: 256 EGO hypotheses' keys in flight per round
-constexpr int kWalkBatch = 12;     // chronological walk: 384 cells in flight per round
+constexpr int kWalkCells = 384;    // chronological walk: cells copied at once
 
-__global__ void __launch_bounds__(64) ego_kernel(const RiskArgs a) {
+template <bool IN_PLACE>
+__global__ void __launch_bounds__(32 * kEgoWarps) ego_kernel(const RiskArgs a) {
     pdl_trigger();
+    __shared__ unsigned long long s_cells[kEgoWarps][kWalkCells];
+    __shared__ unsigned short s_index[kEgoWarps][kWalkCells];
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31;
-    const long long g = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const long long g = (long long)blockIdx.x * kEgoWarps + (threadIdx.x >> 5);
     // the scenario of EGO hypothesis g and its descriptor: uploaded data, read before the wait
     int lo = 0;
     ScenDesc sd{};
@@ -243,13 +259,18 @@ __global__ void __launch_bounds__(64) ego_kernel(const RiskArgs a) {
         sd = a.scens[lo];
     }
     pdl_wait();
+    const long long i = g - sd.e_base;
+    unsigned long long hits = 0;
+    double pe = 0.0;
+    float pef = 0.0f;
+    if (g < a.h_e) {                       // in flight while the pair totals are converted
+        hits = a.acc.hits[g];
+        pe = a.prob[sd.e_traj + i];
+        pef = a.probf[sd.e_traj + i];
+    }
     convert_pair_totals(a, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
     if (g < a.h_e) {
         const int N = sd.n_steps, n_obj = sd.n_obj;
-        const long long i = g - sd.e_base;
-        const double pe = a.prob[sd.e_traj + i];
-        const float pef = a.probf[sd.e_traj + i];
-        const unsigned long long hits = a.acc.hits[g];
         double naive = 0.0, cond = 0.0, indep = 0.0;
         if (!hits) {
             if (a.escape) {
@@ -275,37 +296,47 @@ __global__ void __launch_bounds__(64) ego_kernel(const RiskArgs a) {
             }
             if (lane == 0) atomicAdd(a.acc.n_escape + lo, 1ull);
         } else {
-            // per-object masses: naive sum and independence product
-            double surv = 1.0, mass_sum = 0.0;
-            const unsigned long long *ms = a.acc.mass + sd.mass_base + i * n_obj;
-            for (int b = lane; b < n_obj; b += 32) {
-                const double m = from_fixed(ms[b], kFixProb);
-                mass_sum += m;
-                surv *= 1.0 - m;
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) surv *= __shfl_xor_sync(0xffffffffu, surv, d);
-            naive = warp_sum(mass_sum);
-            indep = 1.0 - surv;
-            // chronological walk over the cells, kWalkBatch chunks of 32 loaded at once.  A cell holds
-            // L = sum of -log(1 - p) of its collisions in fixed point, so the survival of every earlier cell
-            // is exp(-(exact integer prefix sum of L)) and the cell's own collision probability is
-            // 1 - exp(-L): the chunks' scans are 64-bit integer additions, independent of each other but
-            // for the carried total
-            const unsigned long long *lc = a.acc.lsum + sd.lsum_base + i * N * n_obj;
+            unsigned long long *cell = s_cells[threadIdx.x >> 5];
+            unsigned short *index = s_index[threadIdx.x >> 5];
+            unsigned long long *lc = a.acc.lsum + sd.lsum_base + i * N * n_obj;
             const long long cells = (long long)N * n_obj;
+            // per-object masses: naive sum and independence product
+            double surv = 1.0, mass_sum = 0.0, part = 0.0;
+            const unsigned long long *ms = a.acc.mass + sd.mass_base + i * n_obj;
             unsigned long long carry = 0;     // L summed over every cell before the chunk
-            double part = 0.0;
-            for (long long g0 = 0; g0 < cells; g0 += 32 * kWalkBatch) {
-                unsigned long long lv[kWalkBatch];
-#pragma unroll
-                for (int u = 0; u < kWalkBatch; ++u) {
-                    const long long c = g0 + 32 * u + lane;
-                    lv[u] = c < cells ? lc[c] : 0ull;
+            for (long long g0 = 0; g0 < cells; g0 += kWalkCells) {
+                const int n = (int)min((long long)kWalkCells, cells - g0);
+                __syncwarp();
+#pragma unroll 1
+                for (int c = lane; c < n; c += 32) cp_async8(cell + c, lc + g0 + c);
+                if (g0 == 0) {                // meanwhile
+                    for (int b = lane; b < n_obj; b += 32) {
+                        const double m = from_fixed(ms[b], kFixProb);
+                        mass_sum += m;
+                        surv *= 1.0 - m;
+                    }
                 }
-#pragma unroll
-                for (int u = 0; u < kWalkBatch; ++u) {
-                    const unsigned long long lf = lv[u];
+                cp_async_wait();
+                __syncwarp();
+                int filled = 0;               // the non-empty cells, moved together
+#pragma unroll 1
+                for (int c0 = 0; c0 < n; c0 += 32) {
+                    const unsigned long long v = c0 + lane < n ? cell[c0 + lane] : 0ull;
+                    const unsigned m = __ballot_sync(0xffffffffu, v != 0ull);
+                    if (!m) continue;
+                    const int at = filled + __popc(m & ((1u << lane) - 1u));   // at <= c0 + lane: read already
+                    __syncwarp();
+                    if (v) {
+                        cell[at] = v;
+                        index[at] = (unsigned short)(c0 + lane);
+                    }
+                    filled += __popc(m);
+                }
+                __syncwarp();
+#pragma unroll 1
+                for (int c0 = 0; c0 < filled; c0 += 32) {
+                    const bool full = c0 + lane < filled;
+                    const unsigned long long lf = full ? cell[c0 + lane] : 0ull;
                     unsigned long long incl = lf;
 #pragma unroll
                     for (int d = 1; d < 32; d <<= 1) {
@@ -314,27 +345,37 @@ __global__ void __launch_bounds__(64) ego_kernel(const RiskArgs a) {
                     }
                     const unsigned long long before = carry + (incl - lf);
                     carry += __shfl_sync(0xffffffffu, incl, 31);
-                    if (!lf) continue;                                    // an empty cell adds nothing
-                    const long long c = g0 + 32 * u + lane;
+                    if (!full) continue;
+                    const long long c = g0 + index[c0 + lane];
                     const float eff = survival(before) * -expm1f(-(float)lf * kLogScale);
                     part += (double)eff;
-                    const int k = (int)(c / n_obj), b = (int)(c - (long long)k * n_obj);
                     const unsigned long long w = to_fixed(pef * eff, kFixProb);
-                    atomicAdd(a.acc.attr_obj + sd.obj0 + b, w);
-                    atomicAdd(a.acc.attr_step + sd.step_base + k, w);
+                    if (IN_PLACE) {
+                        lc[c] = w;
+                    } else {
+                        const int k = (int)(c / n_obj), b = (int)(c - (long long)k * n_obj);
+                        atomicAdd(a.acc.attr_obj + sd.obj0 + b, w);
+                        atomicAdd(a.acc.attr_step + sd.step_base + k, w);
+                    }
                 }
             }
-            cond = warp_sum(part);
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) {
+                surv *= __shfl_xor_sync(0xffffffffu, surv, d);
+                mass_sum += __shfl_xor_sync(0xffffffffu, mass_sum, d);
+                part += __shfl_xor_sync(0xffffffffu, part, d);
+            }
+            naive = mass_sum;
+            indep = 1.0 - surv;
+            cond = part;
         }
-        if (lane == 0) {
-            if (a.naive) a.naive[g] = naive;
-            if (a.cond) a.cond[g] = cond;
-            if (a.indep) a.indep[g] = indep;
-            if (a.hits) a.hits[g] = (int)hits;
-            if (naive != 0.0) atomicAdd(a.acc.scalars + 4 * lo + 0, pe * naive);
-            if (cond != 0.0) atomicAdd(a.acc.scalars + 4 * lo + 1, pe * cond);
-            if (indep != 0.0) atomicAdd(a.acc.scalars + 4 * lo + 2, pe * indep);
+        if (lane < 3) {
+            const double v = lane == 0 ? naive : (lane == 1 ? cond : indep);
+            double *out = lane == 0 ? a.naive : (lane == 1 ? a.cond : a.indep);
+            if (out) out[g] = v;
+            if (v != 0.0) atomicAdd(a.acc.scalars + 4 * lo + lane, pe * v);
         }
+        if (lane == 3 && a.hits) a.hits[g] = (int)hits;
     }
     if (!a.convert_in_walk) return;
     // the last CTA converts the totals once every CTA's atomics are visible
@@ -345,6 +386,52 @@ __global__ void __launch_bounds__(64) ego_kernel(const RiskArgs a) {
     if (s_last) {
         __threadfence();
         convert_walk_totals(a, threadIdx.x, blockDim.x);
+    }
+}
+
+// The attribution sums of scenes with many cells, from the terms the walk left in them: CTA b takes kAttrHyps EGO
+// hypotheses of scenario b mod n_scen (cells read coalesced, a thread per cell), adds the cells up per object and per
+// step in shared memory and then into the totals: two atomics per object and step of a CTA instead of two per cell.
+// Cells the walk did not write are zero (a collision-free hypothesis's, or empty).  HBM-bound: it reads the cells once.
+constexpr int kAttrHyps = 16;
+constexpr int kAttrCells = 2048;
+
+__global__ void __launch_bounds__(256) attribution_kernel(const RiskArgs a) {
+    pdl_trigger();
+    __shared__ unsigned long long s_sum[kAttrCells];
+    const int s = (int)(blockIdx.x % a.n_scen);
+    const ScenDesc sd = a.scens[s];        // uploaded data: before the wait
+    const long long i0 = (long long)(blockIdx.x / a.n_scen) * kAttrHyps;
+    pdl_wait();
+    if (i0 >= sd.h_e) return;
+    const int hyps = (int)min((long long)kAttrHyps, sd.h_e - i0), n_obj = sd.n_obj;
+    const long long cells = (long long)sd.n_steps * n_obj;
+    const unsigned long long *term = a.acc.lsum + sd.lsum_base + i0 * cells;
+    for (long long c0 = 0; c0 < cells; c0 += kAttrCells) {
+        const int n = (int)min((long long)kAttrCells, cells - c0);
+        for (int c = threadIdx.x; c < n; c += blockDim.x) {
+            unsigned long long sum = 0;
+#pragma unroll
+            for (int u = 0; u < kAttrHyps; ++u)
+                if (u < hyps) sum += term[u * cells + c0 + c];
+            s_sum[c] = sum;
+        }
+        __syncthreads();
+        const int k0 = (int)(c0 / n_obj), k1 = (int)((c0 + n - 1) / n_obj);   // the window's steps
+        for (int q = threadIdx.x; q < n_obj + (k1 - k0 + 1); q += blockDim.x) {
+            unsigned long long sum = 0;
+            if (q < n_obj) {               // object q: every n_obj-th cell
+                int c = (int)((q - c0 % n_obj + n_obj) % n_obj);
+                for (; c < n; c += n_obj) sum += s_sum[c];
+                if (sum) atomicAdd(a.acc.attr_obj + sd.obj0 + q, sum);
+            } else {                       // step k: n_obj consecutive cells
+                const long long k = k0 + (q - n_obj);
+                const int c1 = (int)min((long long)n, (k + 1) * n_obj - c0);
+                for (int c = (int)max(0LL, k * n_obj - c0); c < c1; ++c) sum += s_sum[c];
+                if (sum) atomicAdd(a.acc.attr_step + sd.step_base + k, sum);
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -373,18 +460,36 @@ cudaError_t launch_risk_prepare(const RiskArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// From this many cells (EGO hypotheses x steps x objects) the attribution is summed by its own kernel: the 11-object
+// scene's 146 K cells take a launch less with atomics.
+constexpr long long kAttrInPlace = 1LL << 19;
+
+namespace {
+bool attribution_alone(const RiskArgs &a) { return a.h_e > 0 && a.n_cells >= kAttrInPlace; }
+}  // namespace
+
 int risk_tail_launches(const RiskArgs &a) {
-    return (a.h_e > 0 ? 1 : 0) + (a.h_e > 0 && convert_elements(a) <= kConvertInWalk ? 0 : 1);
+    const bool alone = attribution_alone(a);
+    return (a.h_e > 0 ? 1 : 0) + (alone ? 1 : 0) + (a.h_e > 0 && !alone && convert_elements(a) <= kConvertInWalk ? 0 : 1);
 }
 
 cudaError_t launch_risk_tail(const RiskArgs &args, cudaStream_t st, bool pdl) {
     RiskArgs a = args;
     const long long conv = convert_elements(a);
-    a.convert_in_walk = a.h_e > 0 && conv <= kConvertInWalk;
+    const bool alone = attribution_alone(a);
+    a.convert_in_walk = a.h_e > 0 && !alone && conv <= kConvertInWalk;
     if (a.h_e > 0) {
-        cudaError_t e = launch_kernel(ego_kernel, dim3((unsigned)((a.h_e + 1) / 2)), dim3(64), 0, st, pdl, a);
+        const dim3 grid((unsigned)((a.h_e + kEgoWarps - 1) / kEgoWarps)), block(32 * kEgoWarps);
+        cudaError_t e = alone ? launch_kernel(ego_kernel<true>, grid, block, 0, st, pdl, a)
+                              : launch_kernel(ego_kernel<false>, grid, block, 0, st, pdl, a);
         if (e != cudaSuccess) return e;
         pdl = true;
+        if (alone) {
+            const long long ctas = (a.max_h_e + kAttrHyps - 1) / kAttrHyps * a.n_scen;
+            if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
+            e = launch_kernel(attribution_kernel, dim3((unsigned)ctas), dim3(256), 0, st, true, a);
+            if (e != cudaSuccess) return e;
+        }
     }
     if (!a.convert_in_walk) {
         long long blocks = (conv + 255) / 256;
