@@ -340,7 +340,9 @@ struct RiskArgs {
     long long max_h_e, n_cells;    // the most of one scenario; cells [EGO hypothesis][step][object] in all
     long long n_kofs, n_steps_total;   // per-pair step entries, per-scenario step entries
     int max_steps;                 // the longest horizon of the batch
-    int convert_in_walk;           // set by launch_risk_tail: the EGO walk's last CTA converts the totals
+    int convert_in_walk;           // set by launch_risk_tail: the last CTA of the EGO walk (1) or of the attribution (2)
+                                   // converts the totals
+    long long walk_ctas;           // set by launch_risk_tail: CTAs of the EGO walk, before those of the pair totals
     long long n_tiles;
     const int16_t *table;
     const float *weights;          // [n_traj] raw non-negative weights, or null for uniform (or scored)

@@ -211,17 +211,17 @@ __device__ void convert_walk_totals(const RiskArgs &a, long long t, long long nt
 //  * collision-free hypothesis: its escape-route rank (Section VI-A) = the number of collision-free
 //    hypotheses of its scenario more probable than it, ties by index, counted 32 at a time with ballots on
 //    integer keys (probabilities are non-negative, so their bit patterns order like the values);
-//  * otherwise the chronological walk: the (step, object) cells are copied to shared memory 384 at a time and the
-//    non-empty ones (a tenth of them on the 11-object scene) moved together in ascending order; a warp prefix sum of
-//    their fixed-point log-survival sums L (exact 64-bit integers) gives each cell the survival S = exp(-sum of the
+//  * otherwise the chronological walk: the (step, object) cells are copied to shared memory 416 at a time and the
+//    non-empty ones moved together in ascending order, each with the prefix sum of the earlier cells' fixed-point
+//    log-survival sums L (exact 64-bit integers), which gives it the survival S = exp(-sum of the
 //    earlier cells' L), and the cell contributes S q with q = 1 - exp(-L) (Eq. p21 over the cell's collisions:
 //    the product of their survival factors is exp(-L)).  Every term is formed in FP32 (relative error
 //    below 5e-7) and the terms are summed in FP64.
 // The attribution per object and step goes out with atomics, or (IN_PLACE, scenes of many cells) each term replaces
 // its cell's sum, for attribution_kernel to add up: 2,048 hypotheses with 1,600 cells each spent 180 us of 215 in
 // atomics on 82 addresses.
-// Every CTA first converts a slice of the pair totals; the last CTA to finish converts the walk's own
-// totals (or a separate grid-wide kernel does, for large batches).
+// The CTAs past the walk's convert the pair totals (within the walk's CTAs it held up the first of them by 1 us); the
+// last CTA to finish converts the walk's own totals (or a later kernel does, for large batches).
 // Bound by latency: a chain of loads (hits, masses and cells), the walk, a fence and the last CTA's conversion.  The
 // loops stay rolled: each warp runs them about once, and fetching the unrolled code was most of a short walk (40 cells:
 // 3.5 us).
@@ -237,14 +237,27 @@ __device__ __forceinline__ float survival(unsigned long long x) {
 
 constexpr int kEgoWarps = 2;
 constexpr int kEscapeBatch = 8;    // escape ranking: 256 EGO hypotheses' keys in flight per round
-constexpr int kWalkCells = 384;    // chronological walk: cells copied at once
+constexpr int kWalkCells = 416;    // chronological walk: cells copied at once
+
+// The last CTA of the launch to come here converts the totals, once every CTA's atomics are visible.  Every thread of
+// every CTA calls it.
+__device__ __forceinline__ void finish_totals(const RiskArgs &a) {
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(a.acc.done, 1ull) == (unsigned long long)gridDim.x - 1;
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        convert_walk_totals(a, threadIdx.x, blockDim.x);
+    }
+}
 
 template <bool IN_PLACE>
 __global__ void __launch_bounds__(32 * kEgoWarps) ego_kernel(const RiskArgs a) {
     pdl_trigger();
-    __shared__ unsigned long long s_cells[kEgoWarps][kWalkCells];
+    __shared__ unsigned long long s_cells[kEgoWarps][kWalkCells], s_before[kEgoWarps][kWalkCells];
     __shared__ unsigned short s_index[kEgoWarps][kWalkCells];
-    __shared__ bool s_last;
     const int lane = threadIdx.x & 31;
     const long long g = (long long)blockIdx.x * kEgoWarps + (threadIdx.x >> 5);
     // the scenario of EGO hypothesis g and its descriptor: uploaded data, read before the wait
@@ -259,17 +272,14 @@ __global__ void __launch_bounds__(32 * kEgoWarps) ego_kernel(const RiskArgs a) {
         sd = a.scens[lo];
     }
     pdl_wait();
+    if (blockIdx.x >= a.walk_ctas)
+        convert_pair_totals(a, (long long)(blockIdx.x - a.walk_ctas) * blockDim.x + threadIdx.x,
+                            (long long)(gridDim.x - a.walk_ctas) * blockDim.x);
     const long long i = g - sd.e_base;
-    unsigned long long hits = 0;
-    double pe = 0.0;
-    float pef = 0.0f;
-    if (g < a.h_e) {                       // in flight while the pair totals are converted
-        hits = a.acc.hits[g];
-        pe = a.prob[sd.e_traj + i];
-        pef = a.probf[sd.e_traj + i];
-    }
-    convert_pair_totals(a, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
     if (g < a.h_e) {
+        const unsigned long long hits = a.acc.hits[g];
+        const double pe = a.prob[sd.e_traj + i];
+        const float pef = a.probf[sd.e_traj + i];
         const int N = sd.n_steps, n_obj = sd.n_obj;
         double naive = 0.0, cond = 0.0, indep = 0.0;
         if (!hits) {
@@ -297,6 +307,7 @@ __global__ void __launch_bounds__(32 * kEgoWarps) ego_kernel(const RiskArgs a) {
             if (lane == 0) atomicAdd(a.acc.n_escape + lo, 1ull);
         } else {
             unsigned long long *cell = s_cells[threadIdx.x >> 5];
+            unsigned long long *before = s_before[threadIdx.x >> 5];
             unsigned short *index = s_index[threadIdx.x >> 5];
             unsigned long long *lc = a.acc.lsum + sd.lsum_base + i * N * n_obj;
             const long long cells = (long long)N * n_obj;
@@ -318,44 +329,50 @@ __global__ void __launch_bounds__(32 * kEgoWarps) ego_kernel(const RiskArgs a) {
                 }
                 cp_async_wait();
                 __syncwarp();
-                int filled = 0;               // the non-empty cells, moved together
-#pragma unroll 1
-                for (int c0 = 0; c0 < n; c0 += 32) {
-                    const unsigned long long v = c0 + lane < n ? cell[c0 + lane] : 0ull;
-                    const unsigned m = __ballot_sync(0xffffffffu, v != 0ull);
-                    if (!m) continue;
-                    const int at = filled + __popc(m & ((1u << lane) - 1u));   // at <= c0 + lane: read already
-                    __syncwarp();
-                    if (v) {
-                        cell[at] = v;
-                        index[at] = (unsigned short)(c0 + lane);
-                    }
-                    filled += __popc(m);
+                // the lane's share of the window in ascending order (an odd number: no bank conflicts): its non-empty
+                // cells and their sum, then both prefix sums, then the cells moved together with the sum before each
+                const int per = ((n + 31) >> 5) | 1, c0 = min(lane * per, n), c1 = min(c0 + per, n);
+                int count = 0;
+                unsigned long long sum = 0;
+                for (int c = c0; c < c1; ++c) {
+                    const unsigned long long v = cell[c];
+                    sum += v;
+                    count += v != 0ull;
+                }
+                int at = count;
+                unsigned long long incl = sum;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const unsigned long long v = __shfl_up_sync(0xffffffffu, incl, d);
+                    const int q = __shfl_up_sync(0xffffffffu, at, d);
+                    if (lane >= d) { incl += v; at += q; }
+                }
+                const int filled = __shfl_sync(0xffffffffu, at, 31);
+                unsigned long long earlier = carry + (incl - sum);
+                carry += __shfl_sync(0xffffffffu, incl, 31);
+                at -= count;
+                for (int c = c0; c < c1; ++c) {
+                    const unsigned long long v = cell[c];
+                    if (!v) continue;
+                    before[at] = earlier;
+                    index[at++] = (unsigned short)c;
+                    earlier += v;
                 }
                 __syncwarp();
+                const int k0 = (int)(g0 / n_obj), b0 = (int)(g0 - (long long)k0 * n_obj);
 #pragma unroll 1
-                for (int c0 = 0; c0 < filled; c0 += 32) {
-                    const bool full = c0 + lane < filled;
-                    const unsigned long long lf = full ? cell[c0 + lane] : 0ull;
-                    unsigned long long incl = lf;
-#pragma unroll
-                    for (int d = 1; d < 32; d <<= 1) {
-                        const unsigned long long v = __shfl_up_sync(0xffffffffu, incl, d);
-                        if (lane >= d) incl += v;
-                    }
-                    const unsigned long long before = carry + (incl - lf);
-                    carry += __shfl_sync(0xffffffffu, incl, 31);
-                    if (!full) continue;
-                    const long long c = g0 + index[c0 + lane];
-                    const float eff = survival(before) * -expm1f(-(float)lf * kLogScale);
+                for (int q = lane; q < filled; q += 32) {
+                    const int c = index[q];
+                    const unsigned long long lf = cell[c];
+                    const float eff = survival(before[q]) * -expm1f(-(float)lf * kLogScale);
                     part += (double)eff;
                     const unsigned long long w = to_fixed(pef * eff, kFixProb);
                     if (IN_PLACE) {
-                        lc[c] = w;
+                        lc[g0 + c] = w;
                     } else {
-                        const int k = (int)(c / n_obj), b = (int)(c - (long long)k * n_obj);
-                        atomicAdd(a.acc.attr_obj + sd.obj0 + b, w);
-                        atomicAdd(a.acc.attr_step + sd.step_base + k, w);
+                        const unsigned r = (unsigned)(b0 + c), k = r / (unsigned)n_obj;
+                        atomicAdd(a.acc.attr_obj + sd.obj0 + (r - k * (unsigned)n_obj), w);
+                        atomicAdd(a.acc.attr_step + sd.step_base + k0 + k, w);
                     }
                 }
             }
@@ -377,16 +394,7 @@ __global__ void __launch_bounds__(32 * kEgoWarps) ego_kernel(const RiskArgs a) {
         }
         if (lane == 3 && a.hits) a.hits[g] = (int)hits;
     }
-    if (!a.convert_in_walk) return;
-    // the last CTA converts the totals once every CTA's atomics are visible
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(a.acc.done, 1ull) == (unsigned long long)gridDim.x - 1;
-    __syncthreads();
-    if (s_last) {
-        __threadfence();
-        convert_walk_totals(a, threadIdx.x, blockDim.x);
-    }
+    if (a.convert_in_walk == 1) finish_totals(a);
 }
 
 // The attribution sums of scenes with many cells, from the terms the walk left in them: CTA b takes kAttrHyps EGO
@@ -403,9 +411,8 @@ __global__ void __launch_bounds__(256) attribution_kernel(const RiskArgs a) {
     const ScenDesc sd = a.scens[s];        // uploaded data: before the wait
     const long long i0 = (long long)(blockIdx.x / a.n_scen) * kAttrHyps;
     pdl_wait();
-    if (i0 >= sd.h_e) return;
-    const int hyps = (int)min((long long)kAttrHyps, sd.h_e - i0), n_obj = sd.n_obj;
-    const long long cells = (long long)sd.n_steps * n_obj;
+    const int hyps = (int)max(0LL, min((long long)kAttrHyps, sd.h_e - i0)), n_obj = sd.n_obj;
+    const long long cells = hyps ? (long long)sd.n_steps * n_obj : 0;
     const unsigned long long *term = a.acc.lsum + sd.lsum_base + i0 * cells;
     for (long long c0 = 0; c0 < cells; c0 += kAttrCells) {
         const int n = (int)min((long long)kAttrCells, cells - c0);
@@ -433,6 +440,7 @@ __global__ void __launch_bounds__(256) attribution_kernel(const RiskArgs a) {
         }
         __syncthreads();
     }
+    if (a.convert_in_walk == 2) finish_totals(a);
 }
 
 // The walk's totals of a large batch, grid-wide after the walk (and the pair totals too when there is no
@@ -470,16 +478,18 @@ bool attribution_alone(const RiskArgs &a) { return a.h_e > 0 && a.n_cells >= kAt
 
 int risk_tail_launches(const RiskArgs &a) {
     const bool alone = attribution_alone(a);
-    return (a.h_e > 0 ? 1 : 0) + (alone ? 1 : 0) + (a.h_e > 0 && !alone && convert_elements(a) <= kConvertInWalk ? 0 : 1);
+    return (a.h_e > 0 ? 1 : 0) + (alone ? 1 : 0) + (a.h_e > 0 && convert_elements(a) <= kConvertInWalk ? 0 : 1);
 }
 
 cudaError_t launch_risk_tail(const RiskArgs &args, cudaStream_t st, bool pdl) {
     RiskArgs a = args;
     const long long conv = convert_elements(a);
     const bool alone = attribution_alone(a);
-    a.convert_in_walk = a.h_e > 0 && !alone && conv <= kConvertInWalk;
+    a.convert_in_walk = a.h_e > 0 && conv <= kConvertInWalk ? (alone ? 2 : 1) : 0;
     if (a.h_e > 0) {
-        const dim3 grid((unsigned)((a.h_e + kEgoWarps - 1) / kEgoWarps)), block(32 * kEgoWarps);
+        a.walk_ctas = (a.h_e + kEgoWarps - 1) / kEgoWarps;
+        const long long pair_ctas = std::min((a.n_kofs + a.n_pairs + 128 * kEgoWarps - 1) / (128 * kEgoWarps), 152LL * 8);
+        const dim3 grid((unsigned)(a.walk_ctas + pair_ctas)), block(32 * kEgoWarps);
         cudaError_t e = alone ? launch_kernel(ego_kernel<true>, grid, block, 0, st, pdl, a)
                               : launch_kernel(ego_kernel<false>, grid, block, 0, st, pdl, a);
         if (e != cudaSuccess) return e;
