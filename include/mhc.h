@@ -201,11 +201,10 @@ void mhc_destroy(mhc_ctx *ctx);
  *                 6: every active (quarter tile, step) an item, all tested in parallel by persistent warps (a
  *                    pair's first step by atomicMin in scratch, the table and the risk terms written after);
  *                    for small scenes (at most 2^22 items and 2^26 table entries; larger ones use 5);
- *                 7: one 128-thread CTA per 32 x 32 quarter tile, its active steps spread over the four
- *                    warps (each in ascending order), first hits kept in shared memory and a candidate of a
- *                    pair that already hit at an earlier step dropped before its exact test; the CTA stores
- *                    the first hits and their risk terms (the table's -1s are written beforehand);
- *                 8: as 7 for the quarter tiles with an active step only, listed first by one warp per
+ *                 7: one CTA per 32 x 32 quarter tile with an active step, its active steps spread over the
+ *                    CTA's warps; tiles in tile order and listed first, as 4 (every quarter tile of ascending tiles
+ *                    without culling or without room for the list);
+ *                 8: as 7 in ascending tiles, the quarter tiles with an active step listed by one warp per
  *                    quarter tile (records in scratch; up to 2^19 quarter tiles, larger scenarios use 7);
  *                 0 (default): the one mhc_autotune chose for the scenario's size class, else 4 for at
  *                 least 32 tiles per SM, and 7 below that. */

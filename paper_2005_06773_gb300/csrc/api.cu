@@ -782,11 +782,11 @@ int launch_all(mhc_ctx *ctx, const Layout &L, const DevDesc &D, Bump &bump, cons
         float4 *bounds = static_cast<float4 *>(bump.take(sizeof(float4) * (size_t)L.n_bounds));
         if (!bounds) return fail(MHC_E_NOMEM, "arena too small for tile bounds");
         CollideArgs c{};
-        // poses in tile order for layout 4 (and the list of active blocks); without room for them (an
-        // arena sized to the least) or without culling, it takes the blocks of ascending tiles and reads the planes
+        // poses in tile order for layouts 4 and 7 (and the list of active blocks); without room for them (an
+        // arena sized to the least) or without culling, they take the blocks of ascending tiles and read the planes
         float4 *tile_poses = nullptr;
         int *tile_order = nullptr;
-        if (variant == 4 && cull && L.n_tiles > 0) {
+        if ((variant == 4 || variant == 7) && cull && L.n_tiles > 0) {
             tile_poses = static_cast<float4 *>(bump.take(sizeof(float4) * 32 * (size_t)L.n_bounds));
             if (tile_poses) tile_order = static_cast<int *>(bump.take(sizeof(int) * 32 * (size_t)L.n_tiles32));
             if (tile_order) {
@@ -854,7 +854,7 @@ int launch_all(mhc_ctx *ctx, const Layout &L, const DevDesc &D, Bump &bump, cons
             MHC_CUDA(cudaMemsetAsync(c.item_count, 0, 2 * sizeof(unsigned long long), st));
             after_kernel = false;
         }
-        TimedScope ts(ctx, st, MHC_K_COLLIDE, variant == 6 ? 3 : (variant == 8 || tile_poses ? 2 : 1));
+        TimedScope ts(ctx, st, MHC_K_COLLIDE, variant == 6 ? 3 : (variant == 8 ? 2 : (tile_poses ? tiles_launches(c) : 1)));
         cudaError_t e = launch_collide(c, st, pdl());
         if (e != cudaSuccess) return cuda_fail(e, "collision kernel launch");
         if (L.n_tiles > 0) after_kernel = true;

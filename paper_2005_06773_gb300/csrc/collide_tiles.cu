@@ -1,10 +1,10 @@
-// collide_tiles.cu -- collision layout 4: a warp per active 32 x 32 block of hypothesis pairs, in the objects' tile
-// order.
+// collide_tiles.cu -- collision layouts 4 and 7: a warp (4) or a CTA (7) per active 32 x 32 block of hypothesis pairs,
+// in the objects' tile order.
 //
 // The bounds kernel has written each object's poses tile by tile (CollideArgs::tile_poses: 32 poses of one step side
 // by side, in the compact order of hypothesis_at) together with the boxes around them, so that a block's active
 // steps are few and a step's poses are one 16-byte load per lane and side.  Without that array (culling off, or an
-// arena sized to the least) the same kernels take ascending tiles and read the pose planes.
+// arena sized to the least) layout 4's kernel takes ascending tiles and reads the pose planes.
 //
 // A step of a block, by one warp: the 32 + 32 poses go to a shared slot, the broad phase runs on a 4 x 8 micro-block
 // per lane (rows lr + 8 m, columns lc + 4 n), and the candidates are queued and tested one per lane.  Compact tiles
@@ -87,32 +87,6 @@ __device__ __forceinline__ bool boxes_meet(const float4 &a, const float4 &b, flo
     return (a.x - r <= b.z) && (b.x - r <= a.z) && (a.y - r <= b.w) && (b.y - r <= a.w);
 }
 
-// Active steps among k0 .. k0 + 31 of the four 32 x 32 blocks of a 64 x 64 tile (bit b of m[2 qa + qb]: step k0 + b;
-// qa / qb: the second 32 rows / columns), one ballot each.  box_a, box_b: the tile's first boxes.
-struct TileBoxes {
-    long long box_a, box_b;
-    int N;
-    bool two_a, two_b;                 // the tile has a second 32 rows / columns
-    float r_cull;
-};
-
-__device__ __forceinline__ void active_steps(const CollideArgs &a, const TileBoxes &T, int k0, int lane, unsigned m[4]) {
-    const int k = k0 + lane;
-    bool m00 = k < T.N, m01 = m00 && T.two_b, m10 = m00 && T.two_a, m11 = m01 && T.two_a;
-    if (a.cull && m00) {
-        const float4 a0 = a.bounds[T.box_a + k], b0 = a.bounds[T.box_b + k];
-        const float4 a1 = T.two_a ? a.bounds[T.box_a + T.N + k] : a0, b1 = T.two_b ? a.bounds[T.box_b + T.N + k] : b0;
-        m00 = boxes_meet(a0, b0, T.r_cull);
-        m01 = m01 && boxes_meet(a0, b1, T.r_cull);
-        m10 = m10 && boxes_meet(a1, b0, T.r_cull);
-        m11 = m11 && boxes_meet(a1, b1, T.r_cull);
-    }
-    m[0] = __ballot_sync(0xffffffffu, m00);
-    m[1] = __ballot_sync(0xffffffffu, m01);
-    m[2] = __ballot_sync(0xffffffffu, m10);
-    m[3] = __ballot_sync(0xffffffffu, m11);
-}
-
 // Sum of v over the warp (v <= 2^62, and the sum too): three 32-bit reductions.
 __device__ __forceinline__ unsigned long long reduce_terms(unsigned long long v) {
     const unsigned m0 = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xffffffu);
@@ -142,24 +116,43 @@ __global__ void __launch_bounds__(32 * kListWarps) block_list_kernel(const Colli
     if (g0 < a.n_tiles) pair = pair_of_tile(a, g0);   // uploaded data: before the wait
     pdl_wait();
     const int mine = lane >> 2, q = lane & 3;
-    for (int u = 0; u < per_warp && g0 + u < a.n_tiles; ++u) {
-        const long long g = g0 + u;
-        while (pair + 1 < a.n_pairs && a.pairs[pair + 1].tile_start <= g) ++pair;
+    for (int u0 = 0; u0 < per_warp && g0 + u0 < a.n_tiles;) {
+        while (pair + 1 < a.n_pairs && a.pairs[pair + 1].tile_start <= g0 + u0) ++pair;
         const PairDesc &P = a.pairs[pair];
-        const int t = (int)(g - P.tile_start);      // < tiles_a x tiles_b <= n_tiles < 2^31
-        const int ta = t / P.tiles_b, tb = t - ta * P.tiles_b, N = P.n_steps;
-        const TileBoxes T{P.bounds_a + (long long)(2 * ta) * N, P.bounds_b + (long long)(2 * tb) * N, N,
-                          ta * kTile + 32 < P.h_a, tb * kTile + 32 < P.h_b, P.r_cull};
-        if (mine == u) {
+        const int t = (int)(g0 + u0 - P.tile_start);   // < tiles_a x tiles_b <= n_tiles < 2^31
+        const int ta = t / P.tiles_b, tb = t - ta * P.tiles_b, N = P.n_steps, hb = P.h_b;
+        const int run = min(per_warp - u0, P.tiles_b - tb);   // tiles of the same rows: their boxes are loaded once
+        const long long box_a = P.bounds_a + (long long)(2 * ta) * N, box_b = P.bounds_b + (long long)(2 * tb) * N;
+        const bool two_a = ta * kTile + 32 < P.h_a;
+        const float r = P.r_cull;
+        if (mine - u0 >= 0 && mine - u0 < run) {
             ref.pair = pair;
             ref.tile_a = 2 * ta + (q >> 1);
-            ref.tile_b = 2 * tb + (q & 1);
+            ref.tile_b = 2 * (tb + mine - u0) + (q & 1);
+            ref.box_a = (int)(box_a + (q >> 1) * N);
+            ref.box_b = (int)(box_b + (2 * (mine - u0) + (q & 1)) * N);
         }
         for (int k0 = 0; k0 < N; k0 += 32) {
-            unsigned m[4];
-            active_steps(a, T, k0, lane, m);
-            if (mine == u) n += __popc(q < 2 ? (q ? m[1] : m[0]) : (q == 2 ? m[2] : m[3]));
+            const int k = k0 + lane;
+            const bool in = k < N;
+            const float4 far = make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY);   // meets nothing
+            const float4 a0 = in ? a.bounds[box_a + k] : far, a1 = in && two_a ? a.bounds[box_a + N + k] : far;
+            for (int v = 0; v < run; ++v) {
+                const long long bb = box_b + (long long)(2 * v) * N;
+                const bool two_b = (tb + v) * kTile + 32 < hb;
+                const float4 b0 = in ? a.bounds[bb + k] : far, b1 = in && two_b ? a.bounds[bb + N + k] : far;
+                const unsigned m0 = __ballot_sync(0xffffffffu, boxes_meet(a0, b0, r));
+                const unsigned m1 = __ballot_sync(0xffffffffu, boxes_meet(a0, b1, r));
+                const unsigned m2 = __ballot_sync(0xffffffffu, boxes_meet(a1, b0, r));
+                const unsigned m3 = __ballot_sync(0xffffffffu, boxes_meet(a1, b1, r));
+                if (mine == u0 + v) {
+                    const unsigned m = q < 2 ? (q ? m1 : m0) : (q == 2 ? m2 : m3);
+                    if (n == 0) { ref.k0 = k0; ref.mask = m; }
+                    n += __popc(m);
+                }
+            }
         }
+        u0 += run;
     }
     const unsigned active = __ballot_sync(0xffffffffu, n > 0), heavy = __ballot_sync(0xffffffffu, n >= kHeavySteps);
     const unsigned light = active & ~heavy, lt = (1u << lane) - 1u;
@@ -215,7 +208,8 @@ __device__ __forceinline__ void walk_block(const CollideArgs &a, const BlockRef 
     const PairDesc &P = a.pairs[B.pair];               // fields read where used (fewer live registers)
     const int ha = P.h_a, hb = P.h_b, N = P.n_steps;
     const int ia = 32 * B.tile_a + lane, jb = 32 * B.tile_b + lane;   // this lane's positions
-    const long long box_a = P.bounds_a + (long long)B.tile_a * N, box_b = P.bounds_b + (long long)B.tile_b * N;
+    const long long box_a = UNLISTED ? P.bounds_a + (long long)B.tile_a * N : B.box_a;
+    const long long box_b = UNLISTED ? P.bounds_b + (long long)B.tile_b * N : B.box_b;
     const float r_cull = P.r_cull;
     auto chunk = [&](int k0) -> unsigned {             // active steps among k0 .. k0 + 31
         const int k = k0 + lane;
@@ -223,8 +217,8 @@ __device__ __forceinline__ void walk_block(const CollideArgs &a, const BlockRef 
         if (act && (!UNLISTED || a.cull)) act = boxes_meet(a.bounds[box_a + k], a.bounds[box_b + k], r_cull);
         return __ballot_sync(0xffffffffu, act);
     };
-    int k0 = 0;
-    unsigned mask = chunk(0);
+    int k0 = UNLISTED ? 0 : B.k0;
+    unsigned mask = UNLISTED ? chunk(0) : B.mask;
     auto next = [&]() -> int {
         while (!mask) {
             k0 += 32;
@@ -355,19 +349,324 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkCtas) walk_kernel(const 
     }
 }
 
+// ---- layout 7: a CTA per active 32 x 32 block, its active steps spread over its warps ------------------------
+//
+// A scene of few tiles waits for its heaviest blocks, so a block gets a whole CTA.  It takes the block's active steps
+// W at a time, one per warp: every warp stages its step's poses, sweeps the 32 x 32 pairs and puts its candidates
+// into the CTA's queue; after a barrier all warps test the queue, 32 candidates a round.  A pair that overlapped in
+// an earlier batch is dropped at the sweep (`found`: the batches ascend in time), two hits of one batch keep the
+// earlier step (atomicMin).  At the end the CTA stores the first hits and adds their fused risk terms.
+//
+// Bound by latency: a batch of W steps is a chain of 2,300 cycles, the heaviest block has four, and a block's set-up
+// and epilogue take as long as two more.  Measured (whole call replayed as one graph; before: a CTA of four warps per
+// 32 consecutive hypotheses a side, listed or not, a queue per warp): EGO-only scene 154 -> 101 us, 11 objects with
+// outlines 153 -> 133, with lane paths 150 -> 137, 11 objects 46.5 -> 46.8.  Four warps a CTA: 11 objects 53.6, outlines
+// 178; sixteen: 51.3 and 135; four CTAs per SM: 49.5 and 158; the light blocks by a warp each: 50.7 and 140; in
+// arbitrary order: 52.5 and 140.
+constexpr int kBlockWarps = 8;
+constexpr int kBlockCtas = 3;           // per SM: bounds the registers to 80
+constexpr int kBlockSlots = 152 * kBlockCtas;   // CTAs on the chip at once
+constexpr int kLaneQueue = 32;          // candidates queued per lane and round
+
+// queue_offsets for counts up to 63.
+__device__ __forceinline__ bool queue_offsets6(int cnt, int lane, int &off, int &total) {
+    if (!__any_sync(0xffffffffu, cnt > 15)) return queue_offsets(cnt, lane, off, total);
+    const unsigned lt = (1u << lane) - 1u;
+    off = total = 0;
+#pragma unroll
+    for (int b = 0; b < 6; ++b) {
+        const unsigned m = __ballot_sync(0xffffffffu, cnt >> b & 1);
+        off += __popc(m & lt) << b;
+        total += __popc(m) << b;
+    }
+    return true;
+}
+
+constexpr int kHitsPerStep = 16;        // hits per step of a warp's lines from which its terms are summed step by step
+constexpr int kFirstRow = 33;           // (odd: columns read without bank conflicts)
+
+struct BlockSlot {
+    StepSlot step[kBlockWarps];
+    unsigned short queue[kBlockWarps * kLaneQueue * 32];   // step slot << 10 | candidate
+    int at[kBlockWarps];                // the slots' steps
+    int queued[2];                      // candidates in the queue (of alternate rounds)
+    int first[32 * kFirstRow];          // first overlapping step of pair (i, j) at kFirstRow i + j
+    unsigned found[32];                 // [lane] micro-block pairs that overlapped in an earlier batch
+    int order[2][32];                   // hypotheses of the rows and columns
+    float prob[2][32];                  // fused: their probabilities
+    unsigned long long lfix[32], pfix[32];   // fused EGO pair: the CO side's fixed-point terms
+};
+
+// (mask 0: the block's active steps are not known yet, from step 0 on)
+template <bool FUSED, bool OUTL>
+__device__ __forceinline__ void block_work(const CollideArgs &a, const BlockRef &B, BlockSlot &S) {
+    constexpr int W = kBlockWarps, ROWS = 32 / W;
+    constexpr int kNone = 0x7fffffff;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, tid = threadIdx.x;
+    const PairDesc &P = a.pairs[B.pair];
+    const long long box_a = B.box_a, box_b = B.box_b;
+    StepPoses cur{};
+    auto load = [&](int k) {
+        cur.a = load_pose<true>(a, 32 * (box_a + k) + lane, true, 0.0f);
+        cur.b = load_pose<true>(a, 32 * (box_b + k) + lane, true, 0.0f);
+    };
+    // the warp's step of the next batch: of the active steps in `mask` (bit b: step k0 + b), rank base + w
+    int k0 = B.k0, base = 0;
+    unsigned mask = B.mask;
+    auto next_chunk = [&](int from) {               // the next 32 steps with an active one (mask 0: none)
+        base = 0;
+        for (k0 = from; k0 < P.n_steps; k0 += 32) {
+            const int k = k0 + lane;
+            mask = __ballot_sync(0xffffffffu, k < P.n_steps && boxes_meet(a.bounds[box_a + k], a.bounds[box_b + k], P.r_cull));
+            if (mask) return;
+        }
+    };
+    if (!mask) next_chunk(k0);
+    if (!mask) return;                              // (uniform over the CTA)
+    auto mine = [&]() -> int { return base + w < __popc(mask) ? k0 + nth_set_bit(mask, base + w) : -1; };
+    int k = mine();
+    if (k >= 0) load(k);
+    for (int q = tid; q < 32 * kFirstRow; q += 32 * W) S.first[q] = kNone;
+    if (w < 2) {                                    // warp 0: the rows, warp 1: the columns
+        const int tile = w ? B.tile_b : B.tile_a;
+        const bool ok = 32 * tile + lane < (w ? P.h_b : P.h_a);
+        const int h = a.tile_order[32LL * ((w ? P.tile_b : P.tile_a) + tile) + lane];
+        S.order[w][lane] = h;
+        if (FUSED) {                                // asynchronous: the latency hides under the tests
+            const long long traj = (w ? P.traj_b : P.traj_a) + h;
+            if (ok) cp_async4(&S.prob[w][lane], a.probf + traj); else S.prob[w][lane] = 0.0f;
+            if (ok && P.ego_side == 1 - w) {        // the CO's side
+                cp_async8(S.lfix + lane, a.lfix + traj);
+                cp_async8(S.pfix + lane, a.pfix + traj);
+            }
+        }
+    }
+    if (w == W - 1) S.found[lane] = 0u;
+    if (w == W - 2 && lane < 2) S.queued[lane] = 0;
+    const PairShape shape = shape_of(P);
+    const Extents ext{P.hl_a, P.hw_a, P.rad_a, P.hl_b, P.hw_b, P.rad_b};
+    const float rc2 = P.rc2 + kEps0;
+    __syncthreads();                                // S.first, S.found, S.queued initialised
+    unsigned narrow = 0;                            // this lane's exact tests
+    int steps = 0, parity = 0;
+    while (mask) {                                  // (uniform over the CTA)
+        unsigned cand = 0u;
+        if (k >= 0) cand = stage_and_sweep(S.step[w], cur, rc2, lane) & ~S.found[lane];
+        if (lane == 0) S.at[w] = k;
+        steps += k >= 0;
+        base += W;
+        if (base >= __popc(mask)) {
+            mask = 0u;
+            next_chunk(k0 + 32);
+        }
+        k = mine();
+        if (k >= 0) load(k);                        // in flight while the candidates are tested
+        bool more;
+        do {                                        // (a second round only where a lane has over 15 candidates)
+            const int n = min(__popc(cand), kLaneQueue);
+            int off, total, at = 0;
+            if (queue_offsets6(n, lane, off, total)) {
+                if (lane == 0) at = atomicAdd(&S.queued[parity], total);
+                off += __shfl_sync(0xffffffffu, at, 0);
+                for (int u = 0; u < n; ++u, cand &= cand - 1u)
+                    S.queue[off + u] = (unsigned short)(w << 10 | lane << 5 | (__ffs(cand) - 1));
+            }
+            __syncthreads();
+            const int queued = S.queued[parity];
+            if (tid == 0) S.queued[parity ^ 1] = 0;
+            for (int u = tid; u < queued; u += 64 * W) {   // two candidates of a lane in flight
+                const int u2 = u + 32 * W, e = S.queue[u], e2 = S.queue[u2 < queued ? u2 : u];
+                const bool h = overlap<OUTL>(S.step[e >> 10], shape, a.polys, ext, e);
+                const bool h2 = (u2 - lane < queued) && overlap<OUTL>(S.step[e2 >> 10], shape, a.polys, ext, e2);
+                narrow += u2 < queued ? 2 : 1;
+                if (h) {
+                    atomicOr(&S.found[e >> 5 & 31], 1u << (e & 31));
+                    atomicMin(&S.first[kFirstRow * queued_row(e) + queued_col(e)], S.at[e >> 10]);
+                }
+                if (h2 && u2 < queued) {
+                    atomicOr(&S.found[e2 >> 5 & 31], 1u << (e2 & 31));
+                    atomicMin(&S.first[kFirstRow * queued_row(e2) + queued_col(e2)], S.at[e2 >> 10]);
+                }
+            }
+            parity ^= 1;
+            more = __syncthreads_or(cand != 0u);
+        } while (more);
+    }
+    if (a.counters) {
+        narrow = __reduce_add_sync(0xffffffffu, narrow);
+        if (lane == 0) {
+            if (narrow) count_narrow(a, P.combo, narrow);
+            if (steps) atomicAdd(a.counters, (unsigned long long)steps * 32 * 32);
+        }
+    }
+    if (FUSED) {
+        cp_async_wait();
+        __syncthreads();                            // the copies of the first warps
+    }
+
+    // ---- the first hits of the warp's ROWS lines (rows, or columns where b is the EGO object, so that a line is one
+    // EGO hypothesis): the table entries and (fused) the risk terms
+    const int N = P.n_steps, ego_side = P.ego_side, l0 = w * ROWS, line = ego_side == 1 ? 1 : kFirstRow;
+    const int across = ego_side == 1 ? kFirstRow : 1;
+    int at[ROWS];                                   // first steps of this lane's pair in each line
+    unsigned hits = 0u;                             // bit u: the pair in line u hit
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u) {
+        at[u] = S.first[line * (l0 + u) + across * lane];
+        if (at[u] != kNone) hits |= 1u << u;
+    }
+    const int total = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(hits));
+    if (!total) return;
+    const int n_obj_s = P.n_obj_s, co_local = P.co_local, hb = P.h_b;
+    const long long kofs = P.kofs, lsum_base = P.lsum_base, mass_base = P.mass_base, hits_base = P.hits_base;
+    int16_t *tab = a.table + P.off;
+    const int *line_h = S.order[ego_side == 1], hl = S.order[ego_side != 1][lane];   // the lines' hypotheses, the lane's
+    unsigned long long wt[ROWS] = {};
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u) {
+        if (!(hits >> u & 1u)) continue;
+        const int h = line_h[l0 + u];
+        tab[ego_side == 1 ? (long long)hl * hb + h : (long long)h * hb + hl] = (int16_t)at[u];
+        if (FUSED) wt[u] = to_fixed(S.prob[ego_side == 1][l0 + u] * S.prob[ego_side != 1][lane], kFixProb);
+    }
+    if constexpr (FUSED) {
+        // one step of the warp's hits at a time: its terms summed over the lanes, per EGO hypothesis and over the lines
+        const unsigned long long lf = ego_side >= 0 ? S.lfix[lane] : 0ull, pf = ego_side >= 0 ? S.pfix[lane] : 0ull;
+        unsigned count = 0;
+        unsigned long long mass = 0;
+        // Many hits a step: a loop over the steps (one reduction per hit and sum, on few addresses, took up to 34 us for
+        // a block of 1,024 hits; EGO-only call 136 -> 101 us).  Else one reduction per hit: a turn of the loop is 150
+        // instructions (always looping, the 11-object call takes 51.4 us instead of 48.1; from 8 hits a step 49.1).
+        int lo = kNone, hi = 0;
+#pragma unroll
+        for (int u = 0; u < ROWS; ++u)
+            if (hits >> u & 1u) { lo = min(lo, at[u]); hi = max(hi, at[u]); }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        const bool dense = total >= kHitsPerStep * (hi - lo + 1);
+        if (!dense) {
+#pragma unroll
+            for (int u = 0; u < ROWS; ++u) {
+                if (!(hits >> u & 1u)) continue;
+                atomicAdd(a.acc.count_k + kofs + at[u], 1ull);
+                atomicAdd(a.acc.H + kofs + at[u], wt[u]);
+                ++count;
+                mass += wt[u];
+                if (ego_side >= 0)
+                    atomicAdd(a.acc.lsum + lsum_base + ((long long)line_h[l0 + u] * N + at[u]) * n_obj_s + co_local, lf);
+            }
+            count = __reduce_add_sync(0xffffffffu, count);
+            mass = reduce_terms(mass);
+        }
+        for (unsigned left = dense ? hits : 0u;;) {
+            const unsigned lanes = __ballot_sync(0xffffffffu, left != 0u);
+            if (!lanes) break;
+            int k = kNone;                          // the lane's earliest step
+#pragma unroll
+            for (int u = 0; u < ROWS; ++u)
+                if (left >> u & 1u) k = min(k, at[u]);
+            k = __reduce_min_sync(0xffffffffu, k);
+            unsigned c = 0;
+            unsigned long long v = 0;
+#pragma unroll
+            for (int u = 0; u < ROWS; ++u) {
+                const bool now = (left >> u & 1u) && at[u] == k;
+                const unsigned m = __ballot_sync(0xffffffffu, now);
+                if (!m) continue;
+                if (now) {
+                    v += wt[u];
+                    left &= ~(1u << u);
+                }
+                c += __popc(m);
+                if (ego_side < 0) continue;
+                const unsigned long long sum = reduce_terms(now ? lf : 0ull);
+                if (lane == 0)
+                    atomicAdd(a.acc.lsum + lsum_base + ((long long)line_h[l0 + u] * N + k) * n_obj_s + co_local, sum);
+            }
+            v = reduce_terms(v);
+            if (lane == 0) {
+                atomicAdd(a.acc.count_k + kofs + k, (unsigned long long)c);
+                atomicAdd(a.acc.H + kofs + k, v);
+            }
+            count += c;
+            mass += v;
+        }
+        if (ego_side >= 0) {
+#pragma unroll
+            for (int u = 0; u < ROWS; ++u) {
+                const unsigned m = __ballot_sync(0xffffffffu, hits >> u & 1u);
+                if (!m) continue;
+                const unsigned long long sum = reduce_terms(hits >> u & 1u ? pf : 0ull);
+                if (lane == 0) {
+                    const long long e = line_h[l0 + u];
+                    atomicAdd(a.acc.mass + mass_base + e * n_obj_s + co_local, sum);
+                    atomicAdd(a.acc.hits + hits_base + e, (unsigned long long)__popc(m));
+                }
+            }
+        }
+        if (lane == 0) {
+            atomicAdd(a.acc.count + P.index, (unsigned long long)count);
+            atomicAdd(a.acc.P + P.index, mass);
+        }
+    }
+}
+
+// LISTED: CTAs take the listed blocks in order, the heavy ones first.  Otherwise CTA g has block g of the ascending
+// tiles: where all blocks fit on the chip at once the listing would only delay them (3 us of a 19 us call with two
+// objects of 16 hypotheses; with 5,780 blocks, most of them empty, it saves 9 of 56 us).
+
+template <bool FUSED, bool OUTL, bool LISTED>
+__global__ void __launch_bounds__(32 * kBlockWarps, kBlockCtas) block_kernel(const CollideArgs a) {
+    pdl_trigger();
+    __shared__ BlockSlot S;
+    if (!LISTED) {
+        const long long g = blockIdx.x;
+        BlockRef B{};
+        B.pair = pair_of_tile(a, g >> 2);           // uploaded data: before the wait
+        const PairDesc &P = a.pairs[B.pair];
+        const int t = (int)((g >> 2) - P.tile_start), ta = t / P.tiles_b, q = (int)(g & 3);
+        B.tile_a = 2 * ta + (q >> 1);
+        B.tile_b = 2 * (t - ta * P.tiles_b) + (q & 1);
+        B.box_a = (int)(P.bounds_a + (long long)B.tile_a * P.n_steps);
+        B.box_b = (int)(P.bounds_b + (long long)B.tile_b * P.n_steps);
+        const bool in = 32 * B.tile_a < P.h_a && 32 * B.tile_b < P.h_b;
+        pdl_wait();
+        if (in) block_work<FUSED, OUTL>(a, B, S);
+        return;
+    }
+    pdl_wait();
+    const long long front = (long long)a.list_counts[0], listed = front + (long long)a.list_counts[1];
+    for (long long it = blockIdx.x; it < listed; it += gridDim.x) {
+        block_work<FUSED, OUTL>(a, listed_block(a, it, front), S);
+        if (it + gridDim.x < listed) __syncthreads();   // the slots are no longer read
+    }
+}
+
+template <bool OUTL, bool LISTED>
+cudaError_t launch_blocks(const CollideArgs &a, long long ctas, cudaStream_t st, bool pdl) {
+    if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const dim3 grid((unsigned)ctas), block(32 * kBlockWarps);
+    return a.probf ? launch_kernel(block_kernel<true, OUTL, LISTED>, grid, block, 0, st, pdl, a)
+                   : launch_kernel(block_kernel<false, OUTL, LISTED>, grid, block, 0, st, pdl, a);
+}
+
 template <bool OUTL>
 cudaError_t launch_listed(const CollideArgs &a, cudaStream_t st, bool pdl) {
+    const long long blocks = 4 * a.n_tiles;
+    if (a.variant == 7 && blocks <= kBlockSlots) return launch_blocks<OUTL, false>(a, blocks, st, pdl);
     // 8 tiles per warp once that still gives every SM a few warps
     const int per_warp = a.n_tiles >= 152LL * 8 * 32 ? 8 : 1;
     const long long tiles = (long long)kListWarps * per_warp;
     cudaError_t e = launch_kernel(block_list_kernel, dim3((unsigned)((a.n_tiles + tiles - 1) / tiles)), dim3(32 * kListWarps),
                                   0, st, pdl, a, per_warp);
     if (e != cudaSuccess) return e;
+    if (a.variant == 7)                             // up to four waves of CTAs, further blocks in turn
+        return launch_blocks<OUTL, true>(a, std::min(blocks, 4LL * kBlockSlots), st, true);
     // CTAs for every block of every tile (the warps of those past the last listed block leave at once)
     const long long ctas = (4 * a.n_tiles + kWalkWarps * kWalkBlocks - 1) / (kWalkWarps * kWalkBlocks);
-    const dim3 grid((unsigned)ctas), block(32 * kWalkWarps);
-    return a.probf ? launch_kernel(walk_kernel<true, OUTL, false>, grid, block, 0, st, true, a)
-                   : launch_kernel(walk_kernel<false, OUTL, false>, grid, block, 0, st, true, a);
+    const dim3 grid((unsigned)ctas), walk(32 * kWalkWarps);
+    return a.probf ? launch_kernel(walk_kernel<true, OUTL, false>, grid, walk, 0, st, true, a)
+                   : launch_kernel(walk_kernel<false, OUTL, false>, grid, walk, 0, st, true, a);
 }
 
 template <bool OUTL>
@@ -380,6 +679,10 @@ cudaError_t launch_unlisted(const CollideArgs &a, cudaStream_t st, bool pdl) {
 }
 
 }  // namespace
+
+int tiles_launches(const CollideArgs &a) {
+    return a.tile_poses && !(a.variant == 7 && 4 * a.n_tiles <= kBlockSlots) ? 2 : 1;
+}
 
 cudaError_t launch_tiles(const CollideArgs &a, cudaStream_t st, bool pdl) {
     if (a.tile_poses) {     // the table's -1s and the list's counts are written beforehand

@@ -699,13 +699,14 @@ __global__ void __launch_bounds__(256) bounds_kernel(const BoundsArgs a) {
     pdl_trigger();
     const int chunks = (a.max_steps + kBoundSteps - 1) / kBoundSteps;
     const long long total = (long long)a.n_warps * chunks;
-    const long long bound_ctas = (total + 7) / 8;
+    const int warps = blockDim.x >> 5;
+    const long long bound_ctas = (total + warps - 1) / warps;
     if ((long long)blockIdx.x >= bound_ctas) {   // a fill CTA
         fill_part(a.fill, a.n_fill, (long long)blockIdx.x - bound_ctas, (long long)gridDim.x - bound_ctas);
         pdl_wait();
         return;
     }
-    const long long g = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const long long g = (long long)blockIdx.x * warps + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     bool live = g < total;
     int k0 = 0, first = 0, h = 0, n_steps = 0, i = 0, tile = 0;
@@ -802,11 +803,12 @@ cudaError_t launch_generate(const GenArgs &args, cudaStream_t st, bool pdl) {
 cudaError_t launch_bounds(const BoundsArgs &a, cudaStream_t st, bool pdl) {
     const long long total = (long long)a.n_warps * ((a.max_steps + kBoundSteps - 1) / kBoundSteps);
     if (total <= 0) return cudaSuccess;
-    long long blocks = (total + 7) / 8;
-    if (a.fill && a.n_fill > 0) blocks += std::min((long long)kFillCtas, (a.n_fill / 8 + 255) / 256 + 1);
+    const int warps = total < 152 * 8 ? 2 : 8;       // few tasks: spread over the SMs (11 objects: 1 us less than 8)
+    long long blocks = (total + warps - 1) / warps;
+    if (a.fill && a.n_fill > 0) blocks += std::min((long long)kFillCtas * 8 / warps, (a.n_fill / 8 + 32 * warps - 1) / (32 * warps) + 1);
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    return a.tile_poses ? launch_kernel(bounds_kernel<true>, dim3((unsigned)blocks), dim3(256), 0, st, pdl, a)
-                        : launch_kernel(bounds_kernel<false>, dim3((unsigned)blocks), dim3(256), 0, st, pdl, a);
+    return a.tile_poses ? launch_kernel(bounds_kernel<true>, dim3((unsigned)blocks), dim3(32 * warps), 0, st, pdl, a)
+                        : launch_kernel(bounds_kernel<false>, dim3((unsigned)blocks), dim3(32 * warps), 0, st, pdl, a);
 }
 
 }  // namespace mhc

@@ -278,9 +278,13 @@ struct __align__(16) ActiveBlock {
     unsigned mask;
 };
 
-// A 32 x 32 block of layout 4 with an active step: bound tiles tile_a and tile_b of the pair's objects.
+// A 32 x 32 block with an active step (layouts 4 and 7): bound tiles tile_a and tile_b of the pair's objects, the first
+// 32 steps k0 .. with an active one and which these are (bit b of mask: step k0 + b), and the index of the tiles' first
+// boxes (the tile-ordered poses take 512 bytes a box, so 32 bits are enough): the first poses are one load away.
 struct __align__(16) BlockRef {
-    int pair, tile_a, tile_b, pad_;
+    int pair, tile_a, tile_b, k0;
+    unsigned mask;
+    int box_a, box_b, pad_;
 };
 
 // One item of the step-item layout: an active step k of block gw, with the pose indices of the step's first
@@ -309,7 +313,7 @@ struct CollideArgs {
     ItemBlock *blocks;        // [4 n_tiles] the records of the active blocks (indexed by block)
     unsigned long long *active_count;
     ActiveBlock *recs;        // variant 8: [4 n_tiles] the records of the active blocks ([*active_count] valid)
-    BlockRef *list;           // variant 4 with tile_poses: [4 n_tiles] the active blocks, list_counts[0] from the
+    BlockRef *list;           // variants 4, 7 with tile_poses: [4 n_tiles] the active blocks, list_counts[0] from the
                               // front (those with many active steps) and list_counts[1] from the back
     unsigned long long *list_counts;   // [2]: blocks the walk's warps have taken; all three zeroed by the caller
     long long max_items;      // capacity: 4 n_tiles x max_steps
@@ -388,6 +392,7 @@ cudaError_t launch_generate(const GenArgs &a, cudaStream_t st, bool pdl = false)
 cudaError_t launch_bounds(const BoundsArgs &a, cudaStream_t st, bool pdl = false);
 cudaError_t launch_fill_table(int16_t *table, long long n, cudaStream_t st, bool pdl = false);   // table[0, n) = -1
 cudaError_t launch_collide(const CollideArgs &a, cudaStream_t st, bool pdl = false);  // stores first hits only
+int tiles_launches(const CollideArgs &a);   // kernel launches of launch_tiles
 cudaError_t launch_tiles(const CollideArgs &a, cudaStream_t st, bool pdl);   // variant 4 (collide_tiles.cu)
 cudaError_t launch_risk_prepare(const RiskArgs &a, cudaStream_t st);             // zero + normalise
 int risk_tail_launches(const RiskArgs &a);   // kernels launch_risk_tail launches
