@@ -382,7 +382,7 @@ int build_layout(const mhc_scenario *sc, int n_scen, Layout &L) {
 int build_layout(const mhc_scenario *sc, Layout &L) { return build_layout(sc, 1, L); }
 
 // Generation warp tasks: a hypothesis is a sequential chain of sub-steps, so with fewer hypotheses than
-// warp schedulers (4 per SM) each warp takes fewer of them (down to 4) to occupy every scheduler.
+// warp schedulers (4 per SM) each warp takes fewer of them (down to 8) to occupy every scheduler.
 void plan_generation(Layout &L, int n_sm, int mode) {
     L.gen_obj.clear();
     L.gen_first.clear();
@@ -407,11 +407,12 @@ void plan_generation(Layout &L, int n_sm, int mode) {
     L.n_gen_scan = (int)warps;
     L.n_gen_scan_objs = (int)L.gen_obj.size();
     // the others: one thread per hypothesis, `lanes` per warp; with fewer hypotheses than warp schedulers
-    // (4 per SM) each warp takes fewer of them (down to 4) to occupy every scheduler (more, smaller warps
-    // measured slower on large scenes, where the sub-steps' instructions fill the issue slots)
+    // (4 per SM) each warp takes fewer of them (down to 8) to occupy every scheduler (more, smaller warps
+    // measured slower on large scenes, where the sub-steps' instructions fill the issue slots; 3,087 lane-path
+    // hypotheses, whole call: 100.7 us with 8 a warp, 104.7 with 4 and a second warp on a quarter of the schedulers)
     const long long schedulers = 4LL * (n_sm > 0 ? n_sm : 152);
     int lanes = 32;
-    while (lanes > 4 && (seq_traj + lanes - 1) / lanes < schedulers) lanes >>= 1;
+    while (lanes > 8 && (seq_traj + lanes - 1) / lanes < schedulers) lanes >>= 1;
     L.gen_lanes = lanes;
     long long tasks = 0;
     for (int o = 0; o < L.n_obj; ++o)

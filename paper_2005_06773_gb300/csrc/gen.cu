@@ -40,14 +40,8 @@ __device__ __forceinline__ void sincos2(float a_hi, float a_lo, float &sn, float
     sn = fmaf(c0, a_lo, s0);
 }
 
-// sin / cos by the Taylor series to x^9 / x^10 (|x| <= 0.5: error < 2e-11), sincosf beyond.
-__device__ __forceinline__ void sincos_half(float x, float &sn, float &cs) {
-    if (fabsf(x) > 0.5f) {
-        const float2 sc = sincos_any(x);
-        sn = sc.x;
-        cs = sc.y;
-        return;
-    }
+// sin / cos by the Taylor series to x^9 / x^10 (|x| <= 0.5: error < 2e-11).
+__device__ __forceinline__ void sincos_half_series(float x, float &sn, float &cs) {
     const float x2 = x * x;
     float ps = fmaf(x2, 1.0f / 362880.0f, -1.0f / 5040.0f);
     ps = fmaf(x2, ps, 1.0f / 120.0f);
@@ -60,7 +54,25 @@ __device__ __forceinline__ void sincos_half(float x, float &sn, float &cs) {
     cs = fmaf(x2, pc, 1.0f);
 }
 
-// sin / cos by the Taylor series to x^5 / x^6 (|x| <= 0.1: error < 3e-11), sincosf beyond.
+// The series, sincosf beyond its range.
+__device__ __forceinline__ void sincos_half(float x, float &sn, float &cs) {
+    if (fabsf(x) > 0.5f) {
+        const float2 sc = sincos_any(x);
+        sn = sc.x;
+        cs = sc.y;
+        return;
+    }
+    sincos_half_series(x, sn, cs);
+}
+
+// sin / cos by the Taylor series to x^5 / x^6 (|x| <= 0.1: error < 3e-11).
+__device__ __forceinline__ void sincos_tenth_series(float x, float &sn, float &cs) {
+    const float x2 = x * x;
+    sn = fmaf(x * x2, fmaf(x2, 1.0f / 120.0f, -1.0f / 6.0f), x);
+    cs = fmaf(x2, fmaf(x2, fmaf(x2, -1.0f / 720.0f, 1.0f / 24.0f), -0.5f), 1.0f);
+}
+
+// The series, sincosf beyond its range.
 __device__ __forceinline__ void sincos_tenth(float x, float &sn, float &cs) {
     if (fabsf(x) > 0.1f) {
         const float2 sc = sincos_any(x);
@@ -68,9 +80,7 @@ __device__ __forceinline__ void sincos_tenth(float x, float &sn, float &cs) {
         cs = sc.y;
         return;
     }
-    const float x2 = x * x;
-    sn = fmaf(x * x2, fmaf(x2, 1.0f / 120.0f, -1.0f / 6.0f), x);
-    cs = fmaf(x2, fmaf(x2, fmaf(x2, -1.0f / 720.0f, 1.0f / 24.0f), -0.5f), 1.0f);
+    sincos_tenth_series(x, sn, cs);
 }
 
 __device__ void vehicle(const ObjDesc &o, float acc, float delta, const Regime &g, int N, int K, double tau_i_d,
@@ -98,10 +108,12 @@ __device__ void vehicle(const ObjDesc &o, float acc, float delta, const Regime &
     float cps, sps;                      // cos / sin of the heading, carried between output steps
     sincos2(ph, -pc, sps, cps);
     float beta = 0.0f, r = 0.0f, ax = acc, ay = 0.0f;
+    const int last = __reduce_max_sync(__activemask(), n_stop);   // every hypothesis of the warp has stopped after it
     bool stopped = false;
     int n = 0;
     for (int k = 0; k < N; ++k) {
-        for (int q = 0; q < K; ++q, ++n) {
+        // (a warp whose hypotheses have all stopped only stores their poses)
+        for (int q = 0; q < K && n <= last; ++q, ++n) {
             // every lane runs the same straight-line sub-step; regime and stop act through selects
             const bool low = n >= low_lo && n < low_hi;
             const bool stop_now = n == n_stop;
@@ -161,106 +173,162 @@ constexpr float kDeltaMax = 0.5f;     // rad
 constexpr float kDeltaRate = 0.5f;    // rad/s
 constexpr float kPi = 3.14159265358979f;
 
+// a / b, correctly rounded, with y = 1 / b correctly rounded: Markstein's quotient iteration (P. Markstein, Computation
+// of elementary functions on the IBM RISC System/6000 processor, 1990): the first correction leaves q within one unit in
+// the last place, the second, with its exact remainder, rounds it.  Small |a| (a remainder may be subnormal; the sign of
+// a zero) take the division.
+__device__ __forceinline__ float quotient(float a, float b, float y) {
+    float q = a * y;
+    q = fmaf(fmaf(-q, b, a), y, q);
+    q = fmaf(fmaf(-q, b, a), y, q);
+    return fabsf(a) > 1e-20f ? q : a / b;
+}
+
+struct PathConst {                     // of one hypothesis
+    float acc, dv, v0, ti, hti2, lr, L, inv_L, k11, k12, k21, k22, kb1u, kb2u, stop_den, step_max;
+};
+struct PathSection {                   // point, direction, left normal
+    float x, y, psi, nx, ny;
+};
+struct PathState {
+    float xh, xc, yh, yc, ph, pc;      // Kahan sums
+    float cps, sps;
+    float beta, r, ax, ay, delta;
+};
+
+// One sub-step (n).  GENERAL: any state.  Otherwise for a sub-step outside the low-speed regime, without a branch;
+// returns false if a slip angle or heading increment is out of the short series' range (the state is then not valid).
+template <bool GENERAL>
+__device__ __forceinline__ bool path_step(const PathConst &p, const PathSection &sec, PathState &s, int n, bool low,
+                                          bool stop_now, bool stopped) {
+    const float v = fmaf((float)n, p.dv, p.v0);
+    float sb0, cb0;                                              // the course of the state before the step
+    if (GENERAL) sincos_half(s.beta, sb0, cb0); else sincos_half_series(s.beta, sb0, cb0);
+    bool ok = GENERAL || !(fabsf(s.beta) > 0.5f);
+    {   // the controller, on the state before this sub-step
+        const float px = (s.xh - s.xc) + kCtrlTp * v * fmaf(s.cps, cb0, -s.sps * sb0);
+        const float py = (s.yh - s.yc) + kCtrlTp * v * fmaf(s.sps, cb0, s.cps * sb0);
+        const float d_path = fmaf(sec.x - px, sec.nx, (sec.y - py) * sec.ny);
+        float e_psi = sec.psi - (s.ph - s.pc);
+        e_psi -= 2.0f * kPi * floorf((e_psi + kPi) * (0.5f / kPi));
+        const float gd = fabsf(fmaf(-0.018f, v, 1.5f) * d_path);
+        const float cmd = ((gd + 0.5f) * d_path + (9.5f - gd) * (3.8197f * e_psi)) * (kPi / 180.0f);
+        const float delta = fminf(fmaxf(s.delta + fminf(fmaxf(cmd - s.delta, -p.step_max), p.step_max), -kDeltaMax), kDeltaMax);
+        s.delta = stopped ? s.delta : delta;
+    }
+    const float kb1 = p.kb1u * s.delta, kb2 = p.kb2u * s.delta;
+    float beta_kin = 0.0f, kappa = 0.0f;
+    float sb = sb0, cb = cb0;                                    // the one-track step keeps the course
+    if (GENERAL && low) {                                        // the kinematic limit at the new angle
+        const float tdel = tanf(s.delta);
+        beta_kin = atanf(quotient(p.lr * tdel, p.L, p.inv_L));
+        kappa = quotient(cosf(beta_kin) * tdel, p.L, p.inv_L);
+        sincos_half(beta_kin, sb, cb);
+    }
+    const float iv = __fdividef(1.0f, fmaxf(v, 1e-3f));
+    const float bd_ot = fmaf(p.k11 * iv, s.beta, fmaf(fmaf(p.k12 * iv, iv, -1.0f), s.r, kb1 * iv));
+    const float rd_ot = fmaf(p.k21, s.beta, fmaf(p.k22 * iv, s.r, kb2));
+    const float b_use = low ? beta_kin : s.beta;
+    const float r_use = low ? v * kappa : s.r;
+    const float bd = low ? 0.0f : bd_ot;
+    const float rd = low ? 0.0f : rd_ot;
+    const float cpb = fmaf(s.cps, cb, -s.sps * sb);
+    const float spb = fmaf(s.sps, cb, s.cps * sb);
+    const float d_stop = v * v * p.stop_den;
+    const float dx = stop_now ? cpb * d_stop : fmaf(cpb * v, p.ti, fmaf(s.cps, s.ax, -s.sps * s.ay) * p.hti2);
+    const float dy = stop_now ? spb * d_stop : fmaf(spb * v, p.ti, fmaf(s.sps, s.ax, s.cps * s.ay) * p.hti2);
+    const float w = v * (bd + r_use);
+    const float ax_n = fmaf(cb, p.acc, -sb * w);
+    const float ay_n = fmaf(sb, p.acc, cb * w);
+    const float dpsi = fmaf(r_use, p.ti, rd * p.hti2);
+    const bool move = !stopped && !stop_now;                     // a state update beyond the position
+    kahan_add(s.xh, s.xc, stopped ? 0.0f : dx);
+    kahan_add(s.yh, s.yc, stopped ? 0.0f : dy);
+    kahan_add(s.ph, s.pc, move ? dpsi : 0.0f);
+    float sd, cd;                                                // rotate (cos, sin) of the heading by dpsi
+    if (GENERAL) sincos_tenth(move ? dpsi : 0.0f, sd, cd); else sincos_tenth_series(dpsi, sd, cd);
+    ok = ok && (GENERAL || !move || !(fabsf(dpsi) > 0.1f));
+    const float c2 = fmaf(s.cps, cd, -s.sps * sd);
+    const float s2 = fmaf(s.sps, cd, s.cps * sd);
+    const float b2 = fmaf(bd, p.ti, b_use), r2 = fmaf(rd, p.ti, r_use);
+    s.beta = move ? b2 : s.beta;
+    s.r = move ? r2 : s.r;
+    s.ax = move ? ax_n : s.ax;
+    s.ay = move ? ay_n : s.ay;
+    s.sps = move ? s2 : s.sps;
+    s.cps = move ? c2 : s.cps;
+    return ok;
+}
+
+// One path hypothesis, in order: the controller feeds each sub-step's state back.  Latency-bound: a sub-step is a chain
+// of some 170 instructions.  Outside the low-speed regime the warp runs the short body (no branch but the votes), inside
+// it the general one (three times as long: tanf, atanf, cosf and the short series' other case); a hypothesis that has
+// stopped is not in the regime, and a warp whose hypotheses have all stopped only stores their poses.  3,087 path
+// hypotheses (11-object scene): generation 57 us, 90 with the low regime run to the horizon's end, section values indexed
+// in local memory and two divisions per low sub-step (a hypothesis braking at 9 m/s^2 spent three quarters of its time
+// after its stop).
 __device__ void vehicle_path(const ObjDesc &o, float acc, const float *path, const Regime &g, int N, int K,
                              double tau_i_d, long long base, int h, int i, float *X, float *Y, float *C, float *S) {
-    const float dv = (float)__dmul_rn((double)acc, tau_i_d);
-    const int low_lo = g.low_lo, low_hi = g.low_hi, n_stop = g.n_stop;
-    const float ti = (float)tau_i_d;
-    const float hti2 = 0.5f * ti * ti;
-    const float L = o.lf + o.lr;
+    const unsigned lanes = __activemask();
+    const int low_lo = g.low_lo, low_hi = g.low_hi, n_stop = g.n_stop, n1 = o.path_n1, n2 = o.path_n2;
+    PathConst p;
+    p.acc = acc;
+    p.dv = (float)__dmul_rn((double)acc, tau_i_d);
+    p.v0 = o.v0;
+    p.ti = (float)tau_i_d;
+    p.hti2 = 0.5f * p.ti * p.ti;
+    p.lr = o.lr;
+    p.L = o.lf + o.lr;
+    p.inv_L = 1.0f / p.L;
     const float inv_m = 1.0f / o.m, inv_iz = 1.0f / o.Iz;
-    const float k11 = -(o.caf + o.car) * inv_m;
-    const float k12 = (o.car * o.lr - o.caf * o.lf) * inv_m;
-    const float k21 = (o.car * o.lr - o.caf * o.lf) * inv_iz;
-    const float k22 = -(o.caf * o.lf * o.lf + o.car * o.lr * o.lr) * inv_iz;
-    const float kb1u = o.caf * inv_m;                           // b1 * v per rad of steering
-    const float kb2u = o.caf * o.lf * inv_iz;                   // b2 per rad of steering
-    const float stop_den = 0.5f / fabsf(acc == 0.0f ? 1.0f : acc);
-    const float step_max = kDeltaRate * ti;
-    float sec_x[3], sec_y[3], sec_psi[3], sec_nx[3], sec_ny[3];  // sections: point, direction, left normal
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        sec_x[q] = path[3 * q];
-        sec_y[q] = path[3 * q + 1];
-        sec_psi[q] = path[3 * q + 2];
-        float sn, cs;
-        sincosf(sec_psi[q], &sn, &cs);
-        sec_nx[q] = -sn;
-        sec_ny[q] = cs;
-    }
-
-    float xh = o.x0, xc = 0.0f, yh = o.y0, yc = 0.0f, ph = o.psi0, pc = 0.0f;   // Kahan sums
-    float cps, sps;
-    sincos2(ph, -pc, sps, cps);
-    float beta = 0.0f, r = 0.0f, ax = acc, ay = 0.0f, delta = 0.0f;
-    bool stopped = false;
+    p.k11 = -(o.caf + o.car) * inv_m;
+    p.k12 = (o.car * o.lr - o.caf * o.lf) * inv_m;
+    p.k21 = (o.car * o.lr - o.caf * o.lf) * inv_iz;
+    p.k22 = -(o.caf * o.lf * o.lf + o.car * o.lr * o.lr) * inv_iz;
+    p.kb1u = o.caf * inv_m;                                     // b1 * v per rad of steering
+    p.kb2u = o.caf * o.lf * inv_iz;                             // b2 per rad of steering
+    p.stop_den = 0.5f / fabsf(acc == 0.0f ? 1.0f : acc);
+    p.step_max = kDeltaRate * p.ti;
+    PathState s{o.x0, 0.0f, o.y0, 0.0f, o.psi0, 0.0f};
+    sincos2(s.ph, -s.pc, s.sps, s.cps);
+    s.beta = s.r = s.ay = s.delta = 0.0f;
+    s.ax = acc;
+    // over the warp: the sub-step after which every hypothesis has stopped, and the sub-steps with a low-speed one
+    const int last = __reduce_max_sync(lanes, n_stop), low_end = min(low_hi, n_stop + 1);
+    const int any_lo = __reduce_min_sync(lanes, low_lo < low_end ? low_lo : 0x7fffffff);
+    const int any_hi = __reduce_max_sync(lanes, low_lo < low_end ? low_end : 0);
+    PathSection sec{};
     int n = 0;
     for (int k = 0; k < N; ++k) {
-        for (int q = 0; q < K; ++q, ++n) {
-            const bool low = n >= low_lo && n < low_hi;
-            const bool stop_now = n == n_stop;
-            const float v = fmaf((float)n, dv, o.v0);
-            float sb0, cb0;                                      // the course of the state before the step
-            sincos_half(beta, sb0, cb0);
-            if (!stopped) {   // the controller, on the state before this sub-step
-                const int sec = n < o.path_n1 ? 0 : (n < o.path_n2 ? 1 : 2);
-                const float px = (xh - xc) + kCtrlTp * v * fmaf(cps, cb0, -sps * sb0);
-                const float py = (yh - yc) + kCtrlTp * v * fmaf(sps, cb0, cps * sb0);
-                const float d_path = fmaf(sec_x[sec] - px, sec_nx[sec], (sec_y[sec] - py) * sec_ny[sec]);
-                float e_psi = sec_psi[sec] - (ph - pc);
-                e_psi -= 2.0f * kPi * floorf((e_psi + kPi) * (0.5f / kPi));
-                const float gd = fabsf(fmaf(-0.018f, v, 1.5f) * d_path);
-                const float cmd = ((gd + 0.5f) * d_path + (9.5f - gd) * (3.8197f * e_psi)) * (kPi / 180.0f);
-                delta = fminf(fmaxf(delta + fminf(fmaxf(cmd - delta, -step_max), step_max), -kDeltaMax), kDeltaMax);
+        // (a warp whose hypotheses have all stopped only stores their poses)
+        for (int q = 0; q < K && n <= last; ++q, ++n) {
+            if (n == 0 || n == n1 || n == n2) {                  // the section of the sub-steps from here on
+                const float *pt = path + (n < n1 ? 0 : (n < n2 ? 3 : 6));
+                sec.x = pt[0];
+                sec.y = pt[1];
+                sec.psi = pt[2];
+                const float2 sc = sincos_any(sec.psi);
+                sec.nx = -sc.x;
+                sec.ny = sc.y;
             }
-            const float kb1 = kb1u * delta, kb2 = kb2u * delta;
-            float beta_kin = 0.0f, kappa = 0.0f;
-            float sb = sb0, cb = cb0;                            // the one-track step keeps the course
-            if (low) {                                           // the kinematic limit at the new angle
-                const float tdel = tanf(delta);
-                beta_kin = atanf(o.lr * tdel / L);
-                kappa = cosf(beta_kin) * tdel / L;
-                sincos_half(beta_kin, sb, cb);
+            const bool stop_now = n == n_stop, stopped = n > n_stop;
+            const bool low = n >= low_lo && n < low_hi && !stopped;   // (a stopped hypothesis's values are not used)
+            if (n < any_lo || n >= any_hi) {
+                PathState next = s;
+                const bool ok = path_step<false>(p, sec, next, n, false, stop_now, stopped);
+                if (!__any_sync(lanes, !ok)) {
+                    s = next;
+                    continue;
+                }
             }
-            const float iv = __fdividef(1.0f, fmaxf(v, 1e-3f));
-            const float bd_ot = fmaf(k11 * iv, beta, fmaf(fmaf(k12 * iv, iv, -1.0f), r, kb1 * iv));
-            const float rd_ot = fmaf(k21, beta, fmaf(k22 * iv, r, kb2));
-            const float b_use = low ? beta_kin : beta;
-            const float r_use = low ? v * kappa : r;
-            const float bd = low ? 0.0f : bd_ot;
-            const float rd = low ? 0.0f : rd_ot;
-            const float cpb = fmaf(cps, cb, -sps * sb);
-            const float spb = fmaf(sps, cb, cps * sb);
-            const float d_stop = v * v * stop_den;
-            const float dx = stop_now ? cpb * d_stop : fmaf(cpb * v, ti, fmaf(cps, ax, -sps * ay) * hti2);
-            const float dy = stop_now ? spb * d_stop : fmaf(spb * v, ti, fmaf(sps, ax, cps * ay) * hti2);
-            const float w = v * (bd + r_use);
-            const float ax_n = fmaf(cb, acc, -sb * w);
-            const float ay_n = fmaf(sb, acc, cb * w);
-            const float dpsi = fmaf(r_use, ti, rd * hti2);
-            const bool move = !stopped && !stop_now;
-            kahan_add(xh, xc, stopped ? 0.0f : dx);
-            kahan_add(yh, yc, stopped ? 0.0f : dy);
-            kahan_add(ph, pc, move ? dpsi : 0.0f);
-            if (move) {
-                beta = fmaf(bd, ti, b_use);
-                r = fmaf(rd, ti, r_use);
-                ax = ax_n;
-                ay = ay_n;
-                float sd, cd;
-                sincos_tenth(dpsi, sd, cd);
-                const float c2 = fmaf(cps, cd, -sps * sd);
-                sps = fmaf(sps, cd, cps * sd);
-                cps = c2;
-            }
-            stopped = stopped || stop_now;
+            path_step<true>(p, sec, s, n, low, stop_now, stopped);
         }
-        sincos2(ph, -pc, sps, cps);
+        sincos2(s.ph, -s.pc, s.sps, s.cps);
         const long long idx = base + (long long)k * h + i;
-        X[idx] = xh - xc;
-        Y[idx] = yh - yc;
-        C[idx] = cps;
-        S[idx] = sps;
+        X[idx] = s.xh - s.xc;
+        Y[idx] = s.yh - s.yc;
+        C[idx] = s.cps;
+        S[idx] = s.sps;
     }
 }
 
