@@ -193,11 +193,12 @@ __device__ __forceinline__ void for_each_candidate(unsigned cand, int lane, Fn &
     }
 }
 
-// The pair of collision tile g: the last pair (in collision-grid order) whose first tile is <= g.  A 64-way
+// The pair of tile g: the last pair (in the order of a.pairs) whose first tile is <= g.  A 64-way
 // search by the whole warp (every lane must call it with the same g): each round the lanes probe 64
 // evenly spaced pairs at once (two each) and keep the span between the last probe <= g and the next, so up
 // to 64 pairs take one round of loads and 4,096 two (a binary search is a chain of log2 n dependent loads).
-__device__ __forceinline__ int pair_of_tile(const CollideArgs &a, long long g) {
+template <typename Args>
+__device__ __forceinline__ int pair_of_tile(const Args &a, long long g) {
     const int lane = threadIdx.x & 31;
     int lo = 0, hi = a.n_pairs - 1;
     while (lo < hi) {   // 64 probes per round (two per lane): a scene of up to 64 pairs in one round of loads

@@ -15,6 +15,7 @@
 #include <cstdint>
 
 #include "collide_common.cuh"
+#include "hit_terms.cuh"
 
 namespace mhc {
 namespace {
@@ -85,14 +86,6 @@ __device__ __forceinline__ bool overlap(const StepSlot &S, const PairShape &shap
 
 __device__ __forceinline__ bool boxes_meet(const float4 &a, const float4 &b, float r) {
     return (a.x - r <= b.z) && (b.x - r <= a.z) && (a.y - r <= b.w) && (b.y - r <= a.w);
-}
-
-// Sum of v over the warp (v <= 2^62, and the sum too): three 32-bit reductions.
-__device__ __forceinline__ unsigned long long reduce_terms(unsigned long long v) {
-    const unsigned m0 = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xffffffu);
-    const unsigned m1 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 24) & 0xffffffu);
-    const unsigned m2 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 48));
-    return m0 + ((unsigned long long)m1 << 24) + ((unsigned long long)m2 << 48);
 }
 
 // ---- the list of active blocks ------------------------------------------------------------------------------
@@ -382,7 +375,6 @@ __device__ __forceinline__ bool queue_offsets6(int cnt, int lane, int &off, int 
     return true;
 }
 
-constexpr int kHitsPerStep = 16;        // hits per step of a warp's lines from which its terms are summed step by step
 constexpr int kFirstRow = 33;           // (odd: columns read without bank conflicts)
 
 struct BlockSlot {
@@ -506,7 +498,7 @@ __device__ __forceinline__ void block_work(const CollideArgs &a, const BlockRef 
 
     // ---- the first hits of the warp's ROWS lines (rows, or columns where b is the EGO object, so that a line is one
     // EGO hypothesis): the table entries and (fused) the risk terms
-    const int N = P.n_steps, ego_side = P.ego_side, l0 = w * ROWS, line = ego_side == 1 ? 1 : kFirstRow;
+    const int ego_side = P.ego_side, l0 = w * ROWS, line = ego_side == 1 ? 1 : kFirstRow;
     const int across = ego_side == 1 ? kFirstRow : 1;
     int at[ROWS];                                   // first steps of this lane's pair in each line
     unsigned hits = 0u;                             // bit u: the pair in line u hit
@@ -517,8 +509,7 @@ __device__ __forceinline__ void block_work(const CollideArgs &a, const BlockRef 
     }
     const int total = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(hits));
     if (!total) return;
-    const int n_obj_s = P.n_obj_s, co_local = P.co_local, hb = P.h_b;
-    const long long kofs = P.kofs, lsum_base = P.lsum_base, mass_base = P.mass_base, hits_base = P.hits_base;
+    const int hb = P.h_b;
     int16_t *tab = a.table + P.off;
     const int *line_h = S.order[ego_side == 1], hl = S.order[ego_side != 1][lane];   // the lines' hypotheses, the lane's
     unsigned long long wt[ROWS] = {};
@@ -530,84 +521,9 @@ __device__ __forceinline__ void block_work(const CollideArgs &a, const BlockRef 
         if (FUSED) wt[u] = to_fixed(S.prob[ego_side == 1][l0 + u] * S.prob[ego_side != 1][lane], kFixProb);
     }
     if constexpr (FUSED) {
-        // one step of the warp's hits at a time: its terms summed over the lanes, per EGO hypothesis and over the lines
-        const unsigned long long lf = ego_side >= 0 ? S.lfix[lane] : 0ull, pf = ego_side >= 0 ? S.pfix[lane] : 0ull;
-        unsigned count = 0;
-        unsigned long long mass = 0;
-        // Many hits a step: a loop over the steps (one reduction per hit and sum, on few addresses, took up to 34 us for
-        // a block of 1,024 hits; EGO-only call 136 -> 101 us).  Else one reduction per hit: a turn of the loop is 150
-        // instructions (always looping, the 11-object call takes 51.4 us instead of 48.1; from 8 hits a step 49.1).
-        int lo = kNone, hi = 0;
-#pragma unroll
-        for (int u = 0; u < ROWS; ++u)
-            if (hits >> u & 1u) { lo = min(lo, at[u]); hi = max(hi, at[u]); }
-        lo = __reduce_min_sync(0xffffffffu, lo);
-        hi = __reduce_max_sync(0xffffffffu, hi);
-        const bool dense = total >= kHitsPerStep * (hi - lo + 1);
-        if (!dense) {
-#pragma unroll
-            for (int u = 0; u < ROWS; ++u) {
-                if (!(hits >> u & 1u)) continue;
-                atomicAdd(a.acc.count_k + kofs + at[u], 1ull);
-                atomicAdd(a.acc.H + kofs + at[u], wt[u]);
-                ++count;
-                mass += wt[u];
-                if (ego_side >= 0)
-                    atomicAdd(a.acc.lsum + lsum_base + ((long long)line_h[l0 + u] * N + at[u]) * n_obj_s + co_local, lf);
-            }
-            count = __reduce_add_sync(0xffffffffu, count);
-            mass = reduce_terms(mass);
-        }
-        for (unsigned left = dense ? hits : 0u;;) {
-            const unsigned lanes = __ballot_sync(0xffffffffu, left != 0u);
-            if (!lanes) break;
-            int k = kNone;                          // the lane's earliest step
-#pragma unroll
-            for (int u = 0; u < ROWS; ++u)
-                if (left >> u & 1u) k = min(k, at[u]);
-            k = __reduce_min_sync(0xffffffffu, k);
-            unsigned c = 0;
-            unsigned long long v = 0;
-#pragma unroll
-            for (int u = 0; u < ROWS; ++u) {
-                const bool now = (left >> u & 1u) && at[u] == k;
-                const unsigned m = __ballot_sync(0xffffffffu, now);
-                if (!m) continue;
-                if (now) {
-                    v += wt[u];
-                    left &= ~(1u << u);
-                }
-                c += __popc(m);
-                if (ego_side < 0) continue;
-                const unsigned long long sum = reduce_terms(now ? lf : 0ull);
-                if (lane == 0)
-                    atomicAdd(a.acc.lsum + lsum_base + ((long long)line_h[l0 + u] * N + k) * n_obj_s + co_local, sum);
-            }
-            v = reduce_terms(v);
-            if (lane == 0) {
-                atomicAdd(a.acc.count_k + kofs + k, (unsigned long long)c);
-                atomicAdd(a.acc.H + kofs + k, v);
-            }
-            count += c;
-            mass += v;
-        }
-        if (ego_side >= 0) {
-#pragma unroll
-            for (int u = 0; u < ROWS; ++u) {
-                const unsigned m = __ballot_sync(0xffffffffu, hits >> u & 1u);
-                if (!m) continue;
-                const unsigned long long sum = reduce_terms(hits >> u & 1u ? pf : 0ull);
-                if (lane == 0) {
-                    const long long e = line_h[l0 + u];
-                    atomicAdd(a.acc.mass + mass_base + e * n_obj_s + co_local, sum);
-                    atomicAdd(a.acc.hits + hits_base + e, (unsigned long long)__popc(m));
-                }
-            }
-        }
-        if (lane == 0) {
-            atomicAdd(a.acc.count + P.index, (unsigned long long)count);
-            atomicAdd(a.acc.P + P.index, mass);
-        }
+        const bool ego = ego_side >= 0;
+        add_hit_terms<ROWS>(a.acc, P, ego, at, hits, total, wt, [&](int u) { return line_h[l0 + u]; },
+                            ego ? S.lfix[lane] : 0ull, ego ? S.pfix[lane] : 0ull);
     }
 }
 
