@@ -689,8 +689,10 @@ __global__ void __launch_bounds__(128, 6) gen_kernel(const GenArgs a) {
         prepare_block(a.prep, bid - a.gen_blocks, a.prep_blocks);
         return;
     }
-    const int w = bid * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    int w = bid * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (w >= a.n_warps) return;                          // whole warps leave
+    if (LAYOUTS == 3) w = a.n_warps - 1 - w;             // the long sequential chains start first (24 uneven scenarios:
+                                                         // 0.18 ms, 0.22 when they ended the launch)
     if ((LAYOUTS & 1) && (LAYOUTS == 1 || w < a.n_scan)) {   // one hypothesis by the whole warp
         __shared__ ScanSlot slots[4];
         const int lane = threadIdx.x & 31;
@@ -753,10 +755,10 @@ __global__ void __launch_bounds__(128, 6) gen_kernel(const GenArgs a) {
 constexpr int kFillCtas = 152 * 4;
 // Fill CTAs of the generation launch (the rest of each SM integrates).  Two per SM spread the fill's stores
 // over every SM, which a table much larger than the generation work needs to reach the HBM rate (32-vehicle
-// scene: 0.74 ms at two per SM, 0.94 ms at one); when the generation work is comparable, half an SM's worth
-// leaves it more room and both finish sooner (256-scenario batch: 1.68 ms against 2.01 ms).
+// scene: 0.74 ms at two per SM, 0.94 ms at one); when the generation work is comparable, one per SM leaves it more room
+// and both finish sooner (256-scenario batch: 1.69 ms, 1.78 with half as many, 1.83 with twice).
 constexpr int kGenFillCtas = 152 * 2;
-constexpr int kGenFillCtasShared = 76;
+constexpr int kGenFillCtasShared = 152;
 constexpr long long kFillPerHypothesis = 8192;   // table entries per hypothesis above which the fill dominates
 constexpr int kBoundSteps = 8;          // steps per warp task
 
