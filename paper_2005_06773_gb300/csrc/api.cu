@@ -665,10 +665,13 @@ int log2_floor(long long v) {
     return r;
 }
 
-// The collision layout without tuning.  Large scenes (32 tiles per SM and more): a warp per active block, in step
-// order; small ones, whose time is the closest pairs' step chains: a CTA per block, its steps spread over the warps.
+// The collision layout without tuning.  Large scenes: a warp per active block, in step order; small ones, whose time is
+// the closest pairs' step chains: a CTA per block, its steps spread over the warps.  The line by the number of tiles
+// (whole replayed step, layout 4 / 7): 11-object scenes in batches, 5,780 tiles 171 / 137 us, 8,670 212 / 195, 10,115 231 /
+// 227, 11,560 242 / 253; uneven scenes 3,950 177 / 128, 10,899 232 / 259.  Outlines, whose tests are ten times as long:
+// 11,560 tiles 922 / 518, 17,340 1089 / 802.
 int default_variant(const mhc_ctx *ctx, const Layout &L) {
-    return L.n_tiles >= 32LL * ctx->n_sm ? 4 : 7;
+    return L.n_tiles >= (L.polys.empty() ? 64LL : 160LL) * ctx->n_sm ? 4 : 7;
 }
 
 // Collision configuration for a scenario: the forced variant, else the tuned one of its size class, else the
