@@ -106,6 +106,23 @@ void append_rectangle(float hl, float hw, std::vector<PolyVertex> &out) {
     out.push_back(make_float4(-hl, -hw, 0.f, -1.f));
 }
 
+// Half extents of a rectangle about the pose point that lies 1 mm inside the outline: the outline's own extents, scaled
+// until the corners are inside every edge.
+void core_rectangle(const PolyVertex *v, int n, float &core_l, float &core_w) {
+    double l = 0.0, w = 0.0, s = 1.0;
+    for (int q = 0; q < n; ++q) {
+        l = std::max(l, std::fabs((double)v[q].x));
+        w = std::max(w, std::fabs((double)v[q].y));
+    }
+    for (int q = 0; q < n; ++q) {
+        const double nx = v[q].z, ny = v[q].w, support = nx * v[q].x + ny * v[q].y;
+        s = std::min(s, support / (std::fabs(nx) * l + std::fabs(ny) * w));
+    }
+    const bool inside = s * l > 0.002 && s * w > 0.002;
+    core_l = inside ? (float)(s * l - 0.001) : -1e30f;
+    core_w = inside ? (float)(s * w - 0.001) : -1e30f;
+}
+
 // How an object's hypotheses lie in space t seconds ahead: the distance of neighbours along grid_a and along grid_b.
 // Vehicles: da t^2 / 2 and, for steering angles, v^2 db t^2 / (2 L); path hypotheses: the paths' mean distance at
 // their last section.  Pedestrians: da t for speeds (da t^2 / 2 for accelerations) and speed x heading step x t.
@@ -226,6 +243,7 @@ int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
                     append_rectangle(d.hl, d.hw, L.polys);
                 }
                 d.n_poly = (int)L.polys.size() - d.poly_off;
+                core_rectangle(L.polys.data() + d.poly_off, d.n_poly, d.core_l, d.core_w);
             }
         } else {
             if (src.n_vertices != 0) return fail(MHC_E_INVALID, where() + "pedestrians take no outline");

@@ -84,6 +84,70 @@ __device__ __forceinline__ bool overlap(const StepSlot &S, const PairShape &shap
                             x.la, x.wa, x.lb, x.wb, x.ra, x.rb);
 }
 
+__device__ __forceinline__ Verdict first_look(const StepSlot &S, const PairShape &shape, const PolyVertex *polys,
+                                              const Extents &x, int e, const unsigned char *faces) {
+    const float4 qa = S.qa[queued_row(e)], qb = S.qb[queued_col(e)];
+    return outline_verdict(shape, polys, qb.x - qa.x, qb.y - qa.y, make_float2(qa.z, qa.w), make_float2(qb.z, qb.w), x.la,
+                           x.wa, x.lb, x.wb, x.ra, x.rb, faces);
+}
+
+__device__ __forceinline__ bool edge_decides(const StepSlot &S, const PairShape &shape, const PolyVertex *polys,
+                                             const Extents &x, int e, int g, int edges) {
+    const float4 qa = S.qa[queued_row(e)], qb = S.qb[queued_col(e)];
+    return g < edges && outline_edge(shape, polys, qb.x - qa.x, qb.y - qa.y, make_float2(qa.z, qa.w),
+                                     make_float2(qb.z, qb.w), x.ra, x.rb, g);
+}
+
+// A pair's outlines in shared memory, the vertices of two outlines padded to a multiple of four by copies of the first
+// (another vertex, or edge, that is there already: no test changes).
+constexpr int kOutlineSlots = 16;      // MHC_MAX_VERTICES
+__device__ __forceinline__ void load_outline(PolyVertex *slot, const PolyVertex *polys, const PairDesc &P, int side, int lane) {
+    const int first = side ? P.poly_b : P.poly_a, n = side ? P.nv_b : P.nv_a;
+    if (lane < kOutlineSlots && n > 0) slot[lane] = polys[first + (lane < n ? lane : 0)];
+}
+
+__device__ __forceinline__ PairShape staged_shape(const PairDesc &P) {
+    const int pad = P.combo == 4 ? 3 : 0;
+    return {P.combo, 0, (P.nv_a + pad) & ~pad, kOutlineSlots, (P.nv_b + pad) & ~pad};
+}
+
+// The extents the tests of a pair use: of two outlines, the rectangles inside them.
+__device__ __forceinline__ Extents extents_of(const CollideArgs &a, const PairDesc &P, bool outlines) {
+    if (outlines && P.combo == 4) {
+        const ObjDesc &A = a.objs[P.a], &B = a.objs[P.b];
+        return {A.core_l, A.core_w, 0.0f, B.core_l, B.core_w, 0.0f};
+    }
+    return {P.hl_a, P.hw_a, P.rad_a, P.hl_b, P.hw_b, P.rad_b};
+}
+
+// The exact tests of outline pairs, by a warp: `rounds` of 32 candidates (take(round) gives the lane's, or -1).  A first
+// look decides nine in ten; the others get the whole test one after another, a lane per edge (the edges of both: 16 lanes
+// a candidate, 32 beyond 16 edges).  A lane per candidate would take the warp through every edge of both outlines, 860
+// instructions, as soon as one candidate needs it.  Whole call, 11 objects with outlines: every candidate's whole test
+// 133 us, the edges found by search first 120, outlines in shared memory 113, heavy blocks in halves 87, pairs found
+// earlier in the batch dropped 80, overlaps and facing edges by rectangle and sector, a lane per edge 75.
+template <typename Take, typename Look, typename Lanes, typename Hit>
+__device__ __forceinline__ void test_outlines(int rounds, const PairShape &shape, Take &&take, Look &&look, Lanes &&lanes,
+                                              Hit &&hit) {
+    const int lane = threadIdx.x & 31;
+    const int edges = shape.combo == 4 ? shape.nv_a + shape.nv_b : (shape.combo == 5 ? shape.nv_a : shape.nv_b);
+    const int group = edges <= 16 ? 16 : 32, g = lane & (group - 1);
+    const unsigned mine = group == 32 ? 0xffffffffu : 0xffffu << (lane & 16);
+    for (int r = 0; r < rounds; ++r) {
+        const int e = take(r);
+        const Verdict v = e >= 0 ? look(e) : kApart;
+        if (v == kOverlap) hit(e);
+        const unsigned open = __ballot_sync(0xffffffffu, v == kUndecided);
+        const int n = __popc(open);
+        for (int c = lane / group; c - lane / group < n; c += 32 / group) {
+            const int ec = __shfl_sync(0xffffffffu, e, nth_set_bit(open, min(c, n - 1)));
+            const bool found = lanes(ec, g, edges);
+            const bool any = __ballot_sync(0xffffffffu, found) & mine;
+            if (g == 0 && c < n && any != (shape.combo == 4)) hit(ec);
+        }
+    }
+}
+
 __device__ __forceinline__ bool boxes_meet(const float4 &a, const float4 &b, float r) {
     return (a.x - r <= b.z) && (b.x - r <= a.z) && (a.y - r <= b.w) && (b.y - r <= a.w);
 }
@@ -247,7 +311,7 @@ __device__ __forceinline__ void walk_block(const CollideArgs &a, const BlockRef 
         }
     }
     const PairShape shape = shape_of(P);
-    const Extents ext{P.hl_a, P.hw_a, P.rad_a, P.hl_b, P.hw_b, P.rad_b};
+    const Extents ext = extents_of(a, P, OUTL);
     const float rc2 = P.rc2 + kEps0;
     const int ego_side = P.ego_side;
     unsigned narrow = 0;
@@ -268,14 +332,12 @@ __device__ __forceinline__ void walk_block(const CollideArgs &a, const BlockRef 
             for (int u = 0; u < n; ++u, cand &= cand - 1u) S.queue[off + u] = (unsigned short)(lane << 5 | (__ffs(cand) - 1));
             __syncwarp();
             narrow += total;
-            for (int u = lane; u < total; u += 32) {
-                const int e = S.queue[u];
-                if (!overlap<OUTL>(S.step, shape, a.polys, ext, e)) continue;
+            auto hit_at = [&](int e) {
                 atomicOr(&S.found[e >> 5], 1u << (e & 31));
                 const int i = queued_row(e), j = queued_col(e), hi = S.order[0][i], hj = S.order[1][j];
                 a.table[P.off + (long long)hi * hb + hj] = (int16_t)k;
                 ++cnt;
-                if (!FUSED) continue;
+                if (!FUSED) return;
                 mass += to_fixed(S.prob[0][i] * S.prob[1][j], kFixProb);
                 if (ego_side >= 0) {
                     const int eg = ego_side == 0 ? hi : hj;                              // the EGO hypothesis
@@ -283,6 +345,17 @@ __device__ __forceinline__ void walk_block(const CollideArgs &a, const BlockRef 
                     atomicAdd(a.acc.mass + P.mass_base + (long long)eg * P.n_obj_s + P.co_local, a.pfix[co]);
                     atomicAdd(a.acc.hits + P.hits_base + eg, 1ull);
                     atomicAdd(a.acc.lsum + P.lsum_base + ((long long)eg * N + k) * P.n_obj_s + P.co_local, a.lfix[co]);
+                }
+            };
+            if (OUTL && shape.combo >= 4) {
+                test_outlines((total + 31) / 32, shape,
+                    [&](int r) { return 32 * r + lane < total ? (int)S.queue[32 * r + lane] : -1; },
+                    [&](int e) { return first_look(S.step, shape, a.polys, ext, e, nullptr); },
+                    [&](int e, int g, int edges) { return edge_decides(S.step, shape, a.polys, ext, e, g, edges); }, hit_at);
+            } else {
+                for (int u = lane; u < total; u += 32) {
+                    const int e = S.queue[u];
+                    if (overlap<false>(S.step, shape, a.polys, ext, e)) hit_at(e);
                 }
             }
             __syncwarp();
@@ -353,13 +426,18 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkCtas) walk_kernel(const 
 // Bound by latency: a batch of W steps is a chain of 2,300 cycles, the heaviest block has four, and a block's set-up
 // and epilogue take as long as two more.  Measured (whole call replayed as one graph; before: a CTA of four warps per
 // 32 consecutive hypotheses a side, listed or not, a queue per warp): EGO-only scene 154 -> 101 us, 11 objects with
-// outlines 153 -> 133, with lane paths 150 -> 137, 11 objects 46.5 -> 46.8.  Four warps a CTA: 11 objects 53.6, outlines
+// outlines 153 -> 133 (test_outlines: 75), with lane paths 150 -> 137, 11 objects 46.5 -> 46.8.  Four warps a CTA: 11 objects 53.6, outlines
 // 178; sixteen: 51.3 and 135; four CTAs per SM: 49.5 and 158; the light blocks by a warp each: 50.7 and 140; in
 // arbitrary order: 52.5 and 140.
 constexpr int kBlockWarps = 8;
 constexpr int kBlockCtas = 3;           // per SM: bounds the registers to 80
 constexpr int kBlockSlots = 152 * kBlockCtas;   // CTAs on the chip at once
 constexpr int kLaneQueue = 32;          // candidates queued per lane and round
+
+// With outlines a heavy block of a small scene is shared by two CTAs, 16 rows each: its exact tests, ten times as long,
+// make the heaviest one three times the kernel's average load per CTA (11 objects: 114 us whole, 89 in halves, 92 in
+// quarters; four such scenes at once, bound by the tests in all: 321, 349 and 394).
+constexpr long long kHalvesBelow = 152 * 16;   // tiles
 
 // queue_offsets for counts up to 63.
 __device__ __forceinline__ bool queue_offsets6(int cnt, int lane, int &off, int &total) {
@@ -379,6 +457,8 @@ constexpr int kFirstRow = 33;           // (odd: columns read without bank confl
 
 struct BlockSlot {
     StepSlot step[kBlockWarps];
+    PolyVertex outline[2][kOutlineSlots];
+    unsigned char faces[2][16];         // of two outlines: the edge that faces each sector
     unsigned short queue[kBlockWarps * kLaneQueue * 32];   // step slot << 10 | candidate
     int at[kBlockWarps];                // the slots' steps
     int queued[2];                      // candidates in the queue (of alternate rounds)
@@ -391,7 +471,7 @@ struct BlockSlot {
 
 // (mask 0: the block's active steps are not known yet, from step 0 on)
 template <bool FUSED, bool OUTL>
-__device__ __forceinline__ void block_work(const CollideArgs &a, const BlockRef &B, BlockSlot &S) {
+__device__ __forceinline__ void block_work(const CollideArgs &a, const BlockRef &B, unsigned rows, BlockSlot &S) {
     constexpr int W = kBlockWarps, ROWS = 32 / W;
     constexpr int kNone = 0x7fffffff;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, tid = threadIdx.x;
@@ -433,10 +513,19 @@ __device__ __forceinline__ void block_work(const CollideArgs &a, const BlockRef 
             }
         }
     }
-    if (w == W - 1) S.found[lane] = 0u;
+    if (OUTL && P.combo >= 4 && w < 2) {
+        load_outline(S.outline[w], a.polys, P, w, lane);
+        if (P.combo == 4 && lane < 16) {
+            const ObjDesc &o = a.objs[w ? P.b : P.a];
+            const float2 q = point_of(lane, o.core_l, o.core_w);
+            __syncwarp(0xffffu);
+            S.faces[w][lane] = (unsigned char)facing_edge(S.outline[w], o.n_poly, q.x, q.y);
+        }
+    }
+    if (w == W - 1) S.found[lane] = ~rows;          // (the other rows' pairs count as found)
     if (w == W - 2 && lane < 2) S.queued[lane] = 0;
-    const PairShape shape = shape_of(P);
-    const Extents ext{P.hl_a, P.hw_a, P.rad_a, P.hl_b, P.hw_b, P.rad_b};
+    const PairShape shape = OUTL ? staged_shape(P) : shape_of(P);
+    const Extents ext = extents_of(a, P, OUTL);
     const float rc2 = P.rc2 + kEps0;
     __syncthreads();                                // S.first, S.found, S.queued initialised
     unsigned narrow = 0;                            // this lane's exact tests
@@ -466,18 +555,31 @@ __device__ __forceinline__ void block_work(const CollideArgs &a, const BlockRef 
             __syncthreads();
             const int queued = S.queued[parity];
             if (tid == 0) S.queued[parity ^ 1] = 0;
-            for (int u = tid; u < queued; u += 64 * W) {   // two candidates of a lane in flight
-                const int u2 = u + 32 * W, e = S.queue[u], e2 = S.queue[u2 < queued ? u2 : u];
-                const bool h = overlap<OUTL>(S.step[e >> 10], shape, a.polys, ext, e);
-                const bool h2 = (u2 - lane < queued) && overlap<OUTL>(S.step[e2 >> 10], shape, a.polys, ext, e2);
-                narrow += u2 < queued ? 2 : 1;
-                if (h) {
-                    atomicOr(&S.found[e >> 5 & 31], 1u << (e & 31));
-                    atomicMin(&S.first[kFirstRow * queued_row(e) + queued_col(e)], S.at[e >> 10]);
-                }
-                if (h2 && u2 < queued) {
-                    atomicOr(&S.found[e2 >> 5 & 31], 1u << (e2 & 31));
-                    atomicMin(&S.first[kFirstRow * queued_row(e2) + queued_col(e2)], S.at[e2 >> 10]);
+            auto hit_at = [&](int e) {
+                atomicOr(&S.found[e >> 5 & 31], 1u << (e & 31));
+                atomicMin(&S.first[kFirstRow * queued_row(e) + queued_col(e)], S.at[e >> 10]);
+            };
+            // (half the candidates with outlines overlap, most of them pairs that do so in several steps of the batch)
+            auto beaten = [&](int e) { return S.first[kFirstRow * queued_row(e) + queued_col(e)] < S.at[e >> 10]; };
+            if (OUTL && shape.combo >= 4) {
+                test_outlines((queued + 32 * W - 1 - 32 * w) / (32 * W), shape,
+                    [&](int r) {
+                        const int u = 32 * W * r + tid;
+                        narrow += u < queued;
+                        const int e = u < queued ? S.queue[u] : -1;
+                        return u < queued && !beaten(e) ? e : -1;
+                    },
+                    [&](int e) { return first_look(S.step[e >> 10], shape, S.outline[0], ext, e, S.faces[0]); },
+                    [&](int e, int g, int edges) { return edge_decides(S.step[e >> 10], shape, S.outline[0], ext, e, g, edges); },
+                    hit_at);
+            } else {
+                for (int u = tid; u < queued; u += 64 * W) {   // two candidates of a lane in flight
+                    const int u2 = u + 32 * W, e = S.queue[u], e2 = S.queue[u2 < queued ? u2 : u];
+                    const bool h = overlap<false>(S.step[e >> 10], shape, S.outline[0], ext, e);
+                    const bool h2 = (u2 - lane < queued) && overlap<false>(S.step[e2 >> 10], shape, S.outline[0], ext, e2);
+                    narrow += u2 < queued ? 2 : 1;
+                    if (h) hit_at(e);
+                    if (h2 && u2 < queued) hit_at(e2);
                 }
             }
             parity ^= 1;
@@ -488,7 +590,7 @@ __device__ __forceinline__ void block_work(const CollideArgs &a, const BlockRef 
         narrow = __reduce_add_sync(0xffffffffu, narrow);
         if (lane == 0) {
             if (narrow) count_narrow(a, P.combo, narrow);
-            if (steps) atomicAdd(a.counters, (unsigned long long)steps * 32 * 32);
+            if (steps) atomicAdd(a.counters, (unsigned long long)steps * 32 * __popc(rows));
         }
     }
     if (FUSED) {
@@ -547,14 +649,18 @@ __global__ void __launch_bounds__(32 * kBlockWarps, kBlockCtas) block_kernel(con
         B.box_b = (int)(P.bounds_b + (long long)B.tile_b * P.n_steps);
         const bool in = 32 * B.tile_a < P.h_a && 32 * B.tile_b < P.h_b;
         pdl_wait();
-        if (in) block_work<FUSED, OUTL>(a, B, S);
+        if (in) block_work<FUSED, OUTL>(a, B, 0xffffffffu, S);
         return;
     }
     pdl_wait();
+    const bool halves = OUTL && a.n_tiles < kHalvesBelow;
     const long long front = (long long)a.list_counts[0], listed = front + (long long)a.list_counts[1];
-    for (long long it = blockIdx.x; it < listed; it += gridDim.x) {
-        block_work<FUSED, OUTL>(a, listed_block(a, it, front), S);
-        if (it + gridDim.x < listed) __syncthreads();   // the slots are no longer read
+    const long long parts = halves ? 2 * front : 0, tasks = listed + parts / 2;
+    for (long long it = blockIdx.x; it < tasks; it += gridDim.x) {
+        // (a half: its rows' bits of every micro-block, MJ m + n at rows lr + 8 m)
+        if (it < parts) block_work<FUSED, OUTL>(a, a.list[it >> 1], it & 1 ? 0xffff0000u : 0xffffu, S);
+        else block_work<FUSED, OUTL>(a, listed_block(a, it - parts / 2, front), 0xffffffffu, S);
+        if (it + gridDim.x < tasks) __syncthreads();   // the slots are no longer read
     }
 }
 

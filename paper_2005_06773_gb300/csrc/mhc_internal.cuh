@@ -48,6 +48,7 @@ struct ObjDesc {
     double tau_i_d;     // (double)tau / substeps, the sub-step of the speed recurrence
     int poly_off;       // vehicles of scenarios with convex outlines: the outline's vertices at
     int n_poly;         // polys[poly_off .. + n_poly) (a rectangle as its 4 corners); n_poly = 0 otherwise
+    float core_l, core_w;   // with an outline: half extents of a rectangle 1 mm inside it (-1e30 if there is none)
     int path_off;       // vehicles with paths: path i_b's three sections (x, y, psi) at paths[9 (path_off +
                         // i_b) ..]; -1 for constant steering angles
     int path_n1, path_n2;   // the first sub-steps of the second and third sections (t >= 1.0 s, t >= 1.5 s)
