@@ -243,7 +243,7 @@ __device__ __forceinline__ BlockRef listed_block(const CollideArgs &a, long long
 //
 // A block's steps come in order, so the first overlap of a pair is its first collision step: it is stored at once,
 // and the pair's bit in `found` drops its later candidates.  The warps take the listed blocks one after another from
-// a counter, up to kWalkBlocks each.  Without the list (UNLISTED: culling off, or no room for the tile-ordered poses) they take every block
+// a counter, until their CTA has walked kWalkSteps.  Without the list (UNLISTED: culling off, or no room for the tile-ordered poses) they take every block
 // of ascending tiles, strided, and read the pose planes.
 //
 // Bound by instruction issue: about 400 warp instructions per (block, step) item, half of them the sweep.  Measured
@@ -253,7 +253,12 @@ __device__ __forceinline__ BlockRef listed_block(const CollideArgs &a, long long
 // the list is empty 1.73 ms (requests of higher priority then wait for the whole launch).
 constexpr int kWalkWarps = 4;
 constexpr int kWalkCtas = 6;            // per SM: bounds the registers to 80
-constexpr int kWalkBlocks = 16;         // blocks a warp takes before its CTA makes room (for a stream of higher priority)
+constexpr int kWalkBlocks = 16;         // blocks per warp that the grid is sized for (its last CTAs take what is left)
+// Steps after which a CTA makes room for a stream of higher priority (unless it is one of the last).  By steps and for the
+// CTA as a whole: its warps end together.  A small request behind 32 cars in the serving loop is done 0.4 ms after its
+// submission so, 0.9 to 1.2 ms with 16 blocks a warp or 1,024 steps; 32 cars take 2.66 ms, with 96 steps 2.68, with 1,024
+// 2.59; 256 scenarios (collision stage) 6.32, 6.40 and 6.18 ms, 6.33 with 16 blocks a warp.
+constexpr int kWalkSteps = 192;
 
 struct WalkSlot {
     StepSlot step;
@@ -264,7 +269,7 @@ struct WalkSlot {
 };
 
 template <bool FUSED, bool OUTL, bool UNLISTED>
-__device__ __forceinline__ void walk_block(const CollideArgs &a, const BlockRef &B, int lane, WalkSlot &S) {
+__device__ __forceinline__ int walk_block(const CollideArgs &a, const BlockRef &B, int lane, WalkSlot &S) {
     const PairDesc &P = a.pairs[B.pair];               // fields read where used (fewer live registers)
     const int ha = P.h_a, hb = P.h_b, N = P.n_steps;
     const int ia = 32 * B.tile_a + lane, jb = 32 * B.tile_b + lane;   // this lane's positions
@@ -290,7 +295,7 @@ __device__ __forceinline__ void walk_block(const CollideArgs &a, const BlockRef 
         return k0 + b;
     };
     int k = next();
-    if (k < 0) return;
+    if (k < 0) return 0;
     StepPoses cur;
     auto load = [&](int kk) {
         if (UNLISTED) {
@@ -375,7 +380,7 @@ __device__ __forceinline__ void walk_block(const CollideArgs &a, const BlockRef 
         }
         k = kn;
     }
-    if (lane != 0) return;
+    if (lane != 0) return steps;
     if (a.counters) {
         if (narrow) count_narrow(a, P.combo, narrow);
         atomicAdd(a.counters, (unsigned long long)steps * 32 * 32);
@@ -384,6 +389,7 @@ __device__ __forceinline__ void walk_block(const CollideArgs &a, const BlockRef 
         atomicAdd(a.acc.count + P.index, hit_cnt);
         atomicAdd(a.acc.P + P.index, hit_mass);
     }
+    return steps;
 }
 
 template <bool FUSED, bool OUTL, bool UNLISTED>
@@ -406,14 +412,25 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkCtas) walk_kernel(const 
         }
         return;
     }
+    __shared__ int s_steps;                         // steps the CTA has walked
+    if (threadIdx.x == 0) s_steps = 0;
+    __syncthreads();
+    const bool leaves = blockIdx.x + kWalkCtas * 152 < gridDim.x;   // not one of the last: others come after it
     const long long front = (long long)a.list_counts[0], listed = front + (long long)a.list_counts[1];
     unsigned long long taken = 0;
     if (lane == 0) taken = atomicAdd(a.list_counts + 2, 1ull);
-    for (int u = 0; u < kWalkBlocks; ++u) {
+    for (;;) {
         const long long it = (long long)__shfl_sync(0xffffffffu, taken, 0);
         if (it >= listed) return;
-        if (lane == 0 && u + 1 < kWalkBlocks) taken = atomicAdd(a.list_counts + 2, 1ull);   // in flight meanwhile
-        walk_block<FUSED, OUTL, false>(a, listed_block(a, it, front), lane, S);
+        int total = 0;
+        if (lane == 0) {
+            total = *(volatile int *)&s_steps;
+            if (!leaves || total < kWalkSteps) taken = atomicAdd(a.list_counts + 2, 1ull);   // in flight meanwhile
+        }
+        const int steps = walk_block<FUSED, OUTL, false>(a, listed_block(a, it, front), lane, S);
+        total = __shfl_sync(0xffffffffu, total, 0);
+        if (leaves && total >= kWalkSteps) return;
+        if (lane == 0) atomicAdd(&s_steps, steps);
         __syncwarp();
     }
 }
