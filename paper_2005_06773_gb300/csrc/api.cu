@@ -46,17 +46,18 @@ Regime speed_regime(float v0f, float acc, int model, int NK, double tau_i_d) {
         return n;
     };
     Regime g{0, 0, NK, 0};
+    const double per = acc != 0.0f ? 1.0 / dv : 0.0;   // (the guesses need not be exact)
     if (model == MHC_MODEL_KIN) {
         g.low_hi = NK;
     } else if (acc > 0.0f) {
-        g.low_hi = first([&](int n) { return speed(n) >= kVMinD; }, (kVMinD - v0) / dv);
+        g.low_hi = first([&](int n) { return speed(n) >= kVMinD; }, (kVMinD - v0) * per);
     } else if (acc < 0.0f) {
-        g.low_lo = first([&](int n) { return speed(n) < kVMinD; }, (kVMinD - v0) / dv);
+        g.low_lo = first([&](int n) { return speed(n) < kVMinD; }, (kVMinD - v0) * per);
         g.low_hi = NK;
     } else if (v0 < kVMinD) {
         g.low_hi = NK;
     }
-    if (acc < 0.0f) g.n_stop = first([&](int n) { return speed(n + 1) < 0.0; }, -v0 / dv - 1.0);
+    if (acc < 0.0f) g.n_stop = first([&](int n) { return speed(n + 1) < 0.0; }, -v0 * per - 1.0);
     return g;
 }
 
@@ -203,16 +204,18 @@ int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
             return fail(MHC_E_INVALID, where() + "grids too large");
         d.kind = src.kind; d.flags = src.flags; d.n_a = src.n_a; d.n_b = src.n_b; d.h = src.n_a * src.n_b;
         d.grid_off = (int)L.grids.size();
+        bool finite_a = true, finite_b = true, speeds = true;
         for (int q = 0; q < src.n_a; ++q) {
-            if (!finite(src.grid_a[q])) return fail(MHC_E_INVALID, where() + "grid_a not finite");
-            if (src.kind == MHC_PEDESTRIAN && !(src.flags & MHC_PED_ACCEL_GRID) && src.grid_a[q] < 0.f)
-                return fail(MHC_E_INVALID, where() + "pedestrian speeds must be >= 0");
-            L.grids.push_back(src.grid_a[q]);
+            finite_a &= finite(src.grid_a[q]);
+            speeds &= !(src.grid_a[q] < 0.f);
         }
-        for (int q = 0; q < src.n_b; ++q) {
-            if (!finite(src.grid_b[q])) return fail(MHC_E_INVALID, where() + "grid_b not finite");
-            L.grids.push_back(src.grid_b[q]);
-        }
+        for (int q = 0; q < src.n_b; ++q) finite_b &= finite(src.grid_b[q]);
+        if (!finite_a) return fail(MHC_E_INVALID, where() + "grid_a not finite");
+        if (src.kind == MHC_PEDESTRIAN && !(src.flags & MHC_PED_ACCEL_GRID) && !speeds)
+            return fail(MHC_E_INVALID, where() + "pedestrian speeds must be >= 0");
+        if (!finite_b) return fail(MHC_E_INVALID, where() + "grid_b not finite");
+        L.grids.insert(L.grids.end(), src.grid_a, src.grid_a + src.n_a);
+        L.grids.insert(L.grids.end(), src.grid_b, src.grid_b + src.n_b);
         d.traj_off = L.n_traj;
         d.pose_base = L.n_pose;
         L.n_traj += d.h;
@@ -298,9 +301,11 @@ int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
     L.n_mass += (long long)S.h_e * n_obj_s;
     L.n_steps_total += N;
     L.entry0.push_back(L.n_entries);
+    int p_index = 0;
     auto add_pair = [&](int la, int lb) {
-        PairDesc p;
-        std::memset(&p, 0, sizeof p);
+        p_index = (int)L.pairs.size();
+        L.pairs.emplace_back();             // zeroed
+        PairDesc &p = L.pairs.back();
         const int a = obj0 + la, b = obj0 + lb;
         const ObjDesc &A = L.objs[a], &B = L.objs[b];
         p.a = a; p.b = b;
@@ -323,11 +328,10 @@ int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
         p.hits_base = S.e_base;
         p.n_obj_s = n_obj_s;
         p.co_local = p.ego_side == 0 ? lb : (p.ego_side == 1 ? la : 0);
-        p.index = (int)L.pairs.size();
+        p.index = p_index;
         L.n_entries += (long long)A.h * B.h;
         L.n_tiles += pair_tiles(p);
         L.n_kofs += N;
-        L.pairs.push_back(p);
     };
     if ((long long)L.pairs.size() + (long long)n_obj_s * (n_obj_s - 1) / 2 > 0x7fffffffLL)
         return fail(MHC_E_INVALID, "too many object pairs in the batch");
@@ -385,14 +389,13 @@ int build_layout(const mhc_scenario *sc, int n_scen, Layout &L) {
         const float dx = A.x0 - B.x0, dy = A.y0 - B.y0;
         key[p] = {std::sqrt(dx * dx + dy * dy) - A.circ - B.circ, (int)p};
     }
-    std::stable_sort(key.begin(), key.end());
-    L.pairs_c.resize(L.pairs.size());
+    std::sort(key.begin(), key.end());   // (ties by index)
+    L.pairs_c.reserve(L.pairs.size());
     long long tiles = 0;
-    for (size_t q = 0; q < key.size(); ++q) {
-        PairDesc d = L.pairs[key[q].second];
-        d.tile_start = tiles;
-        tiles += pair_tiles(d);
-        L.pairs_c[q] = d;
+    for (const auto &q : key) {
+        L.pairs_c.push_back(L.pairs[q.second]);
+        L.pairs_c.back().tile_start = tiles;
+        tiles += pair_tiles(L.pairs_c.back());
     }
     return MHC_OK;
 }
@@ -616,18 +619,26 @@ int gather_weights(const Layout &L, const float *const *w, std::vector<float> &o
     out.resize((size_t)L.n_traj);
     for (int o = 0; o < L.n_obj; ++o) {
         const ObjDesc &d = L.objs[o];
-        double sum = 0.0;
-        for (int i = 0; i < d.h; ++i) {
-            const float v = w[o] ? w[o][i] : 1.0f;
-            if (!(v >= 0.f) || !finite(v)) {
-                char msg[96];
-                std::snprintf(msg, sizeof msg, "object %d: weights must be finite and non-negative", o);
-                return fail(MHC_E_INVALID, msg);
-            }
-            out[(size_t)d.traj_off + i] = v;
-            sum += v;
+        float *dst = out.data() + d.traj_off;
+        if (!w[o]) {
+            std::fill(dst, dst + d.h, 1.0f);
+            continue;
         }
-        if (!(sum > 0.0)) {
+        // by the bit patterns, so that the loop vectorises: finite and non-negative (or -0), and one above zero
+        unsigned bad = 0u, positive = 0u;
+        for (int i = 0; i < d.h; ++i) {
+            unsigned b;
+            std::memcpy(&b, w[o] + i, 4);
+            bad |= (unsigned)(b > 0x7f7fffffu) & (unsigned)(b != 0x80000000u);
+            positive |= b & 0x7fffffffu;
+        }
+        std::memcpy(dst, w[o], sizeof(float) * (size_t)d.h);
+        if (bad) {
+            char msg[96];
+            std::snprintf(msg, sizeof msg, "object %d: weights must be finite and non-negative", o);
+            return fail(MHC_E_INVALID, msg);
+        }
+        if (!positive) {
             char msg[96];
             std::snprintf(msg, sizeof msg, "object %d: weights sum to zero", o);
             return fail(MHC_E_INVALID, msg);
