@@ -252,7 +252,7 @@ __device__ __forceinline__ BlockRef listed_block(const CollideArgs &a, long long
 // without the list 2.67 and 8.9 ms (a third of the launch was its last warps), with it but with warps that stay until
 // the list is empty 1.73 ms (requests of higher priority then wait for the whole launch).
 constexpr int kWalkWarps = 4;
-constexpr int kWalkCtas = 6;            // per SM: bounds the registers to 80
+constexpr int kWalkCtas = 7;            // per SM: bounds the registers to 72 (256 scenarios, collision stage: 6.00 ms; 5, 6, 8: 6.80, 6.33, 6.17)
 constexpr int kWalkBlocks = 16;         // blocks per warp that the grid is sized for (its last CTAs take what is left)
 // Steps after which a CTA makes room for a stream of higher priority (unless it is one of the last).  By steps and for the
 // CTA as a whole: its warps end together.  A small request behind 32 cars in the serving loop is done 0.4 ms after its
