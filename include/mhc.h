@@ -207,7 +207,7 @@ void mhc_destroy(mhc_ctx *ctx);
  *                 8: as 7 in ascending tiles, the quarter tiles with an active step listed by one warp per
  *                    quarter tile (records in scratch; up to 2^19 quarter tiles, larger scenarios use 7);
  *                 0 (default): the one mhc_autotune chose for the scenario's size class, else 4 for at
- *                 least 64 tiles per SM (160 with outlines), and 7 below that. */
+ *                 least 64 tiles per SM (160 with outlines, 32 where tiles are wide in any order), and 7 below that. */
 #define MHC_OPT_COLLIDE_VARIANT 3
 /*   MHC_OPT_GEN_SCAN  trajectory generation: 1 one warp per hypothesis, its sub-steps in parallel (warp
  *                 scans of the state maps and of the heading / position increments); 0 one thread per

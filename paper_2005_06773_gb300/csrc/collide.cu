@@ -36,6 +36,7 @@
 #include <cstdint>
 
 #include "collide_common.cuh"
+#include "hit_terms.cuh"
 
 namespace mhc {
 namespace {
@@ -1185,8 +1186,9 @@ __global__ void __launch_bounds__(128) items_table_kernel(const CollideArgs a) {
 // ---- block layout (variant 7 without tile-ordered poses): one CTA per 32 x 32 block, its active steps spread over the
 // CTA's warps --
 //
-// Variant 7 runs this kernel where culling is off or the arena has no room for the poses in tile order: there it is the
-// faster of the two (11 objects, culling off: 67 us against 108 for collide_tiles.cu's block kernel reading the planes).
+// Variant 7 runs this kernel where culling is off, the arena has no room for the poses in tile order, or many tiles are
+// wide in any order (wide_tiles): there it is the faster of the two (11 objects, culling off: 67 us against 108 for
+// collide_tiles.cu's block kernel reading the planes; 16 cars of 8 x 28 hypotheses, whole call: 84 against 97).
 //
 // Each CTA owns one 32 x 32 block of hypothesis pairs.  Every warp reads the block's descriptors (before
 // the wait for the previous kernel: they are uploaded data) and decides the block's active steps itself
@@ -1360,14 +1362,44 @@ __device__ __forceinline__ void block_work(const CollideArgs &a, const BlockJob 
     if (FUSED) cp_async_wait();
     __syncthreads();                                // every first hit of the block is in s_first (and the copies)
 
-    // ---- the first hits of this warp's rows, one hit per lane: the table entry and (fused) the risk terms ----
+    // ---- the first hits of this warp's rows: the table entry and (fused) the risk terms, one hit per lane, or summed
+    // over the warp first where hits come crowded (add_hit_terms) or b is the EGO object (then the warp's columns, so that
+    // a line is one EGO hypothesis) ----
     const int r0 = w * ROWS;
-    if (r0 >= rows) return;
-    unsigned hits = 0u;                             // bit u: row r0 + u of this lane's column hit
+    const bool by_col = FUSED && P.ego_side == 1;
+    if (r0 >= (by_col ? cols : rows)) return;
+    unsigned hits = 0u;                             // bit u: this lane's pair in line r0 + u hit
+    int at[ROWS], lo = kNone, hi = 0;
 #pragma unroll
-    for (int u = 0; u < ROWS; ++u)
-        if (r0 + u < rows && col_ok && s_first[32 * (r0 + u) + lane] != kNone) hits |= 1u << u;
-    if (!__ballot_sync(0xffffffffu, hits != 0u)) return;
+    for (int u = 0; u < ROWS; ++u) {
+        at[u] = s_first[by_col ? 32 * lane + r0 + u : 32 * (r0 + u) + lane];
+        if (at[u] == kNone) continue;
+        hits |= 1u << u;
+        lo = min(lo, at[u]);
+        hi = max(hi, at[u]);
+    }
+    const int total = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(hits));
+    if (!total) return;
+    if constexpr (FUSED) {
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (by_col || total >= kHitsPerStep * (hi - lo + 1)) {
+            unsigned long long wt[ROWS] = {};
+            const float p_lane = by_col ? s_prow[lane] : s_pcol[lane];
+#pragma unroll
+            for (int u = 0; u < ROWS; ++u) {
+                if (!(hits >> u & 1u)) continue;
+                const int r = by_col ? lane : r0 + u, c = by_col ? r0 + u : lane;
+                a.table[J.entry0 + (long long)r * hb + c] = (int16_t)at[u];
+                wt[u] = to_fixed((by_col ? s_pcol[c] : s_prow[r]) * p_lane, kFixProb);
+            }
+            const bool ego = P.ego_side >= 0;
+            const int line0 = (by_col ? J.j0 : J.i0) + r0;
+            add_hit_terms<ROWS>(a.acc, P, ego, at, hits, total, wt, [&](int u) { return line0 + u; },
+                                ego ? s_lfix[lane] : 0ull, ego ? s_pfix[lane] : 0ull);
+            return;
+        }
+    }
     // the pair's risk fields in registers (read through the descriptor they would be read again after
     // every atomic)
     const int ego_side = P.ego_side, n_obj_s = P.n_obj_s, co_local = P.co_local, pidx = P.index;

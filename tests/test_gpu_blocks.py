@@ -54,7 +54,8 @@ def _same(a, b):
             assert torch.equal(a[1][k], b[1][k]), k
 
 
-@pytest.mark.parametrize("n_obj,n_a,n_b,n_steps", [(2, 1, 1, 40), (3, 5, 13, 31), (3, 33, 2, 97), (4, 31, 33, 37), (5, 23, 29, 64)])
+@pytest.mark.parametrize("n_obj,n_a,n_b,n_steps", [(2, 1, 1, 40), (3, 5, 13, 31), (3, 33, 2, 97), (4, 31, 33, 37), (5, 23, 29, 64),
+                                                   (4, 31, 33, 9), (4, 19, 17, 70)])
 @pytest.mark.parametrize("ego", [0, 1])
 @pytest.mark.parametrize("crowded", [False, True])
 def test_blocks(mhc, n_obj, n_a, n_b, n_steps, ego, crowded):
