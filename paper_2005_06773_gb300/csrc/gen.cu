@@ -750,7 +750,7 @@ __global__ void __launch_bounds__(128, 6) gen_kernel(const GenArgs a) {
 // table, so the HBM-rate fill overlaps the generation kernel's tail, and the collision kernel stores first
 // hits only.  TILED: the tiles are taken in the objects' tile order (hypothesis_at) and the poses go out once more,
 // 512 bytes per tile and step, so that the walk reads a step of a tile with one 16-byte load per lane: 35 us
-// instead of 15 on the 32-vehicle scene, 0.35 ms instead of 0.11 on the 256-scenario batch (HBM: 52 and 340 MB of
+// instead of 15 on the 32-vehicle scene, 0.28 ms instead of 0.11 on the 256-scenario batch (HBM: 52 and 340 MB of
 // poses read and written), for collision kernels 2.9 and 5.4 ms shorter.
 constexpr int kFillCtas = 152 * 4;
 // Fill CTAs of the generation launch (the rest of each SM integrates).  Two per SM spread the fill's stores
