@@ -700,13 +700,14 @@ int log2_floor(long long v) {
 }
 
 // Whether layout 7 leaves the tile order and the list alone.  With coarse grids or long horizons a tile of 32 hypotheses
-// stays wide in any order (here: its expected side half-way, on average over the hypotheses, from 4.5 m): many steps are
+// stays wide in any order (here: its expected side half-way, on average over the hypotheses, from 9.5 m): many steps are
 // active, few candidates each, and with enough tiles to fill the chip a warp per step without barriers (the kernel of
-// collide.cu) is ahead.  Whole call, listed / that kernel: 16 cars of 8 x 28 hypotheses (1,920 tiles, 17 m) 97 / 84 us, 11
-// objects of 18 x 32 (1,700, 5 m) 136 / 119, of 21 x 21 (1,445, 3 m) 58 / 63, 8 cars of 20 x 12 (448, 15 m) 61 / 70.
+// collide.cu) is ahead.  Whole call, listed / that kernel (six placements each): 16 cars of 8 x 28 hypotheses (1,920 tiles,
+// 16 m) 98-102 / 84-91 us, 11 objects of 18 x 32 (1,700, 10.5 m) 118-150 / 113-150, of 30 x 20 (8.5 m) 106-141 / 110-147, of
+// 21 x 21 (1,445, 5.4 m) 48-65 / 48-67, 24 cars of 10 x 10 (1,104, 9 m) 46-49 / 51-57, 8 cars of 20 x 12 (448, 15 m) 61 / 70.
 // EGO-only pairs come crowded with hits (109 / 140), outlines with long tests: always listed.
 bool wide_tiles(const Layout &L) {
-    return L.polys.empty() && L.n_tiles >= 800 && L.sprawl >= 4.5 * (double)L.n_traj;
+    return L.polys.empty() && L.n_tiles >= 800 && L.sprawl >= 9.5 * (double)L.n_traj;
 }
 
 // The collision layout without tuning.  Large scenes: a warp per active block, in step order; small ones, whose time is
