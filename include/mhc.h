@@ -203,7 +203,7 @@ void mhc_destroy(mhc_ctx *ctx);
  *                    for small scenes (at most 2^22 items and 2^26 table entries; larger ones use 5);
  *                 7: one CTA per 32 x 32 quarter tile with an active step, its active steps spread over the
  *                    CTA's warps; tiles in tile order and listed first, as 4 (every quarter tile of ascending tiles
- *                    without culling or without room for the list);
+ *                    without culling, without room for the list, or for many tiles that are wide in any order);
  *                 8: as 7 in ascending tiles, the quarter tiles with an active step listed by one warp per
  *                    quarter tile (records in scratch; up to 2^19 quarter tiles, larger scenarios use 7);
  *                 0 (default): the one mhc_autotune chose for the scenario's size class, else 4 for at
