@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(32 * kListWarps) block_list_kernel(const Colli
         for (int k0 = 0; k0 < N; k0 += 32) {
             const int k = k0 + lane;
             const bool in = k < N;
-            const float4 far = make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY);   // meets nothing
+            const float4 far = make_float4(INFINITY, INFINITY, -INFINITY, -INFINITY);   // meets no finite box
             const float4 a0 = in ? a.bounds[box_a + k] : far, a1 = in && two_a ? a.bounds[box_a + N + k] : far;
             for (int v = 0; v < run; ++v) {
                 const long long bb = box_b + (long long)(2 * v) * N;
@@ -205,7 +205,9 @@ __global__ void __launch_bounds__(32 * kListWarps) block_list_kernel(const Colli
                 const unsigned m1 = __ballot_sync(0xffffffffu, boxes_meet(a0, b1, r));
                 const unsigned m2 = __ballot_sync(0xffffffffu, boxes_meet(a1, b0, r));
                 const unsigned m3 = __ballot_sync(0xffffffffu, boxes_meet(a1, b1, r));
-                if (mine == u0 + v) {
+                // (a tile past the object's end is never listed: `far` does meet the box of poses that have
+                // overflowed to both infinities)
+                if (mine == u0 + v && (two_a || q < 2) && (two_b || !(q & 1))) {
                     const unsigned m = q < 2 ? (q ? m1 : m0) : (q == 2 ? m2 : m3);
                     if (n == 0) { ref.k0 = k0; ref.mask = m; }
                     n += __popc(m);
