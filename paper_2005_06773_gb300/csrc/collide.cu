@@ -1581,36 +1581,36 @@ cudaError_t launch_fill_table(int16_t *table, long long n, cudaStream_t st, bool
     return launch_kernel(fill_kernel, dim3((unsigned)blocks), dim3(256), 0, st, pdl, table, n);
 }
 
+// Dynamic shared memory of the layouts with a CTA per tile: the staged steps and, fused, the per-step histograms and EGO
+// cells (`steps` up to their limits).
+constexpr size_t step_bytes(size_t base, bool fused, int steps) {
+    return base + (fused && steps <= kFusedHistSteps ? 8 * ((size_t)steps + (steps + 1) / 2) : 0) +
+           (fused && steps <= kFusedCellSteps ? 8 * (size_t)kTile * steps : 0);
+}
+
+// Above the default 48 KiB with the kernels' static part (about 5 KiB): opts in to the most that the layout can need.
+template <typename Kernel>
+cudaError_t allow_steps(Kernel kernel, size_t base, bool fused, size_t smem) {
+    if (smem <= 32 * 1024) return cudaSuccess;
+    return allow_shared(kernel, std::max(step_bytes(base, fused, kFusedHistSteps), step_bytes(base, fused, kFusedCellSteps)));
+}
+
 template <int THREADS, int MI, int MJ, int CH, bool FUSED, bool OUTL>
 cudaError_t launch_variant(const CollideArgs &a, cudaStream_t st, bool pdl) {
-    size_t smem = (size_t)CH * kTile * (2 * sizeof(float4) + 2 * sizeof(float2));
-    if (FUSED) {
-        if (a.max_steps <= kFusedHistSteps) smem += 8 * ((size_t)a.max_steps + (a.max_steps + 1) / 2);
-        if (a.max_steps <= kFusedCellSteps) smem += 8 * (size_t)kTile * a.max_steps;
-    }
-    if (smem > 32 * 1024) {   // dynamic + static (about 5 KiB) above the default 48 KiB needs the opt-in
-        cudaError_t e = cudaFuncSetAttribute(collide_kernel<THREADS, MI, MJ, CH, FUSED, OUTL>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    return launch_kernel(collide_kernel<THREADS, MI, MJ, CH, FUSED, OUTL>, dim3((unsigned)a.n_tiles), dim3(THREADS),
-                         smem, st, pdl, a);
+    constexpr size_t base = (size_t)CH * kTile * (2 * sizeof(float4) + 2 * sizeof(float2));
+    const size_t smem = step_bytes(base, FUSED, a.max_steps);
+    const auto kernel = collide_kernel<THREADS, MI, MJ, CH, FUSED, OUTL>;
+    const cudaError_t e = allow_steps(kernel, base, FUSED, smem);
+    return e != cudaSuccess ? e : launch_kernel(kernel, dim3((unsigned)a.n_tiles), dim3(THREADS), smem, st, pdl, a);
 }
 
 template <int WARPS, int CH, bool FUSED, bool OUTL>
 cudaError_t launch_warp_variant(const CollideArgs &a, cudaStream_t st, bool pdl) {
-    size_t smem = (size_t)CH * kTile * (2 * sizeof(float4) + 2 * sizeof(float2)) + sizeof(int) * kTile * kTile;
-    if (FUSED) {
-        if (a.max_steps <= kFusedHistSteps) smem += 8 * ((size_t)a.max_steps + (a.max_steps + 1) / 2);
-        if (a.max_steps <= kFusedCellSteps) smem += 8 * (size_t)kTile * a.max_steps;
-    }
-    if (smem > 32 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(collide_warp_kernel<WARPS, CH, FUSED, OUTL>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    return launch_kernel(collide_warp_kernel<WARPS, CH, FUSED, OUTL>, dim3((unsigned)a.n_tiles), dim3(WARPS * 32),
-                         smem, st, pdl, a);
+    constexpr size_t base = (size_t)CH * kTile * (2 * sizeof(float4) + 2 * sizeof(float2)) + sizeof(int) * kTile * kTile;
+    const size_t smem = step_bytes(base, FUSED, a.max_steps);
+    const auto kernel = collide_warp_kernel<WARPS, CH, FUSED, OUTL>;
+    const cudaError_t e = allow_steps(kernel, base, FUSED, smem);
+    return e != cudaSuccess ? e : launch_kernel(kernel, dim3((unsigned)a.n_tiles), dim3(WARPS * 32), smem, st, pdl, a);
 }
 
 template <bool FUSED, bool OUTL>

@@ -212,6 +212,14 @@ __device__ __forceinline__ void pdl_start() {
 // memory per CTA) after the copy kernel (none) ran one CTA per SM to its end, 7.4 ms instead of 1.8 on 256 scenarios.
 constexpr int kCarveout = 58;
 
+// Opts a kernel in to `most` bytes of dynamic shared memory, the most that any of its launches asks for: the limit is
+// the function's, for every thread and context of the process, so that one set to the present call's bytes could be
+// lowered by a shorter call between another thread's opt-in and its launch, which then failed.
+template <typename... KArgs>
+inline cudaError_t allow_shared(void (*kernel)(KArgs...), size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // kernel<<<grid, block, smem, st>>>(args...), with programmatic stream serialization when pdl is set.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

@@ -166,9 +166,9 @@ template <bool HIST>
 cudaError_t launch_scan(const RiskArgs &a, cudaStream_t st, bool pdl) {
     const long long ctas = (a.n_tiles * kScanUnits<HIST> + kScanWarps - 1) / kScanWarps;
     if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
-    const size_t smem = HIST ? sizeof(unsigned) * 4 * kScanWarps * (size_t)a.max_steps : 0;
+    const size_t per_step = HIST ? sizeof(unsigned) * 4 * kScanWarps : 0, smem = per_step * (size_t)a.max_steps;
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(scan_kernel<HIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_shared(scan_kernel<HIST>, per_step * kScanHistSteps);
         if (e != cudaSuccess) return e;
     }
     return launch_kernel(scan_kernel<HIST>, dim3((unsigned)ctas), dim3(32 * kScanWarps), smem, st, pdl, a);
