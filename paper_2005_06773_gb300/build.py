@@ -33,7 +33,8 @@ def sources():
 
 
 def _deps():
-    return sources() + glob.glob(os.path.join(SRC_DIR, "*.cuh")) + [os.path.join(ROOT, "include", "mhc.h")]
+    headers = glob.glob(os.path.join(SRC_DIR, "*.cuh")) + glob.glob(os.path.join(SRC_DIR, "*.h"))
+    return sources() + headers + [os.path.join(ROOT, "include", "mhc.h")]
 
 
 def up_to_date() -> bool:
