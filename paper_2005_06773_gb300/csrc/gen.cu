@@ -12,6 +12,7 @@
 
 #include "mhc_internal.cuh"
 #include "prepare.cuh"
+#include "quotient.h"
 
 namespace mhc {
 namespace {
@@ -172,17 +173,6 @@ constexpr float kCtrlTp = 0.5f;       // s: prediction time of the centre of gra
 constexpr float kDeltaMax = 0.5f;     // rad
 constexpr float kDeltaRate = 0.5f;    // rad/s
 constexpr float kPi = 3.14159265358979f;
-
-// a / b, correctly rounded, with y = 1 / b correctly rounded: Markstein's quotient iteration (P. Markstein, Computation
-// of elementary functions on the IBM RISC System/6000 processor, 1990): the first correction leaves q within one unit in
-// the last place, the second, with its exact remainder, rounds it.  Small |a| (a remainder may be subnormal; the sign of
-// a zero) take the division.
-__device__ __forceinline__ float quotient(float a, float b, float y) {
-    float q = a * y;
-    q = fmaf(fmaf(-q, b, a), y, q);
-    q = fmaf(fmaf(-q, b, a), y, q);
-    return fabsf(a) > 1e-20f ? q : a / b;
-}
 
 struct PathConst {                     // of one hypothesis
     float acc, dv, v0, ti, hti2, lr, L, inv_L, k11, k12, k21, k22, kb1u, kb2u, stop_den, step_max;
