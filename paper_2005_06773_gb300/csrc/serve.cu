@@ -488,19 +488,21 @@ int mhc_submit(mhc_ctx *ctx, const mhc_scenario *scen, const float *const *traj_
     if (int r = gather_weights(L, traj_weights, wcheck)) return r;
     Request *r = new Request();
     r->objs.assign(scen->objects, scen->objects + scen->n_objects);
-    r->arrays.reserve(3 * scen->n_objects);
+    r->arrays.reserve(5 * scen->n_objects);
+    auto copied = [&](const float *v, size_t n) -> const float * {
+        if (!v || !n) return nullptr;
+        r->arrays.emplace_back(v, v + n);
+        return r->arrays.back().data();
+    };
     r->weights.resize(scen->n_objects);
     for (int o = 0; o < scen->n_objects; ++o) {
         mhc_object &d = r->objs[o];
         const mhc_object &s = scen->objects[o];
-        r->arrays.emplace_back(s.grid_a, s.grid_a + s.n_a);
-        d.grid_a = r->arrays.back().data();
-        r->arrays.emplace_back(s.grid_b, s.grid_b + s.n_b);
-        d.grid_b = r->arrays.back().data();
-        if (s.veh_params) {
-            r->arrays.emplace_back(s.veh_params, s.veh_params + 6);
-            d.veh_params = r->arrays.back().data();
-        }
+        d.grid_a = copied(s.grid_a, s.n_a);
+        d.grid_b = copied(s.grid_b, s.n_b);
+        d.veh_params = copied(s.veh_params, 6);
+        d.vertices = copied(s.vertices, 2 * (size_t)s.n_vertices);
+        d.paths = copied(s.paths, 9 * (size_t)s.n_b);
         if (traj_weights && traj_weights[o]) {
             r->weights[o].assign(traj_weights[o], traj_weights[o] + (size_t)s.n_a * s.n_b);
             r->has_w = true;
