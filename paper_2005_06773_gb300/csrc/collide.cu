@@ -7,7 +7,8 @@
 //         earliest hit kept with a shared atomicMin;
 //   3     a CTA of 4 warps per tile, each warp testing whole steps;
 //   4     one warp per 32 x 32 block with an active step, the objects' hypotheses in a compact order
-//         (collide_tiles.cu; the large-scene default);
+//         (collide_tiles.cu; the large-scene default); without that order, one warp per 64 x 64 tile on large
+//         scenes of rectangles and discs;
 //   5     one warp per 32 x 32 quarter tile (1-warp CTAs) walking the active steps in ascending order: a
 //         register mask remembers the pairs that already hit, so only first hits are stored and later
 //         candidates of those pairs cost nothing; the warp stages its own poses with the next step's loads in
@@ -34,6 +35,7 @@
 // whole (result-preserving).
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "collide_common.cuh"
 #include "hit_terms.cuh"
@@ -645,22 +647,28 @@ __global__ void __launch_bounds__(WARPS * 32) collide_warp_kernel(const CollideA
     }
 }
 
-// Warp-per-block layout: each warp owns one 32 x 32 block of hypothesis pairs (a quarter of a 64 x 64 tile) and walks
-// its active steps in ascending order on its own (no CTA barrier anywhere).  A lane holds a 4 x 8 micro-block (rows
-// lr + 8 m, columns lc + 4 n, lr = lane / 4, lc = lane % 4) and a register mask of its pairs that have already hit:
-// because the steps come in order, the first narrow-phase hit of a pair is its first collision step, it is stored at
-// once, and later candidates of that pair are dropped before any further work.  The warp stages each step's poses in
-// its own shared-memory slot; the next active step's poses are loaded into registers while the current step is
-// tested.  Activity (culling against the blocks' bounding boxes) is decided 32 steps at a time with one ballot.
-// Fused risk terms are added per hit with global atomics; the per-step histogram terms of one step's hits are summed
-// over the warp first.  One block (warp task gw) walked by the calling warp; pa_s .. s_new are the warp's own slots.
-template <bool FUSED, bool OUTL>
+// Warp-per-block layouts in ascending tiles: each warp owns one TE x TE block of hypothesis pairs (one 32 x 32 quarter
+// of a 64 x 64 tile: layout 5; the whole of it: layout 4 on large scenes without its list) and walks its active steps
+// in ascending order on its own (no CTA barrier anywhere).  A lane holds an MI x MJ micro-block (rows lr + 8 m, columns lc + 4 n, lr = lane / 4,
+// lc = lane % 4; 8 x 16 for TE = 64, 4 x 8 for TE = 32) and a register mask of its pairs that have
+// already hit: because the steps come in order, the first narrow-phase hit of a pair is its first
+// collision step, it is stored at once, and later candidates of that pair are dropped before any further
+// work.  The warp stages each step's poses in its own shared-memory slot; the next active step's poses
+// are loaded into registers while the current step is tested.  Activity (culling against the blocks'
+// bounding boxes) is decided 32 steps at a time with one ballot.  Fused risk terms are added per hit with
+// global atomics; the per-step histogram terms of one step's hits are summed over the warp first.
+// One TE x TE block (warp task gw) walked by the calling warp; pa_s .. s_new are the warp's own slots.
+template <int TE, bool FUSED, bool OUTL>
 __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, int lane, float4 *pa_s, float4 *pb_s,
                                            float2 *ra_s, float2 *rb_s, float *prob_s) {
-    constexpr int MI = 4, MJ = 8;                 // micro-block of a lane
-    const long long g = gw >> 2;                  // the 64 x 64 tile
+    static_assert(TE == 64 || TE == 32, "block edge");
+    constexpr int MI = TE / 8, MJ = TE / 4;       // micro-block of a lane
+    constexpr int SUB = kTile / TE;               // blocks per tile edge
+    using Word = std::conditional_t<TE == 64, unsigned long long, unsigned>;   // the micro-block's pairs in WORDS words
+    constexpr int BITS = 8 * (int)sizeof(Word), WORDS = MI * MJ / BITS;
+    const long long g = gw / (SUB * SUB);                 // the 64 x 64 tile
     if (g >= a.n_tiles) return;
-    const int quarter = (int)(gw & 3);
+    const int quarter = (int)(gw - g * (SUB * SUB));
     const int lo = pair_of_tile(a, g);
     const PairDesc &P = a.pairs[lo];   // fields read where used (fewer live registers)
     const PairShape shape = shape_of(P);
@@ -668,26 +676,32 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
     const ObjDesc &B = a.objs[P.b];
     const int t = (int)(g - P.tile_start);          // < tiles_a x tiles_b <= n_tiles < 2^31
     const int ta = t / P.tiles_b, tb = t - ta * P.tiles_b;
-    const int i0 = (ta * 2 + (quarter >> 1)) * 32, j0 = (tb * 2 + (quarter & 1)) * 32;
-    const int rows = min(32, A.h - i0), cols = min(32, B.h - j0);
+    const int ba_idx = ta * SUB + quarter / SUB, bb_idx = tb * SUB + quarter % SUB;   // blocks along a, b
+    const int i0 = ba_idx * TE, j0 = bb_idx * TE;
+    const int rows = min(TE, A.h - i0), cols = min(TE, B.h - j0);
     if (rows <= 0 || cols <= 0) return;                    // a quarter past a ragged edge
     const int lr = lane >> 2, lc = lane & 3;
     const int N = P.n_steps;
+    const int na = (rows + kBoundTile - 1) / kBoundTile, nb = (cols + kBoundTile - 1) / kBoundTile;
     const float4 *bA0 = a.bounds + A.bounds_base + (long long)(i0 / kBoundTile) * N;
     const float4 *bB0 = a.bounds + B.bounds_base + (long long)(j0 / kBoundTile) * N;
     const float la = A.hl, wa = A.hw, ra = A.rad, lb = B.hl, wb = B.hw, rb = B.rad;
     const float rc2 = P.rc2 + kEps0;
     const float ka = 0.5f * (1.0f - kEps);
     const float r_cull = P.r_cull;
-    if (a.fill_blocks) {   // this block's table entries start as -1 (coalesced 64-byte row stores)
+    if (TE == 32 && a.fill_blocks) {   // this block's table entries start as -1 (coalesced 64-byte row stores)
         int16_t *row = a.table + P.off + (long long)i0 * B.h + j0;
         for (int r = 0; r < rows; ++r, row += B.h)
             for (int c = lane; c < cols; c += 32) row[c] = (int16_t)-1;
         __syncwarp();      // the fill is ordered before this warp's first-hit stores
     }
     if (FUSED) {   // the block's probabilities, read at every first hit (kept off the hit path's latency)
-        prob_s[lane] = lane < rows ? a.probf[A.traj_off + i0 + lane] : 0.0f;
-        prob_s[32 + lane] = lane < cols ? a.probf[B.traj_off + j0 + lane] : 0.0f;
+#pragma unroll
+        for (int u = 0; u < TE / 32; ++u) {
+            const int r = lane + 32 * u;
+            prob_s[r] = r < rows ? a.probf[A.traj_off + i0 + r] : 0.0f;
+            prob_s[TE + r] = r < cols ? a.probf[B.traj_off + j0 + r] : 0.0f;
+        }
     }
 
     // activity of the 32 steps from k0 (one ballot)
@@ -695,7 +709,16 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
         const int k = k0 + lane;
         bool act = k < N;
         if (act && a.cull) {
-            const float4 ba = bA0[k], bb = bB0[k];
+            float4 ba = bA0[k];
+            if (na > 1) {
+                const float4 q = bA0[N + k];
+                ba = make_float4(fminf(ba.x, q.x), fminf(ba.y, q.y), fmaxf(ba.z, q.z), fmaxf(ba.w, q.w));
+            }
+            float4 bb = bB0[k];
+            if (nb > 1) {
+                const float4 q = bB0[N + k];
+                bb = make_float4(fminf(bb.x, q.x), fminf(bb.y, q.y), fmaxf(bb.z, q.z), fmaxf(bb.w, q.w));
+            }
             act = (ba.x - r_cull <= bb.z) && (bb.x - r_cull <= ba.z) && (ba.y - r_cull <= bb.w) &&
                   (bb.y - r_cull <= ba.w);
         }
@@ -714,14 +737,17 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
         }
         return k0 + __ffs(m) - 1;
     };
-    // this lane's share of a step's poses: row `lane` of A, then column `lane` of B
-    float px[2], py[2], pc[2], ps[2];
+    // this lane's share of a step's poses: rows lane (+ 32) of A, then columns lane (+ 32) of B
+    constexpr int NU = 2 * (TE / 32);
+    float px[NU], py[NU], pc[NU], ps[NU];
     auto load_step = [&](int k) {
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const bool isA = u == 0, ok = isA ? lane < rows : lane < cols;
-            const long long idx = isA ? A.pose_base + (long long)k * A.h + i0 + lane
-                                      : B.pose_base + (long long)k * B.h + j0 + lane;
+        for (int u = 0; u < NU; ++u) {
+            const bool isA = u < NU / 2;
+            const int r = lane + 32 * (isA ? u : u - NU / 2);
+            const bool ok = isA ? r < rows : r < cols;
+            const long long idx = isA ? A.pose_base + (long long)k * A.h + i0 + r
+                                      : B.pose_base + (long long)k * B.h + j0 + r;
             px[u] = ok ? __ldg(a.x + idx) : (isA ? kFar : -kFar);
             py[u] = ok ? __ldg(a.y + idx) : 0.0f;
             pc[u] = ok ? __ldg(a.c + idx) : 1.0f;
@@ -729,7 +755,7 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
         }
     };
 
-    unsigned found = 0u;                // bit MJ m + n of the lane's pairs
+    Word found[WORDS] = {};             // bit MJ m + n of the lane's pairs
     unsigned long long narrow = 0, hit_cnt = 0, hit_mass = 0;
     int active_steps = 0;
     int k = next_step(-1);
@@ -737,14 +763,16 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
     while (k >= 0) {
         __syncwarp();                       // the previous step's slot is no longer read
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < NU; ++u) {
+            const bool isA = u < NU / 2;
+            const int r = lane + 32 * (isA ? u : u - NU / 2);
             const float q2 = fmaf(px[u], px[u], py[u] * py[u]);
-            if (u == 0) {
-                pa_s[lane] = make_float4(px[u], py[u], ka * q2, 0.0f);
-                ra_s[lane] = make_float2(pc[u], ps[u]);
+            if (isA) {
+                pa_s[r] = make_float4(px[u], py[u], ka * q2, 0.0f);
+                ra_s[r] = make_float2(pc[u], ps[u]);
             } else {
-                pb_s[lane] = make_float4(px[u], py[u], 0.5f * fmaf(1.0f - kEps, q2, -rc2), 0.0f);
-                rb_s[lane] = make_float2(pc[u], ps[u]);
+                pb_s[r] = make_float4(px[u], py[u], 0.5f * fmaf(1.0f - kEps, q2, -rc2), 0.0f);
+                rb_s[r] = make_float2(pc[u], ps[u]);
             }
         }
         __syncwarp();
@@ -758,46 +786,52 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
             const float4 q = pa_s[lr + 8 * m];
             ax[m] = q.x; ay[m] = q.y; ah[m] = q.z;
         }
-        unsigned cand = 0u;
+        Word cand[WORDS] = {}, any = 0;
 #pragma unroll
         for (int n = 0; n < MJ; ++n) {
             const float4 qb = pb_s[lc + 4 * n];
 #pragma unroll
             for (int m = 0; m < MI; ++m)
-                if (fmaf(ax[m], qb.x, fmaf(ay[m], qb.y, -qb.z)) >= ah[m]) cand |= 1u << (MJ * m + n);
+                if (fmaf(ax[m], qb.x, fmaf(ay[m], qb.y, -qb.z)) >= ah[m])
+                    cand[(MJ * m + n) / BITS] |= (Word)1 << (MJ * m + n) % BITS;
         }
-        cand &= ~found;
-        if (__ballot_sync(0xffffffffu, cand != 0u)) {
+#pragma unroll
+        for (int h = 0; h < WORDS; ++h) any |= cand[h] &= ~found[h];
+        if (__ballot_sync(0xffffffffu, any != 0)) {
             bool any_hit = false;
             unsigned long long step_cnt = 0, step_mass = 0;
             // each lane tests the candidates of its own micro-block (a loop as long as the lane with the most;
             // measured faster than compacting them into a warp queue first), so a hit sets its own mask bit
-            while (cand) {
-                const int bit = __ffs(cand) - 1;
-                cand &= cand - 1u;
-                ++narrow;
-                const int m = bit / MJ, n = bit % MJ;
-                const int i = lr + 8 * m, j = lc + 4 * n;
-                const float4 qa4 = pa_s[i], qb4 = pb_s[j];
-                const float dx = qb4.x - qa4.x, dy = qb4.y - qa4.y;
-                const float2 qa = ra_s[i], qb = rb_s[j];
-                if (!narrow_hit<OUTL>(shape, a.polys, dx, dy, qa, qb, la, wa, lb, wb, ra, rb)) continue;
-                any_hit = true;
-                found |= 1u << bit;
-                a.table[P.off + (long long)(i0 + i) * B.h + j0 + j] = (int16_t)k;
-                if (FUSED) {
-                    const float pa_ = prob_s[i], pb_ = prob_s[32 + j];
-                    const unsigned long long w = to_fixed(pa_ * pb_, kFixProb);
-                    ++step_cnt;
-                    step_mass += w;
-                    if (P.ego_side >= 0) {
-                        const int e = P.ego_side == 0 ? i0 + i : j0 + j;     // the EGO hypothesis
-                        const float pco = P.ego_side == 0 ? pb_ : pa_;       // the CO hypothesis
-                        atomicAdd(a.acc.mass + P.mass_base + (long long)e * P.n_obj_s + P.co_local,
-                                  to_fixed(pco, kFixProb));
-                        atomicAdd(a.acc.hits + P.hits_base + e, 1ull);
-                        atomicAdd(a.acc.lsum + P.lsum_base + ((long long)e * N + k) * P.n_obj_s + P.co_local,
-                                  to_fixed(neg_log_survival(pco), kFixLog));
+#pragma unroll
+            for (int h = 0; h < WORDS; ++h) {
+                Word cm = cand[h];
+                while (cm) {
+                    const int low = (TE == 64 ? __ffsll((long long)cm) : __ffs((int)cm)) - 1, bit = BITS * h + low;
+                    cm &= cm - 1;
+                    ++narrow;
+                    const int m = bit / MJ, n = bit % MJ;
+                    const int i = lr + 8 * m, j = lc + 4 * n;
+                    const float4 qa4 = pa_s[i], qb4 = pb_s[j];
+                    const float dx = qb4.x - qa4.x, dy = qb4.y - qa4.y;
+                    const float2 qa = ra_s[i], qb = rb_s[j];
+                    if (!narrow_hit<OUTL>(shape, a.polys, dx, dy, qa, qb, la, wa, lb, wb, ra, rb)) continue;
+                    any_hit = true;
+                    found[h] |= (Word)1 << low;
+                    a.table[P.off + (long long)(i0 + i) * B.h + j0 + j] = (int16_t)k;
+                    if (FUSED) {
+                        const float pa_ = prob_s[i], pb_ = prob_s[TE + j];
+                        const unsigned long long w = to_fixed(pa_ * pb_, kFixProb);
+                        ++step_cnt;
+                        step_mass += w;
+                        if (P.ego_side >= 0) {
+                            const int e = P.ego_side == 0 ? i0 + i : j0 + j;     // the EGO hypothesis
+                            const float pco = P.ego_side == 0 ? pb_ : pa_;       // the CO hypothesis
+                            atomicAdd(a.acc.mass + P.mass_base + (long long)e * P.n_obj_s + P.co_local,
+                                      to_fixed(pco, kFixProb));
+                            atomicAdd(a.acc.hits + P.hits_base + e, 1ull);
+                            atomicAdd(a.acc.lsum + P.lsum_base + ((long long)e * N + k) * P.n_obj_s + P.co_local,
+                                      to_fixed(neg_log_survival(pco), kFixLog));
+                        }
                     }
                 }
             }
@@ -825,7 +859,7 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
     }
     if (a.counters && lane == 0) {
         if (narrow) count_narrow(a, P.combo, narrow);
-        if (active_steps) atomicAdd(a.counters, (unsigned long long)active_steps * 32 * 32);
+        if (active_steps) atomicAdd(a.counters, (unsigned long long)active_steps * TE * TE);
     }
     if (FUSED && lane == 0 && hit_cnt) {
         atomicAdd(a.acc.count + P.index, hit_cnt);
@@ -833,16 +867,21 @@ __device__ __forceinline__ void tile_block(const CollideArgs &a, long long gw, i
     }
 }
 
-// Each warp (a CTA of its own: a finished warp frees its slot at once) takes blocks gw = blockIdx.x, then every
-// gridDim.x further (a grid smaller than the work, max_ctas, leaves SM room to other streams).
-template <bool FUSED, bool OUTL>
-__global__ void __launch_bounds__(32, 24) collide_tile_kernel(const CollideArgs a) {
+// The warp-per-block layouts: each warp takes blocks gw = blockIdx.x * WARPS + warp, then every
+// gridDim.x * WARPS further (a grid smaller than the work, max_ctas, leaves SM room to other streams).
+template <int WARPS, int TE, bool FUSED, bool OUTL>
+__global__ void __launch_bounds__(WARPS * 32, (TE == 64 ? 16 : 24) / WARPS) collide_tile_kernel(const CollideArgs a) {
     pdl_start();
-    __shared__ float4 s_pa[32], s_pb[32];         // x, y, h
-    __shared__ float2 s_ra[32], s_rb[32];         // c, s
-    __shared__ float s_prob[FUSED ? 64 : 1];      // fused: the block's row and column probabilities
-    for (long long gw = blockIdx.x; gw < a.n_tiles * 4; gw += gridDim.x)
-        tile_block<FUSED, OUTL>(a, gw, threadIdx.x, s_pa, s_pb, s_ra, s_rb, s_prob);
+    constexpr int SUB = kTile / TE;
+    __shared__ float4 s_pa[WARPS][TE];            // x, y, h_a
+    __shared__ float4 s_pb[WARPS][TE];            // x, y, h_b
+    __shared__ float2 s_ra[WARPS][TE];            // c, s
+    __shared__ float2 s_rb[WARPS][TE];
+    __shared__ float s_prob[WARPS][FUSED ? 2 * TE : 1];    // fused: the block's row and column probabilities
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long total = a.n_tiles * (SUB * SUB);
+    for (long long gw = (long long)blockIdx.x * WARPS + warp; gw < total; gw += (long long)gridDim.x * WARPS)
+        tile_block<TE, FUSED, OUTL>(a, gw, lane, s_pa[warp], s_pb[warp], s_ra[warp], s_rb[warp], s_prob[warp]);
 }
 
 // ---- step-item layout (variant 6): the active (block, step) pairs of a small scene in parallel ----------
@@ -1613,12 +1652,22 @@ cudaError_t launch_warp_variant(const CollideArgs &a, cudaStream_t st, bool pdl)
     return e != cudaSuccess ? e : launch_kernel(kernel, dim3((unsigned)a.n_tiles), dim3(WARPS * 32), smem, st, pdl, a);
 }
 
-template <bool FUSED, bool OUTL>
+// Layout 4 without its list (culling off, or no room for the poses in tile order): from this many tiles a warp walks a
+// whole tile, whose sweep costs less per pair.  Whole call, the walk over every 32 x 32 block (collide_tiles.cu) / this
+// kernel: culling off, 7,168 tiles 541 / 655 us, 11,154 542 / 401, 21,384 992 / 587, 67,584 5031 / 2895; culling on, no
+// room, 152,064 tiles 1529 / 1266, 507,904 7611 / 5739.  With outlines the walk's test of them decides (culling off,
+// 11,154 tiles 885 / 2160 us, 48,000 5487 / 6398), so this kernel has none.
+constexpr long long kWholeTiles = 152 * 64;
+
+template <int WARPS, int TE, bool FUSED, bool OUTL>
 cudaError_t launch_tile_variant(const CollideArgs &a, cudaStream_t st, bool pdl) {
-    long long blocks = a.n_tiles * 4;
+    constexpr int SUB = kTile / TE;
+    const long long warps = a.n_tiles * SUB * SUB;
+    long long blocks = (warps + WARPS - 1) / WARPS;
     if (a.max_ctas > 0 && blocks > a.max_ctas) blocks = a.max_ctas;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    return launch_kernel(collide_tile_kernel<FUSED, OUTL>, dim3((unsigned)blocks), dim3(32), 0, st, pdl, a);
+    return launch_kernel(collide_tile_kernel<WARPS, TE, FUSED, OUTL>, dim3((unsigned)blocks), dim3(WARPS * 32), 0,
+                         st, pdl, a);
 }
 
 template <bool OUTL>
@@ -1660,9 +1709,13 @@ cudaError_t launch_collide_t(const CollideArgs &a, cudaStream_t st, bool pdl) {
         return a.probf ? launch_kernel(block_kernel<kBlockWarps, true, OUTL>, grid, block, 0, st, pdl, a)
                        : launch_kernel(block_kernel<kBlockWarps, false, OUTL>, grid, block, 0, st, pdl, a);
     }
+    if constexpr (!OUTL) {
+        if (a.variant == 4 && !a.tile_poses && a.n_tiles >= kWholeTiles)
+            return a.probf ? launch_tile_variant<4, 64, true, OUTL>(a, st, pdl) : launch_tile_variant<4, 64, false, OUTL>(a, st, pdl);
+    }
     if (a.variant == 4) return launch_tiles(a, st, pdl);
     if (a.variant == 5)   // one warp per CTA: a finished warp frees its slot at once (small, uneven grids)
-        return a.probf ? launch_tile_variant<true, OUTL>(a, st, pdl) : launch_tile_variant<false, OUTL>(a, st, pdl);
+        return a.probf ? launch_tile_variant<1, 32, true, OUTL>(a, st, pdl) : launch_tile_variant<1, 32, false, OUTL>(a, st, pdl);
     // variant 1: 4 x 4 micro-tiles with 256 threads (8 warps share each tile's tests); variant 2: 8 x 8 with
     // 64 threads; variant 3: one warp per step (8 x 16 lanes).  The caller picks one (autotuned per size).
     const bool many = a.variant == 2;

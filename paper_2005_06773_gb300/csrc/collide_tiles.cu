@@ -4,7 +4,8 @@
 // The bounds kernel has written each object's poses tile by tile (CollideArgs::tile_poses: 32 poses of one step side
 // by side, in the compact order of hypothesis_at) together with the boxes around them, so that a block's active
 // steps are few and a step's poses are one 16-byte load per lane and side.  Without that array (culling off, or an
-// arena sized to the least) layout 4's kernel takes ascending tiles and reads the pose planes.
+// arena sized to the least) layout 4's kernel takes ascending tiles and reads the pose planes (large scenes without
+// outlines: the kernel of whole tiles in collide.cu).
 //
 // A step of a block, by one warp: the 32 + 32 poses go to a shared slot, the broad phase runs on a 4 x 8 micro-block
 // per lane (rows lr + 8 m, columns lc + 4 n), and the candidates are queued and tested one per lane.  Compact tiles
@@ -245,8 +246,9 @@ __device__ __forceinline__ BlockRef listed_block(const CollideArgs &a, long long
 //
 // A block's steps come in order, so the first overlap of a pair is its first collision step: it is stored at once,
 // and the pair's bit in `found` drops its later candidates.  The warps take the listed blocks one after another from
-// a counter, until their CTA has walked kWalkSteps.  Without the list (UNLISTED: culling off, or no room for the tile-ordered poses) they take every block
-// of ascending tiles, strided, and read the pose planes.
+// a counter, until their CTA has walked kWalkSteps. 
+// Without the list (UNLISTED: culling off, or no room for the tile-ordered poses; kWholeTiles in collide.cu) they take
+// every block of ascending tiles, strided, and read the pose planes.
 //
 // Bound by instruction issue: about 400 warp instructions per (block, step) item, half of them the sweep.  Measured
 // (collision stage, listing included): 32 cars of 2048 hypotheses 1.79 ms, 256 uneven scenarios 6.3 ms; a warp per 64 x
