@@ -622,7 +622,6 @@ int make_risk_args(const Layout &L, const DevDesc &D, Bump &bump, const int16_t 
     r.objs = D.objs; r.pairs = D.pairs; r.scens = D.scens;
     r.n_pairs = (int)L.pairs.size(); r.n_obj = L.n_obj; r.n_scen = L.n_scen;
     r.h_e = L.h_e; r.n_kofs = L.n_kofs; r.n_steps_total = L.n_steps_total; r.max_steps = L.max_steps;
-    for (const ScenDesc &S : L.scens) r.max_h_e = std::max<long long>(r.max_h_e, S.h_e);
     r.n_cells = L.n_lsum;
     r.n_tiles = L.n_tiles; r.table = table;
     r.weights = D.weights;

@@ -350,7 +350,7 @@ struct RiskArgs {
     const ScenDesc *scens;
     int n_pairs, n_obj, n_scen;
     long long h_e;                 // EGO hypotheses over all scenarios
-    long long max_h_e, n_cells;    // the most of one scenario; cells [EGO hypothesis][step][object] in all
+    long long n_cells;             // cells [EGO hypothesis][step][object] in all
     long long n_kofs, n_steps_total;   // per-pair step entries, per-scenario step entries
     int max_steps;                 // the longest horizon of the batch
     int convert_in_walk;           // set by launch_risk_tail: the last CTA of the EGO walk (1) or of the attribution (2)
