@@ -195,7 +195,8 @@ void mhc_destroy(mhc_ctx *ctx);
  *                 3: 4 warps per tile, each warp testing whole steps (8 x 16 micro-tiles per lane);
  *                 4: the 32 x 32 blocks with an active step listed first, then one warp per listed block walking its
  *                    steps in order (pairs that already hit dropped from later steps, first hits stored at once); the
- *                    hypotheses are tiled in a compact order of each object's grid, so that few blocks come close;
+ *                    hypotheses are tiled in a compact order of each object's grid, so that few blocks come close (ascending
+ *                    tiles without culling or without room for the list: large scenes one warp per 64 x 64 tile);
  *                 5: one warp per 32 x 32 quarter tile of ascending hypotheses walking its steps in order (4 x 8
  *                    micro-tiles, culling per quarter);
  *                 6: every active (quarter tile, step) an item, all tested in parallel by persistent warps (a
@@ -203,11 +204,11 @@ void mhc_destroy(mhc_ctx *ctx);
  *                    for small scenes (at most 2^22 items and 2^26 table entries; larger ones use 5);
  *                 7: one CTA per 32 x 32 quarter tile with an active step, its active steps spread over the
  *                    CTA's warps; tiles in tile order and listed first, as 4 (every quarter tile of ascending tiles
- *                    without culling, without room for the list, or for many tiles that are wide in any order);
+ *                    without culling or without room for the list);
  *                 8: as 7 in ascending tiles, the quarter tiles with an active step listed by one warp per
  *                    quarter tile (records in scratch; up to 2^19 quarter tiles, larger scenarios use 7);
  *                 0 (default): the one mhc_autotune chose for the scenario's size class, else 4 for at
- *                 least 64 tiles per SM (160 with outlines, 32 where tiles are wide in any order), and 7 below that. */
+ *                 least 64 tiles per SM (160 with outlines), and 7 below that. */
 #define MHC_OPT_COLLIDE_VARIANT 3
 /*   MHC_OPT_GEN_SCAN  trajectory generation: 1 one warp per hypothesis, its sub-steps in parallel (warp
  *                 scans of the state maps and of the heading / position increments); 0 one thread per

@@ -184,11 +184,6 @@ int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
         L.n_traj += d.h;
         L.n_pose += (long long)d.h * N;
         d.tile_base = L.n_tiles32;
-        if (sc->pair_mode == MHC_ALL_PAIRS) {
-            double along_a, along_b;
-            neighbour_distance(src, 0.5 * N * sc->tau, along_a, along_b);
-            L.sprawl += d.h * std::sqrt(32.0 * along_a * along_b);
-        }
         d.n_tiles32 = (d.h + kBoundTile - 1) / kBoundTile;
         if ((long long)L.n_tiles32 + d.n_tiles32 > 0x7fffffffLL) return fail(MHC_E_INVALID, "too many hypotheses in the batch");
         L.n_tiles32 += d.n_tiles32;
@@ -661,25 +656,16 @@ int log2_floor(long long v) {
     return r;
 }
 
-// Whether layout 7 leaves the tile order and the list alone.  With coarse grids or long horizons a tile of 32 hypotheses
-// stays wide in any order (here: its expected side half-way, on average over the hypotheses, from 9.5 m): many steps are
-// active, few candidates each, and with enough tiles to fill the chip a warp per step without barriers (the kernel of
-// collide.cu) is ahead.  Whole call, listed / that kernel (six placements each): 16 cars of 8 x 28 hypotheses (1,920 tiles,
-// 16 m) 98-102 / 84-91 us, 11 objects of 18 x 32 (1,700, 10.5 m) 118-150 / 113-150, of 30 x 20 (8.5 m) 106-141 / 110-147, of
-// 21 x 21 (1,445, 5.4 m) 48-65 / 48-67, 24 cars of 10 x 10 (1,104, 9 m) 46-49 / 51-57, 8 cars of 20 x 12 (448, 15 m) 61 / 70.
-// EGO-only pairs come crowded with hits (109 / 140), outlines with long tests: always listed.
-bool wide_tiles(const Layout &L) {
-    return L.polys.empty() && L.n_tiles >= 800 && L.sprawl >= 9.5 * (double)L.n_traj;
-}
-
 // The collision layout without tuning.  Large scenes: a warp per active block, in step order; small ones, whose time is
 // the closest pairs' step chains: a CTA per block, its steps spread over the warps.  The line by the number of tiles
 // (whole replayed step, layout 4 / 7): 11-object scenes in batches, 5,780 tiles 171 / 137 us, 8,670 212 / 195, 10,115 231 /
 // 227, 11,560 242 / 253; uneven scenes 3,950 177 / 128, 10,899 232 / 259.  Outlines, whose tests are ten times as long:
-// 11,560 tiles 922 / 518, 17,340 1089 / 802.  Wide tiles, for which layout 7 is the kernel of collide.cu: from 32 tiles per
-// SM (19 scenes of 25 x 8 hypotheses in the serving loop: 0.92 ms with 64).
+// 11,560 tiles 922 / 518, 17,340 1089 / 802.  How wide the tiles are does not move the line, nor is the kernel of ascending
+// tiles in collide.cu better where they are: over 130 scenes of 8 to 28 objects (200 to 9,700 tiles, tiles of 2 to 60 m side
+// half-way) layout 7 takes 0.67 to 1.17 of that kernel's time, 0.94 on average, with no relation to the width (correlation
+// of the logarithms -0.02); ten scenes of 5,000 to 9,500 tiles 0.71 to 0.89 of layout 4's.
 int default_variant(const mhc_ctx *ctx, const Layout &L) {
-    return L.n_tiles >= (L.polys.empty() ? (wide_tiles(L) ? 32LL : 64LL) : 160LL) * ctx->n_sm ? 4 : 7;
+    return L.n_tiles >= (L.polys.empty() ? 64LL : 160LL) * ctx->n_sm ? 4 : 7;
 }
 
 // Collision configuration for a scenario: the forced variant, else the tuned one of its size class, else the
@@ -795,11 +781,10 @@ int launch_all(mhc_ctx *ctx, const Layout &L, const DevDesc &D, Bump &bump, cons
         if (!bounds) return fail(MHC_E_NOMEM, "arena too small for tile bounds");
         CollideArgs c{};
         // poses in tile order for layouts 4 and 7 (and the list of active blocks); without room for them (an
-        // arena sized to the least) or without culling, they take the blocks of ascending tiles and read the planes.
-        // So does layout 7 for many tiles that sprawl all the same (wide_tiles)
+        // arena sized to the least) or without culling, they take the blocks of ascending tiles and read the planes
         float4 *tile_poses = nullptr;
         int *tile_order = nullptr;
-        if ((variant == 4 || (variant == 7 && !wide_tiles(L))) && cull && L.n_tiles > 0) {
+        if ((variant == 4 || variant == 7) && cull && L.n_tiles > 0) {
             tile_poses = static_cast<float4 *>(bump.take(sizeof(float4) * 32 * (size_t)L.n_bounds));
             if (tile_poses) tile_order = static_cast<int *>(bump.take(sizeof(int) * 32 * (size_t)L.n_tiles32));
             if (tile_order) {

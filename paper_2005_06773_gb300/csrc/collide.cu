@@ -1225,9 +1225,8 @@ __global__ void __launch_bounds__(128) items_table_kernel(const CollideArgs a) {
 // ---- block layout (variant 7 without tile-ordered poses): one CTA per 32 x 32 block, its active steps spread over the
 // CTA's warps --
 //
-// Variant 7 runs this kernel where culling is off, the arena has no room for the poses in tile order, or many tiles are
-// wide in any order (wide_tiles): there it is the faster of the two (11 objects, culling off: 67 us against 108 for
-// collide_tiles.cu's block kernel reading the planes; 16 cars of 8 x 28 hypotheses, whole call: 84 against 97).
+// Variant 7 runs this kernel where culling is off or the arena has no room for the poses in tile order: there it is the
+// faster of the two (11 objects, culling off: 67 us against 108 for collide_tiles.cu's block kernel reading the planes).
 //
 // Each CTA owns one 32 x 32 block of hypothesis pairs.  Every warp reads the block's descriptors (before
 // the wait for the previous kernel: they are uploaded data) and decides the block's active steps itself

@@ -246,7 +246,7 @@ __device__ __forceinline__ BlockRef listed_block(const CollideArgs &a, long long
 //
 // A block's steps come in order, so the first overlap of a pair is its first collision step: it is stored at once,
 // and the pair's bit in `found` drops its later candidates.  The warps take the listed blocks one after another from
-// a counter, until their CTA has walked kWalkSteps. 
+// a counter, until their CTA has walked kWalkSteps.
 // Without the list (UNLISTED: culling off, or no room for the tile-ordered poses; kWholeTiles in collide.cu) they take
 // every block of ascending tiles, strided, and read the pose planes.
 //

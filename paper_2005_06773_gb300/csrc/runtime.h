@@ -56,7 +56,6 @@ inline bool finite(float v) { return std::isfinite(v); }
 // kernels read.  Objects, pairs, hypotheses, poses, table entries and per-step outputs of the scenarios
 // are concatenated in batch order; each descriptor carries its scenario's horizon and accumulator bases.
 struct Layout {
-    double sprawl = 0.0;           // sum over the hypotheses of all-pairs scenarios: side of their tile half-way (wide_tiles)
     int n_obj = 0, n_scen = 0, max_steps = 0;
     std::vector<ObjDesc> objs;
     std::vector<PairDesc> pairs;
