@@ -263,6 +263,8 @@ int append_scenario(const mhc_scenario *sc, int si, bool batch, Layout &L) {
     L.n_lsum += (long long)S.h_e * N * n_obj_s;
     L.n_mass += (long long)S.h_e * n_obj_s;
     L.n_steps_total += N;
+    S.attr_base = (int)L.n_attr;
+    L.n_attr += (S.h_e + kAttrHyps - 1) / kAttrHyps;
     L.entry0.push_back(L.n_entries);
     int p_index = 0;
     auto add_pair = [&](int la, int lb) {
@@ -618,6 +620,7 @@ int make_risk_args(const Layout &L, const DevDesc &D, Bump &bump, const int16_t 
     r.n_pairs = (int)L.pairs.size(); r.n_obj = L.n_obj; r.n_scen = L.n_scen;
     r.h_e = L.h_e; r.n_kofs = L.n_kofs; r.n_steps_total = L.n_steps_total; r.max_steps = L.max_steps;
     r.n_cells = L.n_lsum;
+    r.attr_ctas = L.n_attr;
     r.n_tiles = L.n_tiles; r.table = table;
     r.weights = D.weights;
     r.prob = static_cast<double *>(bump.take(sizeof(double) * (size_t)L.n_traj));

@@ -272,29 +272,33 @@ __device__ __forceinline__ void for_each_candidate(unsigned cand, int lane, Fn &
     }
 }
 
-// The pair of tile g: the last pair (in the order of a.pairs) whose first tile is <= g.  A 64-way
-// search by the whole warp (every lane must call it with the same g): each round the lanes probe 64
-// evenly spaced pairs at once (two each) and keep the span between the last probe <= g and the next, so up
-// to 64 pairs take one round of loads and 4,096 two (a binary search is a chain of log2 n dependent loads).
-template <typename Args>
-__device__ __forceinline__ int pair_of_tile(const Args &a, long long g) {
+// The last i in [0, n) with le(i), which holds for 0 and up to some entry of an ascending array.  A 64-way search by the
+// whole warp (every lane must call it for the same array and value): each round the lanes probe 64 evenly spaced entries
+// at once (two each) and keep the span between the last probe that holds and the next, so up to 64 entries take one
+// round of loads and 4,096 two (a binary search is a chain of log2 n dependent loads).
+template <typename Le>
+__device__ __forceinline__ int last_where(int n, Le &&le) {
     const int lane = threadIdx.x & 31;
-    int lo = 0, hi = a.n_pairs - 1;
-    while (lo < hi) {   // 64 probes per round (two per lane): a scene of up to 64 pairs in one round of loads
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
         const long long span = hi - lo + 1;
-        const bool le0 = a.pairs[lo + (int)(span * (2 * lane) / 64)].tile_start <= g;
-        const bool le1 = a.pairs[lo + (int)(span * (2 * lane + 1) / 64)].tile_start <= g;
-        const unsigned long long m = (unsigned long long)__ballot_sync(0xffffffffu, le0) |
-                                     (unsigned long long)__ballot_sync(0xffffffffu, le1) << 32;
-        // probe q = 2 lane + (0 | 1) sits at bit lane + 32 (q & 1); probe 0 always holds: pairs[lo] <= g
-        const unsigned even = (unsigned)m, odd = (unsigned)(m >> 32);
-        const int le = 31 - __clz(even), lo2 = odd ? 31 - __clz(odd) : -1;   // last true even / odd probe
-        const int L = 2 * lo2 + 1 > 2 * le ? 2 * lo2 + 1 : 2 * le;           // the true probes form a prefix
+        const bool le0 = le(lo + (int)(span * (2 * lane) / 64));
+        const bool le1 = le(lo + (int)(span * (2 * lane + 1) / 64));
+        // probe q = 2 lane + (0 | 1); probe 0 always holds
+        const unsigned even = __ballot_sync(0xffffffffu, le0), odd = __ballot_sync(0xffffffffu, le1);
+        const int last0 = 31 - __clz(even), last1 = odd ? 31 - __clz(odd) : -1;   // last true even / odd probe
+        const int L = 2 * last1 + 1 > 2 * last0 ? 2 * last1 + 1 : 2 * last0;      // the true probes form a prefix
         const int nlo = lo + (int)(span * L / 64);
         hi = L == 63 ? hi : lo + (int)(span * (L + 1) / 64) - 1;
         lo = nlo;
     }
     return lo;
+}
+
+// The pair of tile g: the last pair (in the order of a.pairs) whose first tile is <= g (every lane with the same g).
+template <typename Args>
+__device__ __forceinline__ int pair_of_tile(const Args &a, long long g) {
+    return last_where(a.n_pairs, [&](int p) { return a.pairs[p].tile_start <= g; });
 }
 
 // Asynchronous 4- and 8-byte copies global -> shared (both addresses aligned to the size); cp_async_wait()

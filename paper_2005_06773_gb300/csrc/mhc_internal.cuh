@@ -110,12 +110,14 @@ struct PairDesc {
     float hl_a, hw_a, rad_a, hl_b, hw_b, rad_b;   // half extents, disc radii
 };
 
+constexpr int kAttrHyps = 16;   // EGO hypotheses per CTA of the attribution kernel
+
 // Per-scenario descriptor of a batch (device; risk stage).
 struct ScenDesc {
     int ego;                  // global object index of the EGO object
     int n_obj, n_steps, h_e;
     int obj0;                 // global index of the scenario's first object
-    int pad_;
+    int attr_base;            // the scenario's first CTA of the attribution kernel (kAttrHyps EGO hypotheses each)
     long long e_base;         // first global EGO hypothesis (per-EGO-hypothesis outputs, hits)
     long long lsum_base, mass_base;
     long long step_base;      // the scenario's n_steps entries of attr_step
@@ -350,7 +352,8 @@ struct RiskArgs {
     const ScenDesc *scens;
     int n_pairs, n_obj, n_scen;
     long long h_e;                 // EGO hypotheses over all scenarios
-    long long n_cells;             // cells [EGO hypothesis][step][object] in all
+    long long n_cells, attr_ctas;  // cells [EGO hypothesis][step][object] in all; CTAs of the attribution kernel
+    int attr_rows;                 // set by launch_risk_tail: the rows that those CTAs' order goes along
     long long n_kofs, n_steps_total;   // per-pair step entries, per-scenario step entries
     int max_steps;                 // the longest horizon of the batch
     int convert_in_walk;           // set by launch_risk_tail: the last CTA of the EGO walk (1) or of the attribution (2)

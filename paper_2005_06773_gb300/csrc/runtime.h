@@ -76,7 +76,7 @@ struct Layout {
     int n_gen_scan_objs = 0;                         // objects those warps cover
     int n_gen_warps = 0;                             // generation warps in all
     long long n_traj = 0, n_pose = 0, n_entries = 0, n_tiles = 0, n_bounds = 0;
-    long long h_e = 0, n_kofs = 0, n_steps_total = 0, n_lsum = 0, n_mass = 0;
+    long long h_e = 0, n_kofs = 0, n_steps_total = 0, n_lsum = 0, n_mass = 0, n_attr = 0;
     int n_tiles32 = 0;
 };
 

@@ -1,5 +1,5 @@
-"""The attribution kernel on batches of very unequal scenes: its CTAs take 16 EGO hypotheses of the batch in turn, so one
-may span many small scenes.  Results bit for bit those of each scene alone (few cells: summed by the walk itself), and
+"""The attribution kernel on batches of very unequal scenes: its CTAs take 16 EGO hypotheses of a scene each, the
+scenes in turn.  Results bit for bit those of each scene alone (few cells: summed by the walk itself), and
 a large scene among thousands of small ones costs no more than both apart."""
 import dataclasses
 
