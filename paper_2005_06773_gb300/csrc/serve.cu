@@ -228,11 +228,15 @@ Batch *build_batch(Server *S, std::vector<Request *> &take) {
 // puts the requests back).
 bool admit_batch(Server *S, Batch *b, std::vector<Request *> &take) {
     if (!pool_alloc(S->pool, b->res_bytes, &b->res_off)) { b->res_bytes = 0; return false; }
-    b->scr_held = pool_alloc(S->pool, b->scr_bytes, &b->scr_off);
-    if (!b->scr_held && b->scr_least < b->scr_bytes) {
-        b->scr_bytes = b->scr_least;
-        b->scr_held = pool_alloc(S->pool, b->scr_bytes, &b->scr_off);
+    // room for the poses in tile order only where it keeps nobody out: every queued request and one more batch like this
+    // still fit.  Else the collision kernels read the planes (32 vehicles: 5.7 ms instead of 2.8)
+    if (b->scr_least < b->scr_bytes) {
+        size_t others = b->res_bytes + b->scr_least;
+        for (const Request *r : S->q_small) others += r->bytes;
+        for (const Request *r : S->q_large) others += r->bytes;
+        if (pool_largest(S->pool) < b->scr_bytes + others) b->scr_bytes = b->scr_least;
     }
+    b->scr_held = pool_alloc(S->pool, b->scr_bytes, &b->scr_off);
     if (!b->scr_held) {
         pool_free(S->pool, b->res_off);
         b->res_bytes = 0;
