@@ -456,14 +456,13 @@ __global__ void __launch_bounds__(32 * kWalkWarps, kWalkCtas) walk_kernel(const 
 constexpr int kBlockWarps = 8;
 constexpr int kBlockCtas = 3;           // per SM: bounds the registers to 80
 constexpr int kBlockSlots = 152 * kBlockCtas;   // CTAs on the chip at once
-constexpr int kLaneQueue = 32;          // candidates queued per lane and round
 
 // With outlines a heavy block of a small scene is shared by two CTAs, 16 rows each: its exact tests, ten times as long,
 // make the heaviest one three times the kernel's average load per CTA (11 objects: 114 us whole, 89 in halves, 92 in
 // quarters; four such scenes at once, bound by the tests in all: 321, 349 and 394).
 constexpr long long kHalvesBelow = 152 * 16;   // tiles
 
-// queue_offsets for counts up to 63.
+// queue_offsets for counts up to 32.
 __device__ __forceinline__ bool queue_offsets6(int cnt, int lane, int &off, int &total) {
     if (!__any_sync(0xffffffffu, cnt > 15)) return queue_offsets(cnt, lane, off, total);
     const unsigned lt = (1u << lane) - 1u;
@@ -483,9 +482,9 @@ struct BlockSlot {
     StepSlot step[kBlockWarps];
     PolyVertex outline[2][kOutlineSlots];
     unsigned char faces[2][16];         // of two outlines: the edge that faces each sector
-    unsigned short queue[kBlockWarps * kLaneQueue * 32];   // step slot << 10 | candidate
+    unsigned short queue[kBlockWarps * 32 * 32];   // step slot << 10 | candidate: room for every pair of every slot
     int at[kBlockWarps];                // the slots' steps
-    int queued[2];                      // candidates in the queue (of alternate rounds)
+    int queued[2];                      // candidates in the queue (of alternate batches)
     int first[32 * kFirstRow];          // first overlapping step of pair (i, j) at kFirstRow i + j
     unsigned found[32];                 // [lane] micro-block pairs that overlapped in an earlier batch
     int order[2][32];                   // hypotheses of the rows and columns
@@ -566,49 +565,45 @@ __device__ __forceinline__ void block_work(const CollideArgs &a, const BlockRef 
         }
         k = mine();
         if (k >= 0) load(k);                        // in flight while the candidates are tested
-        bool more;
-        do {                                        // (a second round only where a lane has over 15 candidates)
-            const int n = min(__popc(cand), kLaneQueue);
-            int off, total, at = 0;
-            if (queue_offsets6(n, lane, off, total)) {
-                if (lane == 0) at = atomicAdd(&S.queued[parity], total);
-                off += __shfl_sync(0xffffffffu, at, 0);
-                for (int u = 0; u < n; ++u, cand &= cand - 1u)
-                    S.queue[off + u] = (unsigned short)(w << 10 | lane << 5 | (__ffs(cand) - 1));
+        int off, total, at = 0;
+        if (queue_offsets6(__popc(cand), lane, off, total)) {
+            if (lane == 0) at = atomicAdd(&S.queued[parity], total);
+            off += __shfl_sync(0xffffffffu, at, 0);
+            for (; cand; cand &= cand - 1u, ++off)
+                S.queue[off] = (unsigned short)(w << 10 | lane << 5 | (__ffs(cand) - 1));
+        }
+        __syncthreads();
+        const int queued = S.queued[parity];
+        if (tid == 0) S.queued[parity ^ 1] = 0;
+        auto hit_at = [&](int e) {
+            atomicOr(&S.found[e >> 5 & 31], 1u << (e & 31));
+            atomicMin(&S.first[kFirstRow * queued_row(e) + queued_col(e)], S.at[e >> 10]);
+        };
+        // (half the candidates with outlines overlap, most of them pairs that do so in several steps of the batch)
+        auto beaten = [&](int e) { return S.first[kFirstRow * queued_row(e) + queued_col(e)] < S.at[e >> 10]; };
+        if (OUTL && shape.combo >= 4) {
+            test_outlines((queued + 32 * W - 1 - 32 * w) / (32 * W), shape,
+                [&](int r) {
+                    const int u = 32 * W * r + tid;
+                    narrow += u < queued;
+                    const int e = u < queued ? S.queue[u] : -1;
+                    return u < queued && !beaten(e) ? e : -1;
+                },
+                [&](int e) { return first_look(S.step[e >> 10], shape, S.outline[0], ext, e, S.faces[0]); },
+                [&](int e, int g, int edges) { return edge_decides(S.step[e >> 10], shape, S.outline[0], ext, e, g, edges); },
+                hit_at);
+        } else {
+            for (int u = tid; u < queued; u += 64 * W) {   // two candidates of a lane in flight
+                const int u2 = u + 32 * W, e = S.queue[u], e2 = S.queue[u2 < queued ? u2 : u];
+                const bool h = overlap<false>(S.step[e >> 10], shape, S.outline[0], ext, e);
+                const bool h2 = (u2 - lane < queued) && overlap<false>(S.step[e2 >> 10], shape, S.outline[0], ext, e2);
+                narrow += u2 < queued ? 2 : 1;
+                if (h) hit_at(e);
+                if (h2 && u2 < queued) hit_at(e2);
             }
-            __syncthreads();
-            const int queued = S.queued[parity];
-            if (tid == 0) S.queued[parity ^ 1] = 0;
-            auto hit_at = [&](int e) {
-                atomicOr(&S.found[e >> 5 & 31], 1u << (e & 31));
-                atomicMin(&S.first[kFirstRow * queued_row(e) + queued_col(e)], S.at[e >> 10]);
-            };
-            // (half the candidates with outlines overlap, most of them pairs that do so in several steps of the batch)
-            auto beaten = [&](int e) { return S.first[kFirstRow * queued_row(e) + queued_col(e)] < S.at[e >> 10]; };
-            if (OUTL && shape.combo >= 4) {
-                test_outlines((queued + 32 * W - 1 - 32 * w) / (32 * W), shape,
-                    [&](int r) {
-                        const int u = 32 * W * r + tid;
-                        narrow += u < queued;
-                        const int e = u < queued ? S.queue[u] : -1;
-                        return u < queued && !beaten(e) ? e : -1;
-                    },
-                    [&](int e) { return first_look(S.step[e >> 10], shape, S.outline[0], ext, e, S.faces[0]); },
-                    [&](int e, int g, int edges) { return edge_decides(S.step[e >> 10], shape, S.outline[0], ext, e, g, edges); },
-                    hit_at);
-            } else {
-                for (int u = tid; u < queued; u += 64 * W) {   // two candidates of a lane in flight
-                    const int u2 = u + 32 * W, e = S.queue[u], e2 = S.queue[u2 < queued ? u2 : u];
-                    const bool h = overlap<false>(S.step[e >> 10], shape, S.outline[0], ext, e);
-                    const bool h2 = (u2 - lane < queued) && overlap<false>(S.step[e2 >> 10], shape, S.outline[0], ext, e2);
-                    narrow += u2 < queued ? 2 : 1;
-                    if (h) hit_at(e);
-                    if (h2 && u2 < queued) hit_at(e2);
-                }
-            }
-            parity ^= 1;
-            more = __syncthreads_or(cand != 0u);
-        } while (more);
+        }
+        parity ^= 1;
+        __syncthreads();
     }
     if (a.counters) {
         narrow = __reduce_add_sync(0xffffffffu, narrow);
