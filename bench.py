@@ -65,9 +65,10 @@ def mean_vertices(sc) -> float:
     return sum(nv) / len(nv) if nv else 0.0
 # the kernel behind each collision layout (MHC_OPT_COLLIDE_VARIANT)
 COLLIDE_KERNELS = {1: "collide_kernel<256, 4, 4, 16>", 2: "collide_kernel<64, 8, 8, 8>", 3: "collide_warp_kernel<4, 8>",
-                   4: "collide_tile_kernel<4, 64>", 5: "collide_tile_kernel<1, 32>",
+                   4: "block_list_kernel + walk_kernel (per-launch figures average the two)", 5: "collide_tile_kernel<1, 32>",
                    6: "items_list_kernel + items_kernel + items_table_kernel (per-launch figures average the three)",
-                   7: "block_kernel<4>", 8: "block_list_kernel + block_rec_kernel<4> (per-launch figures average the two)"}
+                   7: "block_list_kernel + block_kernel (per-launch figures average the two)",
+                   8: "plane_list_kernel + plane_rec_kernel<4> (per-launch figures average the two)"}
 
 
 def parse():

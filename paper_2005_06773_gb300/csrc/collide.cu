@@ -16,9 +16,10 @@
 //   6     step items: (32 x 32 block, active step) pairs listed by one kernel and taken in any order by a
 //         persistent kernel that keeps each pair's earliest step with a global atomicMin; a third kernel
 //         writes the int16 table (and the fused risk terms) for the blocks with active steps;
-//   7     one 128-thread CTA per 32 x 32 block, the block's active steps spread over its four warps, first
-//         hits kept in shared memory (the small-scene default);
-//   8     as 7 for the blocks with an active step only, listed first by one warp per block.
+//   7     one CTA per 32 x 32 block with an active step, in the compact order of 4 (collide_tiles.cu; the
+//         small-scene default); without that order, one 128-thread CTA per block of ascending tiles, its active
+//         steps spread over its four warps, first hits kept in shared memory;
+//   8     the latter for the blocks with an active step only, listed first by one warp per block.
 // The table is -1 outside first hits: a fill kernel (or fill CTAs of the generation or bounds launch) writes
 // it first, or variant 5 writes its own blocks (small tables) and variant 6 its active blocks.
 //
@@ -1253,7 +1254,7 @@ __global__ void __launch_bounds__(128) items_table_kernel(const CollideArgs a) {
 // Four warps per block and a register bound of six CTAs per SM (80 registers): on the 11-object scene the
 // collision stage took 37.8 us so, 39.0 us at eight CTAs per SM (64 registers, small spills), 52-58 us
 // with two or eight warps per block.
-constexpr int kBlockWarps = MHC_BLOCK_WARPS;
+constexpr int kPlaneWarps = MHC_BLOCK_WARPS;
 constexpr int kBlockMinCtas = MHC_BLOCK_MIN_CTAS;
 
 // What the block layouts need of one 32 x 32 block: the pair, the table origin (entry (i, j) at
@@ -1282,7 +1283,7 @@ __device__ __forceinline__ unsigned block_chunk_mask(const CollideArgs &a, const
 // The work of one block with an active step, by the whole CTA (k0 / mask: the first chunk of 32 steps with
 // an active step and its active steps).  The table's -1s are written beforehand; this stores first hits.
 template <int W, bool FUSED, bool OUTL>
-__device__ __forceinline__ void block_work(const CollideArgs &a, const BlockJob &J, int k0, unsigned mask,
+__device__ __forceinline__ void plane_block_work(const CollideArgs &a, const BlockJob &J, int k0, unsigned mask,
                                            float4 (*s_pa)[32], float4 (*s_pb)[32], float2 (*s_ra)[32],
                                            float2 (*s_rb)[32], int *s_first, float *s_prow, float *s_pcol,
                                            unsigned long long *s_lfix, unsigned long long *s_pfix) {
@@ -1510,7 +1511,7 @@ __device__ __forceinline__ BlockJob block_job(const CollideArgs &a, long long gw
 // shared memory, were measured at 57 us against 39 us on the 11-object scene).  Every warp reads the block's
 // descriptors before the wait for the previous kernel (uploaded data) and decides the activity itself.
 template <int W, bool FUSED, bool OUTL>
-__global__ void __launch_bounds__(W * 32, kBlockMinCtas) block_kernel(const CollideArgs a) {
+__global__ void __launch_bounds__(W * 32, kBlockMinCtas) plane_block_kernel(const CollideArgs a) {
     static_assert(W == 1 || W == 2 || W == 4 || W == 8, "warps per block");
     pdl_trigger();
     __shared__ float4 s_pa[W][32], s_pb[W][32];     // x, y, h
@@ -1528,7 +1529,7 @@ __global__ void __launch_bounds__(W * 32, kBlockMinCtas) block_kernel(const Coll
         mask = block_chunk_mask(a, J, k0);
     }
     if (!mask) return;                              // the block never comes close: its entries keep the -1
-    block_work<W, FUSED, OUTL>(a, J, k0, mask, s_pa, s_pb, s_ra, s_rb, s_first, s_prow, s_pcol, s_lfix, s_pfix);
+    plane_block_work<W, FUSED, OUTL>(a, J, k0, mask, s_pa, s_pb, s_ra, s_rb, s_first, s_prow, s_pcol, s_lfix, s_pfix);
 }
 
 // ---- block-list layout (variant 8): active blocks listed first, then a CTA per listed block ----
@@ -1539,7 +1540,7 @@ __global__ void __launch_bounds__(W * 32, kBlockMinCtas) block_kernel(const Coll
 // active block; the block kernel then reads one record per CTA (a single load) and does the work of
 // variant 7.  Both CTAs past the list's end and the listing's empty blocks end at once; the table's -1s are
 // written beforehand.
-__global__ void __launch_bounds__(128, 10) block_list_kernel(const CollideArgs a) {
+__global__ void __launch_bounds__(128, 10) plane_list_kernel(const CollideArgs a) {
     pdl_trigger();
     const int lane = threadIdx.x & 31;
     const long long total = a.n_tiles * 4, stride = (long long)gridDim.x * 4;
@@ -1577,7 +1578,7 @@ __global__ void __launch_bounds__(128, 10) block_list_kernel(const CollideArgs a
 }
 
 template <int W, bool FUSED, bool OUTL>
-__global__ void __launch_bounds__(W * 32, kBlockMinCtas) block_rec_kernel(const CollideArgs a) {
+__global__ void __launch_bounds__(W * 32, kBlockMinCtas) plane_rec_kernel(const CollideArgs a) {
     pdl_start();                                    // the records are the listing kernel's output
     __shared__ float4 s_pa[W][32], s_pb[W][32];
     __shared__ float2 s_ra[W][32], s_rb[W][32];
@@ -1593,7 +1594,7 @@ __global__ void __launch_bounds__(W * 32, kBlockMinCtas) block_rec_kernel(const 
     J.bA0 = a.bounds + r.bounds_a; J.bB0 = a.bounds + r.bounds_b;
     J.ha = r.h_a; J.hb = r.h_b; J.N = r.n_steps; J.rows = r.rows; J.cols = r.cols; J.i0 = r.i0; J.j0 = r.j0;
     J.rcull = r.rcull; J.rc2 = r.rc2; J.la = r.la; J.wa = r.wa; J.ra = r.ra; J.lb = r.lb; J.wb = r.wb; J.rb = r.rb;
-    block_work<W, FUSED, OUTL>(a, J, r.k0, r.mask, s_pa, s_pb, s_ra, s_rb, s_first, s_prow, s_pcol, s_lfix, s_pfix);
+    plane_block_work<W, FUSED, OUTL>(a, J, r.k0, r.mask, s_pa, s_pb, s_ra, s_rb, s_first, s_prow, s_pcol, s_lfix, s_pfix);
 }
 
 // table[0, n) = -1 (no collision), 16-byte stores on the aligned body
@@ -1695,18 +1696,18 @@ cudaError_t launch_collide_t(const CollideArgs &a, cudaStream_t st, bool pdl) {
         if (!a.recs || !a.active_count || a.n_tiles * 4 > 0x7fffffffLL) return cudaErrorInvalidValue;
         long long blocks = (a.n_tiles * 4 + 3) / 4;
         if (blocks > 152 * 16) blocks = 152 * 16;
-        cudaError_t e = launch_kernel(block_list_kernel, dim3((unsigned)blocks), dim3(128), 0, st, pdl, a);
+        cudaError_t e = launch_kernel(plane_list_kernel, dim3((unsigned)blocks), dim3(128), 0, st, pdl, a);
         if (e != cudaSuccess) return e;
-        const dim3 grid((unsigned)(a.n_tiles * 4)), block(32 * kBlockWarps);
-        return a.probf ? launch_kernel(block_rec_kernel<kBlockWarps, true, OUTL>, grid, block, 0, st, true, a)
-                       : launch_kernel(block_rec_kernel<kBlockWarps, false, OUTL>, grid, block, 0, st, true, a);
+        const dim3 grid((unsigned)(a.n_tiles * 4)), block(32 * kPlaneWarps);
+        return a.probf ? launch_kernel(plane_rec_kernel<kPlaneWarps, true, OUTL>, grid, block, 0, st, true, a)
+                       : launch_kernel(plane_rec_kernel<kPlaneWarps, false, OUTL>, grid, block, 0, st, true, a);
     }
     if (a.variant == 7 && a.tile_poses) return launch_tiles(a, st, pdl);
     if (a.variant == 7) {   // one CTA per 32 x 32 block; the table's -1s are written beforehand
         if (a.n_tiles * 4 > 0x7fffffffLL) return cudaErrorInvalidValue;
-        const dim3 grid((unsigned)(a.n_tiles * 4)), block(32 * kBlockWarps);
-        return a.probf ? launch_kernel(block_kernel<kBlockWarps, true, OUTL>, grid, block, 0, st, pdl, a)
-                       : launch_kernel(block_kernel<kBlockWarps, false, OUTL>, grid, block, 0, st, pdl, a);
+        const dim3 grid((unsigned)(a.n_tiles * 4)), block(32 * kPlaneWarps);
+        return a.probf ? launch_kernel(plane_block_kernel<kPlaneWarps, true, OUTL>, grid, block, 0, st, pdl, a)
+                       : launch_kernel(plane_block_kernel<kPlaneWarps, false, OUTL>, grid, block, 0, st, pdl, a);
     }
     if constexpr (!OUTL) {
         if (a.variant == 4 && !a.tile_poses && a.n_tiles >= kWholeTiles)
