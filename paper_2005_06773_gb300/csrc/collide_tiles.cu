@@ -250,18 +250,21 @@ __device__ __forceinline__ BlockRef listed_block(const CollideArgs &a, long long
 // Without the list (UNLISTED: culling off, or no room for the tile-ordered poses; kWholeTiles in collide.cu) they take
 // every block of ascending tiles, strided, and read the pose planes.
 //
-// Bound by instruction issue: about 400 warp instructions per (block, step) item, half of them the sweep.  Measured
-// (collision stage, listing included): 32 cars of 2048 hypotheses 1.79 ms, 256 uneven scenarios 6.3 ms; a warp per 64 x
-// 64 tile of consecutive hypotheses took 4.77 and 11.8 ms (five and two times the executed tests), compact tiles
-// without the list 2.67 and 8.9 ms (a third of the launch was its last warps), with it but with warps that stay until
-// the list is empty 1.73 ms (requests of higher priority then wait for the whole launch).
+// Bound by instruction issue while the list lasts (12 cars of 2,048 hypotheses, ncu: 74 % of the issue slots, 560 warp
+// instructions per (block, step) item with its hits, set-up and listing order) and by the last blocks (SMs active 79 %
+// of the launch); a shorter sweep alone did not shorten it.  Measured (collision stage, listing included): 32 cars 1.90
+// ms, 256 uneven scenarios 6.00 ms; a warp per 64 x 64 tile of consecutive hypotheses took 4.77 and 11.8 ms (five and
+// two times the executed tests), compact tiles without the list 2.67 and 8.9 ms (a third of the launch was its last
+// warps), with it but with warps that stay until the list is empty 1.73 ms for the 32 cars (requests of higher priority
+// then wait for the whole launch).
 constexpr int kWalkWarps = 4;
 constexpr int kWalkCtas = 7;            // per SM: bounds the registers to 72 (256 scenarios, collision stage: 6.00 ms; 5, 6, 8: 6.80, 6.33, 6.17)
 constexpr int kWalkBlocks = 16;         // blocks per warp that the grid is sized for (its last CTAs take what is left)
 // Steps after which a CTA makes room for a stream of higher priority (unless it is one of the last).  By steps and for the
 // CTA as a whole: its warps end together.  A small request behind 32 cars in the serving loop is done 0.4 ms after its
-// submission so, 0.9 to 1.2 ms with 16 blocks a warp or 1,024 steps; 32 cars take 2.66 ms, with 96 steps 2.68, with 1,024
-// 2.59; 256 scenarios (collision stage) 6.32, 6.40 and 6.18 ms, 6.33 with 16 blocks a warp.
+// submission so, 0.9 to 1.2 ms with 16 blocks a warp or 1,024 steps; the whole call on 32 cars takes 2.66 ms, with 96
+// steps 2.68, with 1,024 2.59; 256 scenarios (collision stage, at six CTAs per SM) 6.32, 6.40 and 6.18 ms, 6.33 with 16
+// blocks a warp.
 constexpr int kWalkSteps = 192;
 
 struct WalkSlot {

@@ -254,7 +254,7 @@ __device__ __forceinline__ bool path_step(const PathConst &p, const PathSection 
 // of some 170 instructions.  Outside the low-speed regime the warp runs the short body (no branch but the votes), inside
 // it the general one (three times as long: tanf, atanf, cosf and the short series' other case); a hypothesis that has
 // stopped is not in the regime, and a warp whose hypotheses have all stopped only stores their poses.  3,087 path
-// hypotheses (11-object scene): generation 57 us, 90 with the low regime run to the horizon's end, section values indexed
+// hypotheses (11-object scene): generation 57 us (60 under ncu), 90 with the low regime run to the horizon's end, section values indexed
 // in local memory and two divisions per low sub-step (a hypothesis braking at 9 m/s^2 spent three quarters of its time
 // after its stop).
 __device__ void vehicle_path(const ObjDesc &o, float acc, const float *path, const Regime &g, int N, int K,
