@@ -421,8 +421,9 @@ void mhc_plan_destroy(mhc_plan *plan);
  *
  * The pool is a device buffer the caller owns (e.g. a torch tensor), at least 1 MiB; admission is by its
  * free bytes (first fit).  A batch takes the scratch that the fastest collision kernels want (mhc_layout, mhc_batch_layout)
- * only while every queued request and one more such batch would still fit; in a pool too tight for that it runs with the
- * least, in up to twice the time.  One serving loop per context; while it runs, use the context for nothing else
+ * only while whatever could run beside it would still fit (the queued requests that the other idle slots can take, and one
+ * more such batch where its lane has one); in a pool too tight for that it runs with the least, in up to twice the time.
+ * One serving loop per context; while it runs, use the context for nothing else
  * but the calls below and mhc_set_option / mhc_autotune before mhc_serve_start (the loop keeps a copy of
  * the collision configuration).  mhc_submit / mhc_poll / mhc_release / mhc_request_* / mhc_serve_stats_read
  * are thread-safe.

@@ -224,18 +224,30 @@ Batch *build_batch(Server *S, std::vector<Request *> &take) {
     return b;
 }
 
+// Pool bytes that may be wanted while batch b of the given lane runs (holds mu): by the queued requests that the lanes' other
+// idle slots can take, and by one more batch like b where b's own lane has such a slot.
+size_t beside(const Server *S, const Batch *b, bool small) {
+    size_t bytes = 0;
+    for (const bool lane : {true, false}) {
+        long long idle = lane == small ? -1 : 0;   // (b's own slot is still idle)
+        for (const Slot &sl : S->slots) idle += sl.small == lane && !sl.busy;
+        long long left = idle * S->cfg.max_batch;
+        for (const Request *r : lane ? S->q_small : S->q_large) {
+            if (left-- <= 0) break;
+            bytes += r->bytes;
+        }
+        if (lane == small && idle > 0) bytes += b->res_bytes + b->scr_least;
+    }
+    return bytes;
+}
+
 // The batch's pool blocks and its requests' states (holds mu).  False: the pool has no room (the caller
 // puts the requests back).
-bool admit_batch(Server *S, Batch *b, std::vector<Request *> &take) {
+bool admit_batch(Server *S, Batch *b, std::vector<Request *> &take, bool small) {
     if (!pool_alloc(S->pool, b->res_bytes, &b->res_off)) { b->res_bytes = 0; return false; }
-    // room for the poses in tile order only where it keeps nobody out: every queued request and one more batch like this
-    // still fit.  Else the collision kernels read the planes (32 vehicles: 5.7 ms instead of 2.8)
-    if (b->scr_least < b->scr_bytes) {
-        size_t others = b->res_bytes + b->scr_least;
-        for (const Request *r : S->q_small) others += r->bytes;
-        for (const Request *r : S->q_large) others += r->bytes;
-        if (pool_largest(S->pool) < b->scr_bytes + others) b->scr_bytes = b->scr_least;
-    }
+    // room for the poses in tile order only where it keeps nobody out that could run beside this batch.  Else the
+    // collision kernels read the planes (32 vehicles: 5.7 ms instead of 2.8)
+    if (b->scr_least < b->scr_bytes && pool_largest(S->pool) < b->scr_bytes + beside(S, b, small)) b->scr_bytes = b->scr_least;
     b->scr_held = pool_alloc(S->pool, b->scr_bytes, &b->scr_off);
     if (!b->scr_held) {
         pool_free(S->pool, b->res_off);
@@ -328,7 +340,7 @@ void scheduler(Server *S, bool small_lane) {
                 lk.unlock();
                 Batch *b = build_batch(S, take);
                 lk.lock();
-                if (S->stopping || !b || !admit_batch(S, b, take)) {   // no room (or stopping): back to the queue
+                if (S->stopping || !b || !admit_batch(S, b, take, small_lane)) {   // no room (or stopping): back to the queue
                     delete b;
                     untake(S, take, small_lane);
                     break;

@@ -62,3 +62,32 @@ def test_two_large_requests_at_their_least(mhc):
                 torch.testing.assert_close(a[k], b[k], rtol=1e-12, atol=1e-18)
             else:
                 assert torch.equal(a[k], b[k]), k
+
+
+def test_a_long_queue_does_not_slow_its_requests(mhc):
+    """One large slot: nothing in the queue could run beside the batch, so it gets its larger scratch."""
+    sc = mhc.as_c(S.stress32(4))
+    lay = mhc.layout(sc)
+    ctx = mhc.Context(0, 8 << 20)
+    srv = mhc.Server(ctx, 3 * lay["run_bytes"], large_slots=1, max_batch=1)
+
+    def spans(n):
+        srv.pause(True)
+        tickets = [srv.submit(sc) for _ in range(n)]
+        srv.pause(False)
+        out = []
+        for t in tickets:
+            assert srv.poll(t, None, timeout_us=60_000_000)
+            ns, _ = srv.times(t)
+            out.append(ns[2] - ns[1])
+            srv.release(t)
+        return sorted(out)[n // 2]
+
+    try:
+        spans(1)                                                   # kernels loaded, pinned buffers allocated
+        alone = spans(1)
+        assert spans(6) < 1.5 * alone
+    finally:
+        srv.stop()
+        ctx.close()
+        torch.cuda.empty_cache()
