@@ -264,8 +264,11 @@ int mhc_transfer_bytes(mhc_ctx *ctx, int64_t *h2d, int64_t *d2h);
  *   n_pairs    object pairs tested
  *   n_entries  trajectory combinations sum_p h_a h_b (Eq. threads:coll); the table holds that many int16
  *   h_ego      hypotheses of the EGO object
- *   scratch    arena bytes a call on this scenario needs (mhc_run needs poses + table on top, reported
- *              by mhc_run_bytes)
+ *   scratch    arena bytes for a call on this scenario (mhc_run needs poses + table on top, reported
+ *              by mhc_run_bytes).  On scenes of more than 131,072 collision tiles, or of long horizons, part of
+ *              them only holds the poses in tile order and the list of active blocks of collision layouts 4 and 7:
+ *              an arena (or a plan's scratch) without room for these is accepted, and the call then runs the
+ *              kernels of ascending tiles, with the same results in up to twice the time
  * Errors: MHC_E_INVALID with the reason in mhc_last_error().
  */
 int mhc_layout(const mhc_scenario *scen, int64_t *n_traj, int32_t *n_pairs, int64_t *n_entries,
@@ -352,8 +355,8 @@ typedef struct {
     int64_t n_scen_steps;    /* sum of the scenarios' n_steps: length of attr_step */
     int64_t h_ego;           /* EGO hypotheses of all scenarios */
     int32_t n_pairs, n_objects, n_scenarios, max_steps;
-    size_t scratch;          /* arena bytes mhc_evaluate_batch needs */
-    size_t plan_bytes;       /* device scratch bytes mhc_plan_create needs */
+    size_t scratch;          /* arena bytes for mhc_evaluate_batch (see mhc_layout) */
+    size_t plan_bytes;       /* device scratch bytes for mhc_plan_create (likewise) */
 } mhc_batch_info;
 
 typedef struct {             /* where scenario s sits in the concatenated arrays */
